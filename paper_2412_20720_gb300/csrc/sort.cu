@@ -509,8 +509,10 @@ __global__ void __launch_bounds__(kEmitBlock) pair_scan_kernel(EmitArgs A, Raste
 
 constexpr int kEmitRecCache = 256;  // emission records cached per chunk
 
-// Shared-memory view of one chunk: the pair prefix and (when they fit) the
-// emission records of the depth-sorted positions its pairs belong to.
+// Shared-memory view of one chunk: the pair prefix (up to kEmitChunk
+// positions) and the emission records (up to kEmitRecCache) of the
+// depth-sorted positions its pairs belong to.  Positions without pairs can
+// make them any number; beyond the caches they are read from global memory.
 struct EmitChunkSmem {
   uint32_t j0, ns;
   uint32_t pref[kEmitChunk + 1];
@@ -520,18 +522,25 @@ struct EmitChunkSmem {
 __device__ __forceinline__ void load_emit_chunk(const EmitArgs &A, uint32_t c, uint32_t f1, uint32_t npairs,
                                                 int64_t nvis, EmitChunkSmem &S) {
   if (threadIdx.x == 0) {  // positions holding pair f0 and, at most one past, pair f1 - 1
-    const int64_t j0 = A.chunk_first[c];
-    const int64_t j1 = f1 == npairs ? nvis - 1 : (int64_t)A.chunk_first[c + 1];
+    // (clamped: after a recorded timeout the marks may be stale)
+    const int64_t j0 = min64(A.chunk_first[c], nvis - 1);
+    const int64_t j1 = f1 == npairs ? nvis - 1 : min64(A.chunk_first[c + 1], nvis - 1);
     S.j0 = (uint32_t)j0;
-    S.ns = (uint32_t)min64(max64(j1 - j0 + 1, 1), kEmitChunk);
+    S.ns = (uint32_t)max64(j1 - j0 + 1, 1);
   }
   __syncthreads();
   const uint32_t j0 = S.j0, ns = S.ns;
-  for (uint32_t k = threadIdx.x; k <= ns; k += kEmitBlock)
-    S.pref[k] = (int64_t)(j0 + k) <= nvis ? A.pair_prefix[j0 + k] : npairs;
+  if (ns <= (uint32_t)kEmitChunk)
+    for (uint32_t k = threadIdx.x; k <= ns; k += kEmitBlock)
+      S.pref[k] = (int64_t)(j0 + k) <= nvis ? A.pair_prefix[j0 + k] : npairs;
   if (ns <= (uint32_t)kEmitRecCache)
     for (uint32_t k = threadIdx.x; k < 3 * ns; k += kEmitBlock) S.rec[k] = A.emit_rec[3 * (size_t)j0 + k];
   __syncthreads();
+}
+
+// First pair of position k of the chunk (k <= ns).
+__device__ __forceinline__ uint32_t chunk_pref(const EmitArgs &A, const EmitChunkSmem &S, int k) {
+  return S.ns <= (uint32_t)kEmitChunk ? S.pref[k] : A.pair_prefix[(size_t)S.j0 + k];
 }
 
 // Walk over consecutive pairs of a chunk: the depth-sorted position the
@@ -567,12 +576,12 @@ __device__ __forceinline__ PairWalk walk_begin(const EmitArgs &A, const EmitChun
   int lo = 0, hi = (int)S.ns - 1;
   while (lo < hi) {  // last position whose pair prefix is <= f
     const int mid = (lo + hi + 1) >> 1;
-    if (S.pref[mid] <= f) lo = mid;
+    if (chunk_pref(A, S, mid) <= f) lo = mid;
     else hi = mid - 1;
   }
   PairWalk w;
   walk_load(A, S, lo, w);
-  const uint32_t local = f - S.pref[lo];
+  const uint32_t local = f - chunk_pref(A, S, lo);
   const uint32_t wd = (uint32_t)max(w.x1 - w.x0, 1);
   const uint32_t qy = local / wd;
   w.tx = w.x0 + (int)(local - qy * wd);
@@ -586,9 +595,9 @@ __device__ __forceinline__ void walk_next(const EmitArgs &A, const EmitChunkSmem
     w.tx = w.x0;
     ++w.ty;
   }
-  if (S.pref[w.lo + 1] <= f) {
-    int lo = w.lo + 1;
-    while (S.pref[lo + 1] <= f) ++lo;  // positions without pairs (capacity clamp)
+  if (chunk_pref(A, S, w.lo + 1) <= f) {
+    int lo = min(w.lo + 1, (int)S.ns - 1);
+    while (lo + 1 < (int)S.ns && chunk_pref(A, S, lo + 1) <= f) ++lo;  // positions without pairs
     walk_load(A, S, lo, w);
     w.tx = w.x0;
     w.ty = w.y0;
