@@ -97,9 +97,11 @@ int compute_layout(const fgs4d_settings *s, int64_t n, const fgs4d_view *views, 
   L.vis_cap = s->vis_capacity ? s->vis_capacity : n * (int64_t)nviews;
   if (L.vis_cap > kMaxCap) return FGS4D_ERR_ARG;  // set vis_capacity explicitly
   L.inst_cap = s->inst_capacity;
+  int64_t cells = 0;
   for (int v = 0; v < nviews; ++v) {
     const int64_t gw = (views[v].width + s->tile - 1) / s->tile, gh = (views[v].height + s->tile - 1) / s->tile;
     L.total_tiles += gw * gh;
+    cells += ((gw + 7) / 8) * ((gh + 7) / 8);
     L.total_pixels += (int64_t)views[v].width * views[v].height;
   }
   if (L.total_tiles > INT32_MAX) return FGS4D_ERR_ARG;
@@ -115,15 +117,21 @@ int compute_layout(const fgs4d_settings *s, int64_t n, const fgs4d_view *views, 
   L.pre_blocks = (int32_t)pb;
   L.emit_blocks = (int32_t)((L.vis_cap + kEmitBlock - 1) / kEmitBlock);
   L.pair_cap = std::min<int64_t>(8 * L.inst_cap, (int64_t)INT32_MAX);
-  L.chunk_cap = (int32_t)((L.pair_cap + kEmitChunk - 1) / kEmitChunk);
+  L.cells = L.vis_cap >= kCellsMinVisible && L.vis_cap >= kCellsMinPerCell * cells;
+  L.total_cells = (int32_t)cells;
+  int cell_bits = 1;
+  while ((1ll << cell_bits) < cells) ++cell_bits;
+  L.cell_passes = (cell_bits + kRadixBits - 1) / kRadixBits;
+  const int64_t chunk = L.cells ? kCellChunk : kEmitChunk;
+  L.chunk_cap = (int32_t)((L.pair_cap + chunk - 1) / chunk);
   // Grids of the latency-bound stages (152 SMs): full-GPU by default, or at
   // most k blocks per SM for preprocess and the radix passes and 2k for the
   // emission when other work shares the GPU (stage_blocks_per_sm = k).
   const int k = s->stage_blocks_per_sm;
   L.pre_grid = k ? std::min(L.pre_blocks, 152 * k) : L.pre_blocks;
   L.sort_grid = 152 * (k ? k : 4);
-  L.tile_sort_sub = s->inst_capacity >= kWideTileSortMinCap ? 3 : 1;
-  L.tile_sort_grid = 152 * (k ? std::min(k, 3) : 3);
+  const int64_t segs = (L.inst_cap + kCellSeg - 1) / kCellSeg;
+  L.cell_grid = (int32_t)std::min<int64_t>(segs, 152 * (k ? 2 * k : 8));
   L.emit_grid = std::max(1, std::min(L.chunk_cap, 152 * (k ? 2 * k : 8)));
   L.depth_blocks = (int32_t)((L.vis_cap + kDepthSortTile - 1) / kDepthSortTile);
   L.tile_blocks = (int32_t)((L.inst_cap + kInstSortTile - 1) / kInstSortTile);
@@ -161,7 +169,15 @@ int compute_layout(const fgs4d_settings *s, int64_t n, const fgs4d_view *views, 
     L.inst_key[k] = take(ic * 4);
     L.inst_val[k] = take(ic * 4);
   }
+  if (L.cells) {
+    L.cell_slot = take(ic * 4);
+    L.cell_mask = take(ic * 8);
+  }
   L.tile_state = take((size_t)L.tile_passes * L.tile_blocks * kRadixBins * sizeof(uint32_t));
+  if (L.cells) {
+    L.cell_ranges = take((size_t)L.total_cells * 8);
+    L.cell_rows = take((size_t)(segs + L.total_cells) * 64 * 4);
+  }
   L.ranges = take((size_t)L.total_tiles * 8);
   L.pix_T = take((size_t)L.total_pixels * 4);
   L.pix_last = take((size_t)L.total_pixels * 4);

@@ -21,9 +21,20 @@ constexpr int kDepthSortItems = 4;  // keys per thread per radix block of the de
 constexpr int kDepthSortTile = kSortThreads * kDepthSortItems;
 constexpr int kInstSortItems = 8;   // keys per thread per radix block of the instance (tile-id) sort
 constexpr int kInstSortTile = kSortThreads * kInstSortItems;
-// Instance capacity from which the instance sort takes three sub-tiles per
-// ticket (a third of the look-backs, fewer resident blocks).
-constexpr int64_t kWideTileSortMinCap = int64_t(1) << 26;
+// Two-level binning (cells.cuh).
+constexpr int kCellChunk = 256;          // candidate (slot, cell) pairs per emission chunk, one per thread
+constexpr int kCellSeg = 256;            // sorted pairs per segment, one per thread
+constexpr int kCellBlock = kCellSeg;     // threads of the count and write kernels: one warp per row of a cell's tiles
+constexpr int kCellPrefixThreads = 512;
+// Two-level binning is taken from these visible capacities on (in all, and per
+// cell): it launches three more kernels than the instance sort and works a
+// cell's list at a time.  bin_sort (us) instance sort / two-level, at 1352x1014
+// (88 cells) unless noted: capacity 48,000 (263k instances) 81.1 / 82.3;
+// 100,000 (553k) 87.1 / 87.3; 300,000 (1.66M) 134 / 113; 361,000 over 482
+// cells (8 views, 1.9M) 168 / 194; 48,000 over 352 cells (8-pixel tiles) 91 /
+// 120; the 6-view street call (5.4M over 810 cells, 685M) 20,900 / 4,100.
+constexpr int64_t kCellsMinVisible = 65536, kCellsMinPerCell = 1024;
+constexpr int64_t kPairScanWideMin = int64_t(1) << 19;
 constexpr int kRadixBits = 8;
 constexpr int kRadixBins = 1 << kRadixBits;
 constexpr int kMaxPasses = 4;
@@ -52,7 +63,10 @@ enum Counter : int {
   kCtrTicketChunk = 9,
   kCtrTicketDepth = 10,  // kMaxPasses entries
   kCtrTicketTile = 14,   // kMaxPasses entries
-  kCtrPairs = 19,        // (slot, rect tile) pairs of all visible slots
+  kCtrCellPairs = 18,    // (cell, slot) pairs with an instance (two-level binning)
+  kCtrPairs = 19,        // (slot, rect tile) pairs of all visible slots, or (slot, cell) pairs
+  kCtrInstances64 = 20,  // 64-bit instance count of the two-level binning
+  kCtrCellDone = 22,     // finished blocks of cell_prefix_kernel
   kCtrCount = 64
 };
 constexpr size_t kSortControlStart = 32;
@@ -77,6 +91,7 @@ struct PreViews {
 
 struct RasterView {
   int32_t tile_base, gw, gh, width, height, tile;  // tile: edge in pixels
+  int32_t cell_base, cgw;  // first cell and cells per row (two-level binning)
   int64_t pix_base;
 };
 
@@ -107,6 +122,8 @@ struct Layout {
   size_t depth_state;   // uint32 [kMaxPasses][depth_blocks][256]
   size_t inst_key[2], inst_val[2];
   size_t tile_state;    // uint32 [kMaxPasses][tile_blocks][256]
+  // Two-level binning: per-pair slot and tile mask, per-cell ranges, per-run counts.
+  size_t cell_slot, cell_mask, cell_ranges, cell_rows;
   size_t ranges;
   size_t pix_T, pix_last;
   size_t slot_grad;
@@ -119,13 +136,14 @@ struct Layout {
   int64_t total_tiles, total_pixels;
   int32_t pre_blocks_per_view, pre_blocks;
   int32_t emit_blocks;    // pair-scan blocks (one visible slot per thread)
-  int64_t pair_cap;       // max (slot, rect tile) pairs: 8 x inst_cap, at most 2^31 - 1
-  int32_t chunk_cap;      // emission chunks of kEmitChunk pairs
+  int64_t pair_cap;       // max (slot, rect tile) or (slot, cell) pairs: 8 x inst_cap, at most 2^31 - 1
+  int32_t chunk_cap;      // emission chunks of kEmitChunk (two-level binning: kCellChunk) pairs
   int32_t emit_grid;      // persistent emission blocks
   int32_t pre_grid;       // persistent preprocess blocks
   int32_t sort_grid;      // persistent radix-pass blocks (at most; one radix tile each at least)
-  int32_t tile_sort_sub;  // sub-tiles of kInstSortTile keys per ticket of the instance sort (1 or 3)
-  int32_t tile_sort_grid; // persistent instance-sort blocks with 3 sub-tiles per ticket
+  bool cells;             // two-level binning (cells.cuh) instead of the instance sort
+  int32_t total_cells, cell_passes;
+  int32_t cell_grid;      // persistent count / write blocks
   int32_t depth_blocks, tile_blocks;
   int32_t depth_passes, tile_passes;
   int32_t tile_bits;
@@ -485,7 +503,7 @@ cudaError_t launch_l1_loss(const float *img, const float *target, int64_t count,
 template <int MAXV>
 inline bool make_raster_views(const Layout &L, const fgs4d_view *views, int32_t nviews, RasterViews<MAXV> *out) {
   if (nviews > MAXV) return false;
-  int64_t tb = 0, pb = 0;
+  int64_t tb = 0, pb = 0, cb = 0;
   for (int v = 0; v < nviews; ++v) {
     RasterView &r = out->v[v];
     r.width = views[v].width;
@@ -495,6 +513,9 @@ inline bool make_raster_views(const Layout &L, const fgs4d_view *views, int32_t 
     r.tile_base = (int32_t)tb;
     r.pix_base = pb;
     r.tile = L.tile;
+    r.cgw = (r.gw + 7) / 8;
+    r.cell_base = (int32_t)cb;
+    cb += (int64_t)r.cgw * ((r.gh + 7) / 8);
     tb += (int64_t)r.gw * r.gh;
     pb += (int64_t)r.width * r.height;
   }

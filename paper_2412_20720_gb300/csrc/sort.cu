@@ -128,78 +128,66 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem, int src
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gmem), "r"(src_bytes) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-// Waits until at most n (0..2) of this thread's copy groups are pending.
-__device__ __forceinline__ void cp_async_wait_pending(int n) {
-  if (n <= 0) asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-  else if (n == 1) asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-  else asm volatile("cp.async.wait_group 2;\n" ::: "memory");
+__device__ __forceinline__ void cp_async_wait_all() {
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
 }
 
 // Shared memory of one radix block: the ticket's keys and values (input,
-// then the block-local order), per-warp digit counts (two sets, alternating
-// between sub-tiles), per-sub-tile digit starts and the digits' global
-// starts.
-template <int kItems, int kSub>
+// then the block-local order), per-warp digit counts, the digits' block-local
+// and global starts.
+template <int kItems>
 struct RadixSmem {
-  uint32_t keys[kSortThreads * kItems * kSub];
-  uint32_t vals[kSortThreads * kItems * kSub];
-  uint32_t wcount[kSub > 1 ? 2 : 1][kSortThreads / 32][kRadixBins];
-  uint32_t bstart[kSub][kRadixBins];  // first block-local position of each digit in sub-tile s
-  uint32_t sbase[kSub][kRadixBins];   // keys of each digit in the sub-tiles before s
-  uint32_t gstart[kRadixBins];        // global position of the ticket's first key of each digit
+  uint32_t keys[kSortThreads * kItems];
+  uint32_t vals[kSortThreads * kItems];
+  uint32_t wcount[kSortThreads / 32][kRadixBins];
+  uint32_t bstart[kRadixBins];  // first block-local position of each digit
+  uint32_t gstart[kRadixBins];  // global position of the ticket's first key of each digit
   uint32_t scan[12];
   uint32_t ticket;
 };
-template <int kItems, int kSub>
+template <int kItems>
 constexpr size_t radix_smem_bytes() {
-  return sizeof(RadixSmem<kItems, kSub>);
+  return sizeof(RadixSmem<kItems>);
 }
 
 // One stable 8-bit LSD pass.  A block takes tickets in launch order; a
-// ticket is kSub consecutive sub-tiles of kSortThreads x kItems keys.  Each
-// warp copies the keys (and values) it ranks into shared memory with
-// cp.async, one copy group per sub-tile, so later sub-tiles arrive while the
-// first is ranked (16-byte copies: keys_in and vals_in start on 16-byte
-// boundaries, as the workspace's arrays do).  Ranking is stable within a
-// warp's segment (item-major, lane-minor): the lanes holding the same digit
-// are found by nine ballots
-// (eight digit bits and the padding bit), and the lowest of them adds the
-// group's size to the warp's count of that digit.  Each sub-tile is then
-// placed in block-local digit order in its own part of the buffer.  One
-// decoupled look-back per ticket gives the ticket's global start of each
-// digit, and the scatter writes each sub-tile's digit runs.  Small sorts
-// (the depth sort) take short sub-tiles, so that more SMs share a pass;
-// very large instance sorts take three sub-tiles per ticket, which divides
-// the look-backs per key by three.
+// ticket is kSortThreads x kItems consecutive keys.  Each warp copies the
+// keys (and values) it ranks into shared memory with cp.async (16-byte
+// copies: keys_in and vals_in start on 16-byte boundaries, as the
+// workspace's arrays do).  Ranking is stable within a warp's segment
+// (item-major, lane-minor): the lanes holding the same digit are found by
+// nine ballots (eight digit bits and the padding bit), and the lowest of them
+// adds the group's size to the warp's count of that digit.  The ticket is
+// then placed in block-local digit order, a decoupled look-back gives its
+// global start of each digit, and the scatter writes each digit's run.  Small
+// sorts (the depth sort) take short tickets, so that more SMs share a pass.
 //
-// With `ranges` (the last pass of the tile sort, keys = global tile ids
-// below total_tiles) the pass also records each tile's [start, end) in the
-// sorted list.  A sub-tile's staged keys are ordered by the full key (the
+// With `ranges` (the last pass of the tile or cell sort, keys = tile or cell
+// ids below total_tiles) the pass also records each id's [start, end) in the
+// sorted list.  A ticket's staged keys are ordered by the full key (the
 // pass input is ordered by the lower digits and the staging is stable), so
-// the equal keys of a sub-tile form one run; its first and last output
+// the equal keys of a ticket form one run; its first and last output
 // positions go to atomicMin on start and atomicMax on end, which the
-// emission initialised to (0xffffffff, 0).  A tile with no instance keeps
+// emission initialised to (0xffffffff, 0).  An id with no key keeps
 // start > end, which every reader takes as empty.
-template <bool kValsAreIndex, int kItems, int kSub>
+template <bool kValsAreIndex, int kItems>
 __global__ void __launch_bounds__(kSortThreads) radix_pass_kernel(
     const uint32_t *__restrict__ keys_in, const uint32_t *__restrict__ vals_in, uint32_t *__restrict__ keys_out,
     uint32_t *__restrict__ vals_out, const uint32_t *__restrict__ count_ptr, int64_t cap, int32_t shift,
     const uint32_t *__restrict__ hist, uint32_t *state, uint32_t *ticket, uint32_t *status, uint2 *ranges,
     int64_t total_tiles) {
-  static_assert(kSub >= 1 && kSub <= 3, "copy groups are waited for by count (at most 2 pending)");
   static_assert(kItems % 4 == 0, "whole 16-byte copies per warp segment");
   grid_dependency_sync();
-  constexpr int kSubKeys = kSortThreads * kItems;
-  constexpr int kTileKeys = kSubKeys * kSub;
+  constexpr int kTileKeys = kSortThreads * kItems;
   constexpr int kWarps = kSortThreads / 32;
-  constexpr int kSegKeys = 32 * kItems;  // keys of one warp in a sub-tile
+  constexpr int kSegKeys = 32 * kItems;  // keys of one warp
   extern __shared__ __align__(16) unsigned char radix_smem[];
-  RadixSmem<kItems, kSub> &S = *reinterpret_cast<RadixSmem<kItems, kSub> *>(radix_smem);
+  RadixSmem<kItems> &S = *reinterpret_cast<RadixSmem<kItems> *>(radix_smem);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t lt_mask = (1u << lane) - 1u;
   const int64_t count = min64((int64_t)*count_ptr, cap);
-  for (int i = threadIdx.x; i < (int)(sizeof S.wcount / sizeof(uint32_t)); i += kSortThreads) (&S.wcount[0][0][0])[i] = 0u;
+  for (int i = threadIdx.x; i < (int)(sizeof S.wcount / sizeof(uint32_t)); i += kSortThreads) (&S.wcount[0][0])[i] = 0u;
   uint32_t total;
   // Keys of the digits below each digit over the whole input: the same for
   // every ticket.
@@ -212,100 +200,86 @@ __global__ void __launch_bounds__(kSortThreads) radix_pass_kernel(
     const int64_t b = S.ticket;
     const int64_t tile0 = b * kTileKeys;
     if (tile0 >= count) return;
-#pragma unroll
-    for (int s = 0; s < kSub; ++s) {
-      const int seg = s * kSubKeys + warp * kSegKeys;
-      for (int c = lane; c < kSegKeys / 4; c += 32) {
-        const int64_t i0 = tile0 + seg + 4 * c;
-        if (i0 < count) {
-          const int bytes = (int)min64(16, (count - i0) * 4);
-          cp_async16(&S.keys[seg + 4 * c], keys_in + i0, bytes);
-          if (!kValsAreIndex) cp_async16(&S.vals[seg + 4 * c], vals_in + i0, bytes);
-        }
+    const int seg = warp * kSegKeys;
+    for (int c = lane; c < kSegKeys / 4; c += 32) {
+      const int64_t i0 = tile0 + seg + 4 * c;
+      if (i0 < count) {
+        const int bytes = (int)min64(16, (count - i0) * 4);
+        cp_async16(&S.keys[seg + 4 * c], keys_in + i0, bytes);
+        if (!kValsAreIndex) cp_async16(&S.vals[seg + 4 * c], vals_in + i0, bytes);
       }
-      cp_async_commit();
     }
+    cp_async_wait_all();
+    __syncwarp();  // the warp's copies are visible to all its lanes
     const int d = threadIdx.x;  // the digit this thread scans and looks back for
-    uint32_t tot = 0u;          // keys of digit d in the sub-tiles so far
+    uint32_t key[kItems], val[kItems], rank[kItems];
+    int dig[kItems];
 #pragma unroll
-    for (int s = 0; s < kSub; ++s) {
-      uint32_t(&wc)[kWarps][kRadixBins] = S.wcount[kSub > 1 ? (s & 1) : 0];
-      cp_async_wait_pending(kSub - 1 - s);
-      __syncwarp();  // the warp's copies of sub-tile s are visible to all its lanes
-      const int seg = s * kSubKeys + warp * kSegKeys;
-      uint32_t key[kItems], val[kItems], rank[kItems];
-      int dig[kItems];
-#pragma unroll
-      for (int k = 0; k < kItems; ++k) {
-        const int li = seg + k * 32 + lane;
-        if (tile0 + li < count) {
-          key[k] = S.keys[li];
-          val[k] = kValsAreIndex ? (uint32_t)(tile0 + li) : S.vals[li];
-          dig[k] = (key[k] >> shift) & (kRadixBins - 1);
-        } else {
-          key[k] = 0u;
-          val[k] = 0u;
-          dig[k] = kRadixBins;  // padding: ranked nowhere
-        }
+    for (int k = 0; k < kItems; ++k) {
+      const int li = seg + k * 32 + lane;
+      if (tile0 + li < count) {
+        key[k] = S.keys[li];
+        val[k] = kValsAreIndex ? (uint32_t)(tile0 + li) : S.vals[li];
+        dig[k] = (key[k] >> shift) & (kRadixBins - 1);
+      } else {
+        key[k] = 0u;
+        val[k] = 0u;
+        dig[k] = kRadixBins;  // padding: ranked nowhere
       }
-#pragma unroll
-      for (int k = 0; k < kItems; ++k) {
-        const int dk = dig[k];
-        uint32_t peers = 0xffffffffu;
-#pragma unroll
-        for (int bit = 0; bit < 9; ++bit) {
-          const uint32_t set = (uint32_t)((dk >> bit) & 1);
-          peers &= ~(__ballot_sync(0xffffffffu, set) ^ (0u - set));
-        }
-        const int leader = __ffs(peers) - 1;
-        uint32_t base = 0u;
-        if (lane == leader && dk < kRadixBins) base = atomicAdd(&wc[warp][dk], (uint32_t)__popc(peers));
-        base = __shfl_sync(0xffffffffu, base, leader);
-        __syncwarp();  // item k's counts land before item k + 1's
-        rank[k] = base + __popc(peers & lt_mask);
-      }
-      __syncthreads();
-      // Per digit: exclusive prefix over warps; sub-tile count and start.
-      uint32_t cnt = 0u;
-#pragma unroll
-      for (int w = 0; w < kWarps; ++w) {
-        const uint32_t c = wc[w][d];
-        wc[w][d] = cnt;
-        cnt += c;
-      }
-      S.sbase[s][d] = tot;
-      tot += cnt;
-      S.bstart[s][d] = block_exclusive_scan(cnt, S.scan, &total);
-      __syncthreads();
-#pragma unroll
-      for (int k = 0; k < kItems; ++k) {
-        if (dig[k] < kRadixBins) {
-          const uint32_t pos = s * kSubKeys + S.bstart[s][dig[k]] + wc[warp][dig[k]] + rank[k];
-          S.keys[pos] = key[k];
-          S.vals[pos] = val[k];
-        }
-      }
-      __syncwarp();
-      for (int i = lane; i < kRadixBins; i += 32) wc[warp][i] = 0u;  // the warp's row, for sub-tile s + 2
     }
-    S.gstart[d] = gpre + radix_lookback(state, b, d, tot, status);
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) {
+      const int dk = dig[k];
+      uint32_t peers = 0xffffffffu;
+#pragma unroll
+      for (int bit = 0; bit < 9; ++bit) {
+        const uint32_t set = (uint32_t)((dk >> bit) & 1);
+        peers &= ~(__ballot_sync(0xffffffffu, set) ^ (0u - set));
+      }
+      const int leader = __ffs(peers) - 1;
+      uint32_t base = 0u;
+      if (lane == leader && dk < kRadixBins) base = atomicAdd(&S.wcount[warp][dk], (uint32_t)__popc(peers));
+      base = __shfl_sync(0xffffffffu, base, leader);
+      __syncwarp();  // item k's counts land before item k + 1's
+      rank[k] = base + __popc(peers & lt_mask);
+    }
     __syncthreads();
-    // Coalesced runs per digit and sub-tile.
+    // Per digit: exclusive prefix over warps; ticket count and start.
+    uint32_t cnt = 0u;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+      const uint32_t c = S.wcount[w][d];
+      S.wcount[w][d] = cnt;
+      cnt += c;
+    }
+    S.bstart[d] = block_exclusive_scan(cnt, S.scan, &total);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) {
+      if (dig[k] < kRadixBins) {
+        const uint32_t pos = S.bstart[dig[k]] + S.wcount[warp][dig[k]] + rank[k];
+        S.keys[pos] = key[k];
+        S.vals[pos] = val[k];
+      }
+    }
+    __syncwarp();
+    for (int i = lane; i < kRadixBins; i += 32) S.wcount[warp][i] = 0u;  // the warp's row, for the next ticket
+    S.gstart[d] = gpre + radix_lookback(state, b, d, cnt, status);
+    __syncthreads();
+    // Coalesced runs per digit.
     const int32_t nvalid = (int32_t)min64(kTileKeys, count - tile0);
     for (int p = threadIdx.x; p < nvalid; p += kSortThreads) {
-      const int s = p / kSubKeys, q = p - s * kSubKeys;
       const uint32_t kk = S.keys[p];
       const int dd = (kk >> shift) & (kRadixBins - 1);
-      const uint32_t gpos = S.gstart[dd] + S.sbase[s][dd] + ((uint32_t)q - S.bstart[s][dd]);
+      const uint32_t gpos = S.gstart[dd] + ((uint32_t)p - S.bstart[dd]);
       if ((int64_t)gpos < count) {
         keys_out[gpos] = kk;
         vals_out[gpos] = S.vals[p];
         if (ranges) {
           if ((int64_t)kk < total_tiles) {
-            const int qend = min(kSubKeys, nvalid - s * kSubKeys);
             uint32_t *r = reinterpret_cast<uint32_t *>(&ranges[kk]);
-            if (q == 0 || S.keys[p - 1] != kk) atomicMin(&r[0], gpos);
-            if (q == qend - 1 || S.keys[p + 1] != kk) atomicMax(&r[1], gpos + 1u);
+            if (p == 0 || S.keys[p - 1] != kk) atomicMin(&r[0], gpos);
+            if (p == nvalid - 1 || S.keys[p + 1] != kk) atomicMax(&r[1], gpos + 1u);
           } else {
             atomicOr(status, kStatusInternal);
           }
@@ -393,7 +367,7 @@ struct EmitArgs {
 // test of the emission rejects as well).  With tile
 // edge T, tile tx's centre box [T tx + 0.5, T tx + T - 0.5] can meet
 // [u - rx, u + rx] only for ceil((u - rx - T + 0.5) / T) <= tx <= floor((u + rx - 0.5) / T).
-template <int MAXV>
+template <int MAXV, bool kCells>
 __device__ __forceinline__ uint32_t pair_record(const EmitArgs &A, const RasterViews<MAXV> &rv, uint32_t s, int64_t j,
                                                 int64_t nvis) {
   uint32_t area = 0u;
@@ -421,7 +395,9 @@ __device__ __forceinline__ uint32_t pair_record(const EmitArgs &A, const RasterV
       if (ly > (float)y0) y0 = (int)fminf(ly, (float)y1);
       if (hy + 1.0f < (float)y1) y1 = (int)fmaxf(hy + 1.0f, (float)y0);
     }
-    area = (uint32_t)(max(x1 - x0, 0) * max(y1 - y0, 0));
+    if (!kCells) area = (uint32_t)(max(x1 - x0, 0) * max(y1 - y0, 0));
+    else if (x1 > x0 && y1 > y0)
+      area = (uint32_t)((((x1 - 1) >> 3) - (x0 >> 3) + 1) * (((y1 - 1) >> 3) - (y0 >> 3) + 1));
     mm.z = x0 | (y0 << 16);
     mm.w = x1 | (y1 << 16);
   } else {
@@ -438,8 +414,9 @@ __device__ __forceinline__ uint32_t pair_record(const EmitArgs &A, const RasterV
 
 // Pairs [p0, p1) of depth-sorted position j: every emission chunk whose first
 // pair falls among them records j and has its look-back word cleared.
+template <int kChunk>
 __device__ __forceinline__ void mark_chunks(const EmitArgs &A, int64_t j, uint64_t p0, uint64_t p1) {
-  for (uint64_t c = (p0 + kEmitChunk - 1) / kEmitChunk; c * kEmitChunk < p1 && c < (uint64_t)A.chunk_cap; ++c) {
+  for (uint64_t c = (p0 + kChunk - 1) / kChunk; c * kChunk < p1 && c < (uint64_t)A.chunk_cap; ++c) {
     A.chunk_first[c] = (uint32_t)j;
     A.lb_chunk[c] = 0ull;
   }
@@ -447,13 +424,13 @@ __device__ __forceinline__ void mark_chunks(const EmitArgs &A, int64_t j, uint64
 
 // Sets the pair total (clamped to the pair capacity) and, when pairs are lost
 // to the clamp, the instance bound and the overflow flag.
-__device__ __forceinline__ void set_pair_total(const EmitArgs &A, int64_t nvis, uint64_t all) {
+__device__ __forceinline__ void set_pair_total(const EmitArgs &A, int64_t nvis, uint64_t all, uint32_t per_pair) {
   A.pair_prefix[nvis] = (uint32_t)umin64(all, (uint64_t)A.pair_cap);
   A.counters[kCtrPairs] = (uint32_t)umin64(all, (uint64_t)A.pair_cap);
   if (all > (uint64_t)A.pair_cap) {
-    // Some pairs cannot be examined: report the pair total as the bound on
-    // the instances needed.
-    A.counters[kCtrNeedInstances] = (uint32_t)umin64(all, 0xffffffffull);
+    // Some pairs cannot be examined: report the bound on the instances needed
+    // (per_pair: the most instances of one pair).
+    A.counters[kCtrNeedInstances] = (uint32_t)umin64(all * per_pair, 0xffffffffull);
     atomicOr(&A.counters[kCtrStatus], kStatusInstOverflow);
   }
 }
@@ -465,10 +442,11 @@ __device__ __forceinline__ void set_empty_totals(const EmitArgs &A) {
   A.counters[kCtrNeedInstances] = 0u;
 }
 
-// Pair scan, one thread per depth-sorted visible slot: the exclusive prefix
-// of the slots' rect areas in depth order (decoupled look-back), plus the
-// emission record of every position and the chunk marks.
-template <int MAXV>
+// Pair scan, kItems depth-sorted visible slots per thread (consecutive
+// threads on consecutive slots): the exclusive prefix of the slots' rect areas
+// in depth order (decoupled look-back), plus the emission record of every
+// position and the chunk marks.
+template <int MAXV, bool kCells, int kItems>
 __global__ void __launch_bounds__(kEmitBlock) pair_scan_kernel(EmitArgs A, RasterViews<MAXV> rv) {
   grid_dependency_sync();
   __shared__ uint32_t s_ticket;
@@ -478,23 +456,41 @@ __global__ void __launch_bounds__(kEmitBlock) pair_scan_kernel(EmitArgs A, Raste
   __syncthreads();
   const int64_t b = s_ticket;
   if (b == 0 && nvis == 0 && threadIdx.x == 0) set_empty_totals(A);
-  if (b * kEmitBlock >= nvis) return;
-  const int64_t j = b * kEmitBlock + threadIdx.x;
-  const uint32_t area = j < nvis ? pair_record<MAXV>(A, rv, A.sorted_slots[j], j, nvis) : 0u;
-  uint32_t total;
-  const uint32_t excl = block_exclusive_scan(area, s_scan, &total);
+  const int64_t j0 = b * (kEmitBlock * kItems);
+  if (j0 >= nvis) return;
+  uint32_t slot[kItems], area[kItems], excl[kItems], sum = 0u;
+#pragma unroll
+  for (int k = 0; k < kItems; ++k) {
+    const int64_t j = j0 + k * kEmitBlock + threadIdx.x;
+    slot[k] = j < nvis ? A.sorted_slots[j] : 0u;
+  }
+#pragma unroll
+  for (int k = 0; k < kItems; ++k) {
+    const int64_t j = j0 + k * kEmitBlock + threadIdx.x;
+    area[k] = j < nvis ? pair_record<MAXV, kCells>(A, rv, slot[k], j, nvis) : 0u;
+  }
+#pragma unroll
+  for (int k = 0; k < kItems; ++k) {
+    uint32_t total;
+    excl[k] = sum + block_exclusive_scan(area[k], s_scan, &total);
+    sum += total;
+  }
   __shared__ uint64_t s_base;
   if (threadIdx.x < 32) {
-    const uint64_t prefix = lookback_u64_warp(A.lb_scan, (int32_t)b, total, &A.counters[kCtrStatus]);
+    const uint64_t prefix = lookback_u64_warp(A.lb_scan, (int32_t)b, sum, &A.counters[kCtrStatus]);
     if (threadIdx.x == 0) s_base = prefix;
-    if (threadIdx.x == 0 && (b + 1) * kEmitBlock >= nvis) set_pair_total(A, nvis, prefix + total);
+    if (threadIdx.x == 0 && j0 + kEmitBlock * kItems >= nvis) set_pair_total(A, nvis, prefix + sum, kCells ? 64u : 1u);
   }
   __syncthreads();
-  if (j < nvis) {
-    const uint64_t p0 = umin64(s_base + excl, (uint64_t)A.pair_cap);
-    const uint64_t p1 = umin64(s_base + excl + area, (uint64_t)A.pair_cap);
-    A.pair_prefix[j] = (uint32_t)p0;
-    mark_chunks(A, j, p0, p1);
+#pragma unroll
+  for (int k = 0; k < kItems; ++k) {
+    const int64_t j = j0 + k * kEmitBlock + threadIdx.x;
+    if (j < nvis) {
+      const uint64_t p0 = umin64(s_base + excl[k], (uint64_t)A.pair_cap);
+      const uint64_t p1 = umin64(s_base + excl[k] + area[k], (uint64_t)A.pair_cap);
+      A.pair_prefix[j] = (uint32_t)p0;
+      mark_chunks<kCells ? kCellChunk : kEmitChunk>(A, j, p0, p1);
+    }
   }
 }
 
@@ -742,6 +738,63 @@ __global__ void __launch_bounds__(kEmitBlock) emit_kernel(EmitArgs A, RasterView
   }
 }
 
+#include "cells.cuh"
+
+// Two-level binning of the depth-sorted slots.  The sorted pairs end in the
+// instance buffers the final list does not use; the passes before ping-pong
+// with the final list's buffers, which cell_write fills last.
+template <int MAXV>
+cudaError_t bin_cells(const Layout &L, const EmitArgs &ea_in, const RasterViews<MAXV> &rv, unsigned char *ws,
+                      cudaStream_t st) {
+  EmitArgs ea = ea_in;
+  const int fin = L.tile_passes & 1, tmp = fin ^ 1, P = L.cell_passes;
+  uint32_t *ik[2] = {reinterpret_cast<uint32_t *>(ws + L.inst_key[0]), reinterpret_cast<uint32_t *>(ws + L.inst_key[1])};
+  uint32_t *iv[2] = {reinterpret_cast<uint32_t *>(ws + L.inst_val[0]), reinterpret_cast<uint32_t *>(ws + L.inst_val[1])};
+  ea.inst_key = ik[fin];
+  ea.inst_val = iv[fin];
+  CellArgs C;
+  C.e = ea;
+  C.total_cells = L.total_cells;
+  C.cell_passes = P;
+  const int first = (P & 1) ? fin : tmp;  // buffer of the unsorted cell ids, so that pass P - 1 writes into tmp
+  C.key = ik[first];
+  C.slot = reinterpret_cast<uint32_t *>(ws + L.cell_slot);
+  C.mask = reinterpret_cast<uint2 *>(ws + L.cell_mask);
+  C.skey = ik[tmp];
+  C.sidx = iv[tmp];
+  C.cell_ranges = reinterpret_cast<uint2 *>(ws + L.cell_ranges);
+  C.rows = reinterpret_cast<uint32_t *>(ws + L.cell_rows);
+  uint32_t *ctr = ea.counters;
+  // Four slots a thread from kPairScanWideMin visible slots on: a quarter of
+  // the look-backs, and four independent gathers in flight per thread; below
+  // that the blocks would not fill the SMs.
+  const bool many = L.vis_cap >= kPairScanWideMin;
+  cudaError_t e = many ? launch_pdl(pair_scan_kernel<MAXV, true, 4>, (unsigned)((L.emit_blocks + 3) / 4), kEmitBlock,
+                                    st, ea, rv)
+                       : launch_pdl(pair_scan_kernel<MAXV, true, 1>, (unsigned)L.emit_blocks, kEmitBlock, st, ea, rv);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(cell_emit_kernel<MAXV>, (unsigned)L.emit_grid, kCellChunk, st, C, rv);
+  if (e != cudaSuccess) return e;
+  const int pb = std::min(L.tile_blocks, L.sort_grid);
+  constexpr size_t smem = radix_smem_bytes<kInstSortItems>();
+  for (int p = 0; p < P; ++p) {
+    const int in = (p & 1) ? first ^ 1 : first, out = in ^ 1;
+    e = launch_pdl_smem(p == 0 ? radix_pass_kernel<true, kInstSortItems> : radix_pass_kernel<false, kInstSortItems>,
+                        (unsigned)pb, kSortThreads, smem, st, (const uint32_t *)ik[in],
+                        p == 0 ? (const uint32_t *)nullptr : (const uint32_t *)iv[in], ik[out], iv[out],
+                        (const uint32_t *)(ctr + kCtrCellPairs), (int64_t)L.inst_cap, (int32_t)(kRadixBits * p),
+                        (const uint32_t *)(ea.hist_tile + p * kRadixBins),
+                        ea.tile_state + (size_t)p * L.tile_blocks * kRadixBins, ctr + kCtrTicketTile + p,
+                        ctr + kCtrStatus, p == P - 1 ? C.cell_ranges : (uint2 *)nullptr, (int64_t)L.total_cells);
+    if (e != cudaSuccess) return e;
+  }
+  e = launch_pdl(cell_count_kernel, (unsigned)L.cell_grid, kCellBlock, st, C);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(cell_prefix_kernel<MAXV>, (unsigned)std::min(L.total_cells, 152 * 8), kCellPrefixThreads, st, C, rv);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(cell_write_kernel<MAXV>, (unsigned)L.cell_grid, kCellBlock, st, C, rv);
+}
+
 template <int MAXV>
 cudaError_t bin_sort_typed(const Layout &L, const fgs4d_view *views, int32_t nviews, unsigned char *ws,
                            cudaStream_t st) {
@@ -795,7 +848,7 @@ cudaError_t bin_sort_typed(const Layout &L, const fgs4d_view *views, int32_t nvi
     if (L.depth_blocks > 0) {
       const int hb = std::min(L.depth_blocks, L.sort_grid);
       const int pb = std::min(L.depth_blocks, L.sort_grid);
-      constexpr size_t smem = radix_smem_bytes<kDepthSortItems, 1>();
+      constexpr size_t smem = radix_smem_bytes<kDepthSortItems>();
       e = launch_pdl(radix_hist_kernel<kDepthSortItems>, (unsigned)hb, kSortThreads, st, dkey,
                      (const uint32_t *)(ctr + kCtrVisible), (int64_t)L.vis_cap, (int32_t)L.depth_passes, hist_d,
                      dstate, (int32_t)L.depth_blocks, (uint2 *)nullptr, (int64_t)0);
@@ -805,8 +858,8 @@ cudaError_t bin_sort_typed(const Layout &L, const fgs4d_view *views, int32_t nvi
         uint32_t *state = dstate + (size_t)p * L.depth_blocks * kRadixBins;
         const uint32_t *kin = p == 0 ? dkey : dk[in];
         const uint32_t *vin = p == 0 ? nullptr : dv[in];
-        e = launch_pdl_smem(p == 0 ? radix_pass_kernel<true, kDepthSortItems, 1>
-                                   : radix_pass_kernel<false, kDepthSortItems, 1>,
+        e = launch_pdl_smem(p == 0 ? radix_pass_kernel<true, kDepthSortItems>
+                                   : radix_pass_kernel<false, kDepthSortItems>,
                             (unsigned)pb, kSortThreads, smem, st, kin, vin, dk[out], dv[out],
                        (const uint32_t *)(ctr + kCtrVisible), (int64_t)L.vis_cap, (int32_t)(kRadixBits * p),
                        (const uint32_t *)(hist_d + p * kRadixBins), state, ctr + kCtrTicketDepth + p, status,
@@ -815,29 +868,21 @@ cudaError_t bin_sort_typed(const Layout &L, const fgs4d_view *views, int32_t nvi
       }
     }
     // 2. Instances in depth order.
-    e = launch_pdl(pair_scan_kernel<MAXV>, (unsigned)L.emit_blocks, kEmitBlock, st, ea, rv);
+    if (L.cells) return bin_cells<MAXV>(L, ea, rv, ws, st);
+    e = launch_pdl(pair_scan_kernel<MAXV, false, 1>, (unsigned)L.emit_blocks, kEmitBlock, st, ea, rv);
     if (e != cudaSuccess) return e;
     e = launch_pdl(emit_kernel<MAXV>, (unsigned)L.emit_grid, kEmitBlock, st, ea, rv);
     if (e != cudaSuccess) return e;
   }
   // 3. Stable sort of the instances by global tile id (digit histograms
   // taken by the emission); the last pass also records the tile ranges.
-  // Very large instance lists take three sub-tiles per ticket (at most 3
-  // blocks of 73 KB per SM), the others one.
-  const bool wide = L.tile_sort_sub == 3;
-  const int tickets = (L.tile_blocks + L.tile_sort_sub - 1) / L.tile_sort_sub;
-  const int pbt = std::min(tickets, wide ? L.tile_sort_grid : L.sort_grid);
-  constexpr size_t smem1 = radix_smem_bytes<kInstSortItems, 1>(), smem3 = radix_smem_bytes<kInstSortItems, 3>();
-  if (wide) {
-    e = allow_dynamic_smem(radix_pass_kernel<false, kInstSortItems, 3>, smem3);
-    if (e != cudaSuccess) return e;
-  }
+  const int pbt = std::min(L.tile_blocks, L.sort_grid);
+  constexpr size_t smem1 = radix_smem_bytes<kInstSortItems>();
   for (int p = 0; p < L.tile_passes; ++p) {
     const int in = p & 1, out = in ^ 1;
     const bool last = p == L.tile_passes - 1;
     uint32_t *state = tstate + (size_t)p * L.tile_blocks * kRadixBins;
-    e = launch_pdl_smem(wide ? radix_pass_kernel<false, kInstSortItems, 3> : radix_pass_kernel<false, kInstSortItems, 1>,
-                        (unsigned)pbt, kSortThreads, wide ? smem3 : smem1, st, (const uint32_t *)ik[in],
+    e = launch_pdl_smem(radix_pass_kernel<false, kInstSortItems>, (unsigned)pbt, kSortThreads, smem1, st, (const uint32_t *)ik[in],
                         (const uint32_t *)iv[in], ik[out], iv[out], (const uint32_t *)(ctr + kCtrInstances),
                         (int64_t)L.inst_cap, (int32_t)(kRadixBits * p), (const uint32_t *)(hist_t + p * kRadixBins),
                         state, ctr + kCtrTicketTile + p, status, last ? ranges : (uint2 *)nullptr,
@@ -851,7 +896,8 @@ cudaError_t bin_sort_typed(const Layout &L, const fgs4d_view *views, int32_t nvi
 
 int bin_sort_kernel_count(const Layout &L, int32_t nviews) {
   (void)nviews;
-  const int tail = L.tile_passes;  // tile-sort passes (the last records the ranges)
+  // tile-sort passes (the last records the ranges), or cell-sort passes and the count, prefix and write kernels
+  const int tail = L.cells ? L.cell_passes + 3 : L.tile_passes;
   if (L.emit_blocks == 0) return tail;
   // depth histogram and passes, pair scan, emission
   return (L.depth_blocks > 0 ? 1 + L.depth_passes : 0) + 2 + tail;
@@ -972,7 +1018,7 @@ extern "C" int fgs4d_sort_depth_static(const uint32_t *depth_keys, int64_t n, ui
   if (rc) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int blocks = (int)((n + kSortTile - 1) / kSortTile);
-  constexpr size_t smem = radix_smem_bytes<kSortItems, 1>();
+  constexpr size_t smem = radix_smem_bytes<kSortItems>();
   static_sort_init_kernel<<<1, 256, 0, st>>>(s, (uint32_t)n);
   radix_hist_kernel<kSortItems><<<blocks, kSortThreads, 0, st>>>(depth_keys, &s->ctl[0], FGS4D_STATIC_SORT_MAX,
                                                           kMaxPasses, &s->hist[0][0], &s->state[0][0][0],
@@ -991,11 +1037,11 @@ extern "C" int fgs4d_sort_depth_static(const uint32_t *depth_keys, int64_t n, ui
     const uint32_t *kin = p == 0 ? keys0 : s->keys[in];
     uint32_t *vout = p == kMaxPasses - 1 ? sorted_slots : s->vals[out];
     if (p == 0)
-      radix_pass_kernel<true, kSortItems, 1><<<blocks, kSortThreads, smem, st>>>(kin, nullptr, s->keys[out], vout, &s->ctl[0],
+      radix_pass_kernel<true, kSortItems><<<blocks, kSortThreads, smem, st>>>(kin, nullptr, s->keys[out], vout, &s->ctl[0],
                                                                FGS4D_STATIC_SORT_MAX, kRadixBits * p, s->hist[p],
                                                                &s->state[p][0][0], &s->ctl[8 + p], &s->ctl[1], nullptr, 0);
     else
-      radix_pass_kernel<false, kSortItems, 1><<<blocks, kSortThreads, smem, st>>>(kin, s->vals[in], s->keys[out], vout, &s->ctl[0],
+      radix_pass_kernel<false, kSortItems><<<blocks, kSortThreads, smem, st>>>(kin, s->vals[in], s->keys[out], vout, &s->ctl[0],
                                                                 FGS4D_STATIC_SORT_MAX, kRadixBits * p, s->hist[p],
                                                                 &s->state[p][0][0], &s->ctl[8 + p], &s->ctl[1], nullptr, 0);
   }

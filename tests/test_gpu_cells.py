@@ -1,0 +1,102 @@
+"""Two-level binning (cells of 8x8 tiles): instance lists and ranges against
+the oracle's sort on records written straight into the workspace, at the
+visible capacities that take it (65,536, and 1,024 per cell)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2412_20720_gb300 import fgs4d
+from paper_2412_20720_gb300 import synthetic as sy
+from paper_2412_20720_gb300.render import RenderConfig
+from helpers import canonical_ranges
+from test_gpu_parity import KEEP_ALL, _min_q_over_tile, _read_instances, _synthetic_records, _write_records
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(rec, views, tile, inst_cap, view_of_slot=0, stage_blocks=0, vis_cap=1 << 19):
+    from paper_2412_20720_gb300.render import Renderer
+    n = rec["rect"].shape[0]
+    cfg = RenderConfig(sh_degree=0, t_order=0, inst_capacity=inst_cap, tile=tile, vis_capacity=vis_cap,
+                       stage_blocks_per_sm=stage_blocks)
+    r = Renderer(n, views, cfg)
+    _write_records(r, rec, view_of_slot)
+    fgs4d.bin_sort(n, r.views, r.nviews, r.settings, r.ws.data_ptr(), r.ws_bytes, r.stream())
+    return r, r.status()
+
+
+# one cell; ragged grids whose last cells hold one tile row
+# or column; 8-pixel tiles with 352 cells (two cell-sort passes); lean grids;
+# rects that span up to 5 x 5 cells
+@pytest.mark.parametrize("n,W,H,tile,extent,stage_blocks", [
+    (3, 16, 16, 16, 2, 0), (16_384, 257, 257, 16, 6, 0), (20_001, 1157, 643, 16, 17, 1), (30_011, 1352, 1014, 8, 6, 0),
+    (16_385, 1013, 619, 8, 34, 2), (16_384, 4112, 16, 16, 40, 0)])
+def test_lists_equal_the_oracles(n, W, H, tile, extent, stage_blocks):
+    rng = np.random.default_rng(n + tile)
+    gw, gh = (W + tile - 1) // tile, (H + tile - 1) // tile
+    rec = _synthetic_records(rng, n, W, H, extent, tile=tile, tau=KEEP_ALL)
+    keys, vals, ranges = oracle.sort_instances(rec["rect"], rec["depth"], gw, gh)
+    m = keys.shape[0]
+    r, (code, counts) = _run(rec, [sy.tiny_view(W, H)], tile, m, stage_blocks=stage_blocks)  # exactly the capacity
+    assert code == fgs4d.OK and counts[1] == m and counts[3] == m
+    tiles, slots, gr = _read_instances(r, m, gw * gh)
+    np.testing.assert_array_equal(tiles, (keys >> np.uint64(32)).astype(np.int64))
+    np.testing.assert_array_equal(slots, vals)
+    np.testing.assert_array_equal(canonical_ranges(gr), ranges)
+
+
+def test_capacity_overflow_reports_the_need():
+    n, W, H = 16_384, 640, 480
+    rng = np.random.default_rng(3)
+    rec = _synthetic_records(rng, n, W, H, 9, tau=KEEP_ALL)
+    m = oracle.sort_instances(rec["rect"], rec["depth"], 40, 30)[0].shape[0]
+    for cap in (m - 1, m // 3, n // 2):  # the last holds fewer instances than there are pairs
+        _, (code, counts) = _run(rec, [sy.tiny_view(W, H)], 16, cap)
+        assert code == fgs4d.ERR_CAPACITY and counts[1] == cap and counts[3] == m
+
+
+def test_views_of_mixed_size():
+    sizes, ns = [(200, 150), (64, 48), (1014, 1352), (17, 700)], [5000, 500, 9000, 3000]
+    rng = np.random.default_rng(5)
+    recs = [_synthetic_records(rng, n, w, h, 9, tau=KEEP_ALL) for n, (w, h) in zip(ns, sizes)]
+    rec = {k: np.concatenate([x[k] for x in recs]) for k in recs[0]}
+    tiles_e, slots_e, ranges_e, tb, sb, ib = [], [], [], 0, 0, 0
+    for x, n, (w, h) in zip(recs, ns, sizes):
+        gw, gh = (w + 15) // 16, (h + 15) // 16
+        keys, vals, ranges = oracle.sort_instances(x["rect"], x["depth"], gw, gh)
+        tiles_e.append((keys >> np.uint64(32)).astype(np.int64) + tb)
+        slots_e.append(vals + sb)
+        ranges_e.append(np.where(ranges[:, 1:] > ranges[:, :1], ranges + ib, ranges))
+        tb, sb, ib = tb + gw * gh, sb + n, ib + keys.shape[0]
+    r, (code, counts) = _run(rec, [sy.tiny_view(w, h) for w, h in sizes], 16, ib,
+                             np.concatenate([np.full(n, k) for k, n in enumerate(ns)]))
+    assert code == fgs4d.OK and counts[1] == ib
+    tiles, slots, gr = _read_instances(r, ib, tb)
+    np.testing.assert_array_equal(tiles, np.concatenate(tiles_e))
+    np.testing.assert_array_equal(slots, np.concatenate(slots_e))
+    np.testing.assert_array_equal(canonical_ranges(gr), np.concatenate(ranges_e))
+
+
+@pytest.mark.parametrize("tile", [16, 8])
+def test_left_out_tiles_are_skipped_by_every_pixel(tile):
+    """With finite ellipses (round and elongated, up to 60:1) the list is an
+    order-preserving part of the rect membership, and a left-out pair has q >
+    tau - 4e-3 in FP64 at every pixel centre (4e-3: the margin of the records'
+    tau), so alpha < 1/255 there."""
+    n, W, H = 16_384, 45 * tile + 3, 37 * tile + 5
+    rng = np.random.default_rng(11 + tile)
+    gw, gh = (W + tile - 1) // tile, (H + tile - 1) // tile
+    rec = _synthetic_records(rng, n, W, H, 12, tile=tile)
+    keys, vals, _ = oracle.sort_instances(rec["rect"], rec["depth"], gw, gh)
+    r, (code, counts) = _run(rec, [sy.tiny_view(W, H)], tile, keys.shape[0])
+    assert code == fgs4d.OK
+    tiles, slots, _ = _read_instances(r, counts[1], gw * gh)
+    full = (keys >> np.uint64(32)).astype(np.int64) * n + vals
+    pos = {int(p): j for j, p in enumerate(full)}
+    jj = np.array([pos[int(p)] for p in tiles * n + slots])
+    assert np.all(np.diff(jj) > 0)
+    left = np.setdiff1d(np.arange(full.size), jj)
+    assert 0.2 * full.size < left.size < full.size
+    for j in rng.choice(left, 6000, replace=False):
+        t, i = divmod(int(full[j]), n)
+        assert _min_q_over_tile(rec, i, t % gw, t // gw, W, H, tile) > float(rec["tau"][i]) - 4e-3, (t, i)
