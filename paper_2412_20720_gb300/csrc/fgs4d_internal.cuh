@@ -34,6 +34,8 @@ constexpr int kCellPrefixThreads = 512;
 // cells (8 views, 1.9M) 168 / 194; 48,000 over 352 cells (8-pixel tiles) 91 /
 // 120; the 6-view street call (5.4M over 810 cells, 685M) 20,900 / 4,100.
 constexpr int64_t kCellsMinVisible = 65536, kCellsMinPerCell = 1024;
+// Visible slots up to which the depth sort ranks by counting.
+constexpr int64_t kRankSortMax = 8192;
 constexpr int64_t kPairScanWideMin = int64_t(1) << 19;
 constexpr int kRadixBits = 8;
 constexpr int kRadixBins = 1 << kRadixBits;

@@ -84,14 +84,14 @@ __global__ void __launch_bounds__(kSortThreads) radix_hist_kernel(const uint32_t
                                                                   const uint32_t *__restrict__ count_ptr, int64_t cap,
                                                                   int32_t passes, uint32_t *hist, uint32_t *state,
                                                                   int32_t state_blocks, uint2 *ranges,
-                                                                  int64_t nranges) {
+                                                                  int64_t nranges, int64_t small) {
   grid_dependency_sync();
   __shared__ uint32_t s_hist[kMaxPasses][kRadixBins];
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < nranges; r += (int64_t)gridDim.x * blockDim.x)
     ranges[r] = make_uint2(0u, 0u);
   const int64_t count = min64((int64_t)*count_ptr, cap);
   constexpr int kTileKeys = kSortThreads * kItems;
-  if ((int64_t)blockIdx.x * kTileKeys >= count) return;
+  if ((int64_t)blockIdx.x * kTileKeys >= count || count <= small) return;
   for (int p = 0; p < passes; ++p) s_hist[p][threadIdx.x] = 0u;
   __syncthreads();
   const uint32_t lane = threadIdx.x & 31u;
@@ -133,6 +133,50 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.wait_group 0;\n" ::: "memory");
 }
 
+// Stable order of few keys by counting: key i goes to place #{j : key_j <
+// key_i or (key_j = key_i and j < i)}.  A block takes 32 keys at a time, one
+// per lane, and its warps an eighth of the keys each to compare with (every
+// lane of a warp reads the same four keys per load).  n^2 comparisons over
+// the whole GPU take less time than the passes' launches and look-backs up to
+// kRankSortMax keys (see there).
+__device__ __forceinline__ void rank_sort(const uint32_t *__restrict__ keys, int n, uint32_t *__restrict__ out,
+                                          uint32_t (*s_cnt)[32]) {
+  constexpr int kWarps = kSortThreads / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int per = ((n + 32 * kWarps - 1) / (32 * kWarps)) * 32;  // keys per warp: whole groups of 32
+  const int a = min(warp * per, n), b = min(a + per, n);
+  for (int g = blockIdx.x * 32; g < n; g += gridDim.x * 32) {
+    const int i = g + lane;
+    const uint32_t ki = i < n ? keys[i] : 0u;
+    uint32_t cnt = 0u;
+    // Keys before the group count when equal (k < ki + 1: depth keys are
+    // below 2^31), keys behind it do not; in the group it depends on the lane.
+    for (int j0 = a; j0 < b; j0 += 32) {
+      const int m = min(b - j0, 32);
+      if (j0 == g) {
+        for (int k = 0; k < m; ++k) cnt += keys[j0 + k] < ki + (k < lane ? 1u : 0u);
+      } else {
+        const uint32_t lim = ki + (j0 < g ? 1u : 0u);
+        int k = 0;
+        for (; k + 4 <= m; k += 4) {
+          const uint4 q = *reinterpret_cast<const uint4 *>(keys + j0 + k);
+          cnt += (q.x < lim) + (q.y < lim) + (q.z < lim) + (q.w < lim);
+        }
+        for (; k < m; ++k) cnt += keys[j0 + k] < lim;
+      }
+    }
+    s_cnt[warp][lane] = cnt;
+    __syncthreads();
+    if (warp == 0 && i < n) {
+      uint32_t r = 0u;
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) r += s_cnt[w][lane];
+      out[r] = (uint32_t)i;
+    }
+    __syncthreads();
+  }
+}
+
 // Shared memory of one radix block: the ticket's keys and values (input,
 // then the block-local order), per-warp digit counts, the digits' block-local
 // and global starts.
@@ -145,6 +189,7 @@ struct RadixSmem {
   uint32_t gstart[kRadixBins];  // global position of the ticket's first key of each digit
   uint32_t scan[12];
   uint32_t ticket;
+  uint32_t scan_ranks[kSortThreads / 32][32];  // rank_sort: each warp's counts
 };
 template <int kItems>
 constexpr size_t radix_smem_bytes() {
@@ -176,7 +221,7 @@ __global__ void __launch_bounds__(kSortThreads) radix_pass_kernel(
     const uint32_t *__restrict__ keys_in, const uint32_t *__restrict__ vals_in, uint32_t *__restrict__ keys_out,
     uint32_t *__restrict__ vals_out, const uint32_t *__restrict__ count_ptr, int64_t cap, int32_t shift,
     const uint32_t *__restrict__ hist, uint32_t *state, uint32_t *ticket, uint32_t *status, uint2 *ranges,
-    int64_t total_tiles) {
+    int64_t total_tiles, int64_t small, uint32_t *__restrict__ small_out) {
   static_assert(kItems % 4 == 0, "whole 16-byte copies per warp segment");
   grid_dependency_sync();
   constexpr int kTileKeys = kSortThreads * kItems;
@@ -187,6 +232,10 @@ __global__ void __launch_bounds__(kSortThreads) radix_pass_kernel(
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t lt_mask = (1u << lane) - 1u;
   const int64_t count = min64((int64_t)*count_ptr, cap);
+  if (count <= small) {  // the first pass does all, the others nothing
+    if (kValsAreIndex && small_out) rank_sort(keys_in, (int)count, small_out, S.scan_ranks);
+    return;
+  }
   for (int i = threadIdx.x; i < (int)(sizeof S.wcount / sizeof(uint32_t)); i += kSortThreads) (&S.wcount[0][0])[i] = 0u;
   uint32_t total;
   // Keys of the digits below each digit over the whole input: the same for
@@ -785,7 +834,8 @@ cudaError_t bin_cells(const Layout &L, const EmitArgs &ea_in, const RasterViews<
                         (const uint32_t *)(ctr + kCtrCellPairs), (int64_t)L.inst_cap, (int32_t)(kRadixBits * p),
                         (const uint32_t *)(ea.hist_tile + p * kRadixBins),
                         ea.tile_state + (size_t)p * L.tile_blocks * kRadixBins, ctr + kCtrTicketTile + p,
-                        ctr + kCtrStatus, p == P - 1 ? C.cell_ranges : (uint2 *)nullptr, (int64_t)L.total_cells);
+                        ctr + kCtrStatus, p == P - 1 ? C.cell_ranges : (uint2 *)nullptr, (int64_t)L.total_cells,
+                        (int64_t)-1, (uint32_t *)nullptr);
     if (e != cudaSuccess) return e;
   }
   e = launch_pdl(cell_count_kernel, (unsigned)L.cell_grid, kCellBlock, st, C);
@@ -848,10 +898,12 @@ cudaError_t bin_sort_typed(const Layout &L, const fgs4d_view *views, int32_t nvi
     if (L.depth_blocks > 0) {
       const int hb = std::min(L.depth_blocks, L.sort_grid);
       const int pb = std::min(L.depth_blocks, L.sort_grid);
+      // the first pass ranks few keys 32 at a time: blocks beyond its own for those
+      const int pb0 = std::max(pb, (int)std::min<int64_t>((std::min(L.vis_cap, kRankSortMax) + 31) / 32, 152));
       constexpr size_t smem = radix_smem_bytes<kDepthSortItems>();
       e = launch_pdl(radix_hist_kernel<kDepthSortItems>, (unsigned)hb, kSortThreads, st, dkey,
                      (const uint32_t *)(ctr + kCtrVisible), (int64_t)L.vis_cap, (int32_t)L.depth_passes, hist_d,
-                     dstate, (int32_t)L.depth_blocks, (uint2 *)nullptr, (int64_t)0);
+                     dstate, (int32_t)L.depth_blocks, (uint2 *)nullptr, (int64_t)0, kRankSortMax);
       if (e != cudaSuccess) return e;
       for (int p = 0; p < L.depth_passes; ++p) {
         const int out = p & 1, in = out ^ 1;
@@ -860,10 +912,10 @@ cudaError_t bin_sort_typed(const Layout &L, const fgs4d_view *views, int32_t nvi
         const uint32_t *vin = p == 0 ? nullptr : dv[in];
         e = launch_pdl_smem(p == 0 ? radix_pass_kernel<true, kDepthSortItems>
                                    : radix_pass_kernel<false, kDepthSortItems>,
-                            (unsigned)pb, kSortThreads, smem, st, kin, vin, dk[out], dv[out],
+                            (unsigned)(p == 0 ? pb0 : pb), kSortThreads, smem, st, kin, vin, dk[out], dv[out],
                        (const uint32_t *)(ctr + kCtrVisible), (int64_t)L.vis_cap, (int32_t)(kRadixBits * p),
                        (const uint32_t *)(hist_d + p * kRadixBins), state, ctr + kCtrTicketDepth + p, status,
-                       (uint2 *)nullptr, (int64_t)0);
+                       (uint2 *)nullptr, (int64_t)0, kRankSortMax, p == 0 ? sorted : (uint32_t *)nullptr);
         if (e != cudaSuccess) return e;
       }
     }
@@ -886,7 +938,7 @@ cudaError_t bin_sort_typed(const Layout &L, const fgs4d_view *views, int32_t nvi
                         (const uint32_t *)iv[in], ik[out], iv[out], (const uint32_t *)(ctr + kCtrInstances),
                         (int64_t)L.inst_cap, (int32_t)(kRadixBits * p), (const uint32_t *)(hist_t + p * kRadixBins),
                         state, ctr + kCtrTicketTile + p, status, last ? ranges : (uint2 *)nullptr,
-                        (int64_t)L.total_tiles);
+                        (int64_t)L.total_tiles, (int64_t)-1, (uint32_t *)nullptr);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -1022,7 +1074,7 @@ extern "C" int fgs4d_sort_depth_static(const uint32_t *depth_keys, int64_t n, ui
   static_sort_init_kernel<<<1, 256, 0, st>>>(s, (uint32_t)n);
   radix_hist_kernel<kSortItems><<<blocks, kSortThreads, 0, st>>>(depth_keys, &s->ctl[0], FGS4D_STATIC_SORT_MAX,
                                                           kMaxPasses, &s->hist[0][0], &s->state[0][0][0],
-                                                          kStaticSortBlocks, nullptr, 0);
+                                                          kStaticSortBlocks, nullptr, 0, -1);
   // The passes stage keys with 16-byte copies: keys that do not start on a
   // 16-byte boundary are first copied into the buffer pass 0 does not write.
   const uint32_t *keys0 = depth_keys;
@@ -1039,11 +1091,11 @@ extern "C" int fgs4d_sort_depth_static(const uint32_t *depth_keys, int64_t n, ui
     if (p == 0)
       radix_pass_kernel<true, kSortItems><<<blocks, kSortThreads, smem, st>>>(kin, nullptr, s->keys[out], vout, &s->ctl[0],
                                                                FGS4D_STATIC_SORT_MAX, kRadixBits * p, s->hist[p],
-                                                               &s->state[p][0][0], &s->ctl[8 + p], &s->ctl[1], nullptr, 0);
+                                                               &s->state[p][0][0], &s->ctl[8 + p], &s->ctl[1], nullptr, 0, -1, nullptr);
     else
       radix_pass_kernel<false, kSortItems><<<blocks, kSortThreads, smem, st>>>(kin, s->vals[in], s->keys[out], vout, &s->ctl[0],
                                                                 FGS4D_STATIC_SORT_MAX, kRadixBits * p, s->hist[p],
-                                                                &s->state[p][0][0], &s->ctl[8 + p], &s->ctl[1], nullptr, 0);
+                                                                &s->state[p][0][0], &s->ctl[8 + p], &s->ctl[1], nullptr, 0, -1, nullptr);
   }
   return cudaGetLastError() == cudaSuccess ? FGS4D_OK : FGS4D_ERR_CUDA;
 }

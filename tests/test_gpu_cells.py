@@ -100,3 +100,17 @@ def test_left_out_tiles_are_skipped_by_every_pixel(tile):
     for j in rng.choice(left, 6000, replace=False):
         t, i = divmod(int(full[j]), n)
         assert _min_q_over_tile(rec, i, t % gw, t // gw, W, H, tile) > float(rec["tau"][i]) - 4e-3, (t, i)
+
+
+# one key; a group of 32 less and more one; the last count ranked by counting
+# and the first sorted by passes
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 257, 8191, 8192, 8193])
+def test_depth_order_of_few_slots(n):
+    import torch
+    rng = np.random.default_rng(n)
+    rec = _synthetic_records(rng, n, 320, 240, 3, tau=KEEP_ALL)
+    for cap in (n, 100_000):  # the count, not the capacity, decides
+        r, (code, _) = _run(rec, [sy.tiny_view(320, 240)], 16, 20 * n + 16, vis_cap=cap)
+        assert code == fgs4d.OK
+        got = r.workspace_view(r.layout.sorted_slots, torch.int32, n).cpu().numpy()
+        np.testing.assert_array_equal(got, np.argsort(rec["depth"], kind="stable"))
