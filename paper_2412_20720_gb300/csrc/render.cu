@@ -273,33 +273,6 @@ __global__ void __launch_bounds__(TILE *TILE / PPT, (fwd_min_blocks<TILE, PPT, k
   }
 }
 
-// Sums eight per-lane values over the warp with 9 shuffles instead of 40: at
-// each halving step a lane keeps half of its values and trades the other half
-// with its partner.  On return a[0] of lane l holds the warp total of value
-// l >> 2.
-__device__ __forceinline__ void warp_sum8_transposed(float (&a)[8], int lane) {
-  const bool u16 = (lane & 16) != 0, u8 = (lane & 8) != 0, u4 = (lane & 4) != 0;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float send = u16 ? a[i] : a[i + 4];
-    const float keep = u16 ? a[i + 4] : a[i];
-    a[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const float send = u8 ? a[i] : a[i + 2];
-    const float keep = u8 ? a[i + 2] : a[i];
-    a[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-  }
-  {
-    const float send = u4 ? a[0] : a[1];
-    const float keep = u4 ? a[1] : a[0];
-    a[0] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-  }
-  a[0] += __shfl_xor_sync(0xffffffffu, a[0], 2);
-  a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
-}
-
 // 1/x to within an ulp or so (MUFU reciprocal); the backward pass only needs
 // T recovered to the accuracy of its own accumulated rounding.
 __device__ __forceinline__ float rcp_approx(float x) {
@@ -308,19 +281,53 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return y;
 }
 
+// Gradient sums of one (warp, entry): kRedSums rows of 32 lanes, in the order
+// S_x0, S_1, S_xx, S_x1, S_2, S_0 (moments of gp, below), dr, dg, db, [dz].
+template <bool kAux>
+__host__ __device__ constexpr int red_sums() {
+  return kAux ? 10 : 9;
+}
+constexpr int kRedEntries = 3;  // entries per reduction: 3 x 9 or 10 sums, one per lane
+constexpr int kRedStride = 36;  // floats per row: 16-byte rows whose float4 reads by 8 lanes hit 32 banks
+
+// Resident blocks asked of the compiler for strips on 16x16 tiles: 4 pixels,
+// 16 blocks of 64 threads (64 registers, no spills; 12 at 80 with the
+// auxiliary channels); 8 pixels, 18 of 32 threads (95 registers and 21 blocks
+// instead of 117 and 17).
+template <int TILE, int PPT, bool kAux>
+constexpr int bwd_min_blocks() {
+  if (TILE != 16) return 1;
+  return PPT == 4 ? (kAux ? 12 : 16) : (PPT == 8 && !kAux ? 18 : 1);
+}
+
+// Reverse traversal of a tile's list.  The kernel is bound by instruction
+// issue (86 % of the slots at 4 views of 1352x1014), so a thread's pixels are
+// taken in pairs with two-lane FP32 instructions: a skipped pixel takes part
+// with alpha = 0, which leaves its T and its sums unchanged (1/(1 - 0) = 1),
+// and a pair is skipped when neither pixel composites the entry.  The sums
+// over the warp's pixels go through shared memory: the lanes' partial sums of
+// kRedEntries entries are rows, and each lane then adds up one row (8 float4
+// loads) and adds it with one atomic -- about 25 warp instructions an entry
+// where the transposed shuffle butterfly and its operands took about 70.
+// Train call of 4 views: see launch_bwd_batch for the measured times.
+//
 // kAux: the loss also has gradients dL/dD, dL/dO with respect to the depth
 // and opacity channels (zero background, x_i = z_i resp. 1 in the colour
 // rule); adds dL/dz_i = sum dL/dD alpha_i T_i per slot.
 template <int MAXV, int TILE, int kPPT, bool kAux, int kBatch>
-__global__ void __launch_bounds__(TILE *TILE / kPPT) render_bwd_kernel(RenderBwdArgs A, RasterViews<MAXV> rv) {
+__global__ void __launch_bounds__(TILE *TILE / kPPT, (bwd_min_blocks<TILE, kPPT, kAux>())) render_bwd_kernel(RenderBwdArgs A, RasterViews<MAXV> rv) {
   grid_dependency_sync();
   constexpr int kRenderThreads = TILE * TILE / kPPT;
+  constexpr int kPairs = (kPPT + 1) / 2;  // a 1-pixel strip leaves its second lane empty
+  constexpr int kSums = red_sums<kAux>();
   __shared__ float4 s_geom[kBatch];
   __shared__ float4 s_col[kBatch];
   __shared__ float s_blue[kBatch];
   __shared__ float4 s_aux[kAux ? kBatch : 1];
   __shared__ uint32_t s_slot[kBatch];
   __shared__ uint32_t s_maxlast;
+  __shared__ int s_jb[kRenderThreads / 32][kRedEntries];
+  __shared__ __align__(16) float s_red[kRenderThreads / 32][kRedEntries * kSums][kRedStride];
   const int32_t gt = blockIdx.x;
   const RasterView &V = rv.v[find_view<MAXV>(rv, gt)];
   const int32_t lt = gt - V.tile_base;
@@ -330,45 +337,52 @@ __global__ void __launch_bounds__(TILE *TILE / kPPT) render_bwd_kernel(RenderBwd
   const uint2 range = tile_range(A.ranges, gt);
   const float pxc = (float)px + 0.5f;
   const int64_t HW = (int64_t)V.width * V.height;
-  // Dr[k] = sum over channels of dL/dX * (X composited behind the current
-  // entry), X = R, G, B (and depth, opacity): the "behind" terms of
-  // dL/dalpha enter only through this sum, which grows by w * (dL/dX . x_i).
   constexpr int kGroups = (kPPT + 3) / 4;  // row groups of the strip (see group_w)
   float gyc[kGroups];
 #pragma unroll
   for (int g = 0; g < kGroups; ++g) gyc[g] = row_group_centre(py0 + 4 * g);
-  // Row offsets of the strip's pixels within their groups: -(k mod 4) when
-  // the strip starts a group (4 and 8 rows), else -((py0 + k) mod 4).
+  // Row offset of the strip's first pixel within its group: 0 when the strip
+  // starts a group (4 and 8 rows), else -(py0 mod 4).
   const float base_off = row_offset(py0);
-  float T[kPPT], dC0[kPPT], dC1[kPPT], dC2[kPPT], Dr[kPPT], off[kPPT];
-  float dD[kAux ? kPPT : 1], dO[kAux ? kPPT : 1];
-  uint32_t last[kPPT];
+  // Dr = sum over channels of dL/dX * (X composited behind the current
+  // entry), X = R, G, B (and depth, opacity): the "behind" terms of
+  // dL/dalpha enter only through this sum, which grows by w * (dL/dX . x_i).
+  // nC0, nC1, nC2, nD, nO: the upstream gradients, negated (see entry()).
+  float2 T[kPairs], nC0[kPairs], nC1[kPairs], nC2[kPairs], Dr[kPairs];
+  float2 nD[kAux ? kPairs : 1], nO[kAux ? kPairs : 1];
+  uint32_t last[2 * kPairs];
   uint32_t my_max = 0u;
   const float *g = A.dL_drgb + V.pix_base * 3;
+  bool finite = true;  // every upstream gradient of the thread, then of the warp (see entry())
 #pragma unroll
-  for (int k = 0; k < kPPT; ++k) {
-    off[k] = row_offset(py0 + k);
-    T[k] = 1.0f;
-    dC0[k] = dC1[k] = dC2[k] = 0.f;
+  for (int k = 0; k < 2 * kPairs; ++k) {
+    float t = 1.0f, c0 = 0.f, c1 = 0.f, c2 = 0.f, d = 0.f, o = 0.f;
     last[k] = 0u;
-    if (px < V.width && py0 + k < V.height) {
+    if (k < kPPT && px < V.width && py0 + k < V.height) {
       const int64_t p = (int64_t)(py0 + k) * V.width + px;
-      T[k] = A.pix_T[V.pix_base + p];
+      t = A.pix_T[V.pix_base + p];
       last[k] = A.pix_last[V.pix_base + p];
-      dC0[k] = g[p];
-      dC1[k] = g[HW + p];
-      dC2[k] = g[2 * HW + p];
-    }
-    if (kAux) {
-      dD[k] = dO[k] = 0.f;
-      if (px < V.width && py0 + k < V.height) {
-        const int64_t p = (int64_t)(py0 + k) * V.width + px;
+      c0 = g[p];
+      c1 = g[HW + p];
+      c2 = g[2 * HW + p];
+      if (kAux) {
         const float *ga = A.dL_daux + V.pix_base * 4;
-        dD[k] = ga[p];
-        dO[k] = ga[HW + p];
+        d = ga[p];
+        o = ga[HW + p];
       }
     }
-    Dr[k] = T[k] * (dC0[k] * A.bg0 + dC1[k] * A.bg1 + dC2[k] * A.bg2);  // the background behind all
+    finite = finite && isfinite(c0) && isfinite(c1) && isfinite(c2) && isfinite(d) && isfinite(o);
+    const float dr = t * (c0 * A.bg0 + c1 * A.bg1 + c2 * A.bg2);  // the background behind all
+    auto lane = [k](float2 &v, float x) { (k & 1 ? v.y : v.x) = x; };
+    lane(T[k >> 1], t);
+    lane(nC0[k >> 1], -c0);
+    lane(nC1[k >> 1], -c1);
+    lane(nC2[k >> 1], -c2);
+    lane(Dr[k >> 1], dr);
+    if (kAux) {
+      lane(nD[k >> 1], -d);
+      lane(nO[k >> 1], -o);
+    }
     my_max = max(my_max, last[k]);
   }
   if (threadIdx.x == 0) s_maxlast = 0u;
@@ -376,18 +390,75 @@ __global__ void __launch_bounds__(TILE *TILE / kPPT) render_bwd_kernel(RenderBwd
   if (my_max) atomicMax(&s_maxlast, my_max);
   __syncthreads();
   const uint32_t end = range.x + min(s_maxlast, range.y - range.x);
+  const uint32_t warp_max = __reduce_max_sync(0xffffffffu, my_max);  // past the last entry of the warp's pixels
+  finite = __all_sync(0xffffffffu, finite);
   const int lane = threadIdx.x & 31;
+  float(*red)[kRedStride] = s_red[threadIdx.x >> 5];
+  int buffered = 0;  // entries in `red` (the same in every lane)
+  int *jb = s_jb[threadIdx.x >> 5];  // their positions in the batch
+  // Sums the buffered rows and adds them to the slots.  Lane e kSums + r sums
+  // row r of entry e; the centre and conic gradients follow from the moments
+  // with the natural-log conic (An, Bn, Cn) of the record's factors (A' =
+  // a1^2 + b1^2, B' = 2 b1 b2, C' = b2^2 in base 2):
+  //   du = -(An S_x0 + Bn S_1)   dv = -(Cn S_1 + Bn S_x0)
+  //   dA = -S_xx / 2   dB = -S_x1   dC = -S_2 / 2   da = S_0 / a
+  auto flush = [&]() {
+    __syncwarp();
+    const int e = lane / kSums, r = lane - e * kSums;
+    const bool on = e < buffered;
+    float own = 0.f;
+    if (on) {  // pairwise, lanes 16, 8, 4, 2 and 1 apart
+      const float4 *row = reinterpret_cast<const float4 *>(red[lane]);
+      float2 y[8];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 u = row[q], v = row[q + 4];
+        y[2 * q] = __fadd2_rn(make_float2(u.x, u.y), make_float2(v.x, v.y));
+        y[2 * q + 1] = __fadd2_rn(make_float2(u.z, u.w), make_float2(v.z, v.w));
+      }
+#pragma unroll
+      for (int h = 4; h >= 1; h >>= 1)
+#pragma unroll
+        for (int q = 0; q < h; ++q) y[q] = __fadd2_rn(y[q], y[q + h]);
+      own = y[0].x + y[0].y;
+    }
+    const float other = __shfl_sync(0xffffffffu, own, r == 0 ? lane + 1 : (r == 1 ? lane - 1 : lane));
+    if (on) {
+      const int j = jb[e];
+      const float4 geom = s_geom[j];
+      const float2 ca = *reinterpret_cast<const float2 *>(&s_col[j]);
+      const float k2 = -2.0f * kLn2;
+      float m = r == 5 ? ex2_approx(-ca.y) : 1.0f;
+      if (r == 0) m = k2 * __fmaf_rn(geom.z, geom.z, geom.w * geom.w);
+      if (r == 1) m = k2 * (ca.x * ca.x);
+      if (r == 2 || r == 4) m = -0.5f;
+      if (r == 3) m = -1.0f;
+      float out = m * own;
+      if (r < 2) out = __fmaf_rn(k2 * (geom.w * ca.x), other, out);
+      const uint32_t slot = s_slot[j];
+      if (slot < A.vis_cap) atomicAdd(reinterpret_cast<float *>(A.slot_grad + 3 * (size_t)slot) + r, out);
+    }
+    __syncwarp();  // the rows may be overwritten
+    buffered = 0;
+  };
   const int nbatch = (int)((end - range.x + kBatch - 1) / kBatch);
   for (int bi = nbatch - 1; bi >= 0; --bi) {
     const uint32_t base = range.x + (uint32_t)bi * kBatch;
     __syncthreads();
     stage_batch<kRenderThreads, kBatch>(A.inst_val, A.rec_geom, A.rec_color, A.rec_blue, A.vis_cap, base, end, s_geom,
                                 s_col, s_blue, s_slot, kAux ? A.rec_aux : nullptr, kAux ? s_aux : nullptr);
-    __syncthreads();
     const int nb = (int)min(end - base, (uint32_t)kBatch);
-    // One list entry; kClamp is the entry's clamp case (entry_clamps), taken
-    // per entry as in the forward so that pixels evaluate pixel_alpha<false>
-    // without a per-pixel select for the vast majority of entries.
+    // Whether any staged entry can reach the 0.99 clamp (rare): then the batch
+    // takes the clamping copy of the pixel loop, which gives the entries that
+    // cannot clamp the same alpha.
+    bool my_clamp = false;
+#pragma unroll
+    for (int i = 0; i < kBatch / kRenderThreads; ++i) {
+      const int k = threadIdx.x + i * kRenderThreads;
+      if (k < nb) my_clamp = my_clamp || entry_clamps(s_col[k].y);
+    }
+    const bool clamp_any = __syncthreads_or(my_clamp) != 0;
+    // One list entry.
     auto entry = [&](int j, uint32_t pos, auto clamp_tag) {
       constexpr bool kClamp = decltype(clamp_tag)::value;
       const float4 geom = s_geom[j];
@@ -401,89 +472,125 @@ __global__ void __launch_bounds__(TILE *TILE / kPPT) render_bwd_kernel(RenderBwd
         dy4[g] = __fsub_rn(geom.y, gyc[g]);
         w4[g] = __fmaf_rn(col.x, dy4[g], ct.bdx);
       }
-      // The conic and centre gradients of the strip share dx: accumulate the
-      // moments S0 = sum gp, S1 = sum gp dy, S2 = sum gp dy^2 of
-      // gp = dL/d(natural-log power) and form the five sums once per entry.
-      // A pixel that is not skipped has alpha = a 2^-q (below the clamp), so
-      // gp = g_alpha a 2^-q is also the opacity term: dL/da = S0 / a.
-      // Per row group: P0 = sum gp, P1 = sum o gp, P2 = sum o^2 gp with the
-      // pixel's dy = dyb - o, o = k mod 4 (a constant of the unrolled loop),
-      // so that S1 = dyb P0 - P1 and S2 = dyb^2 P0 - 2 dyb P1 + P2 follow
-      // once per entry.
-      float P0[kGroups], P1[kGroups], P2[kGroups];
-#pragma unroll
-      for (int g = 0; g < kGroups; ++g) P0[g] = P1[g] = P2[g] = 0.f;
-      float gr = 0.f, gg = 0.f, gb = 0.f, gz = 0.f;
       const float zj = kAux ? s_aux[j].x : 0.f;
-      bool contrib = false;
+      // gp = dL/d(natural-log power) of each pixel; a pixel that is not
+      // skipped has alpha = a 2^-q (below the clamp), so gp = g_alpha a 2^-q
+      // is also the opacity term: dL/da = S_0 / a.
+      float2 gp[kPairs], gr = make_float2(0.f, 0.f), gg = gr, gb = gr, gz = gr;
+      bool contrib = false;  // the same in every lane
 #pragma unroll
-      for (int k = 0; k < kPPT; ++k) {
-        if (pos >= last[k]) continue;
-        const AlphaEval e = pixel_alpha<kClamp>(ct, w4[k >> 2], col.x, kPPT >= 4 ? -(float)(k & 3) : off[k]);
-        if (!(e.alpha >= kAlphaMin)) continue;  // the forward's skip decision, NaN included
+      for (int q = 0; q < kPairs; ++q) {
+        gp[q] = make_float2(0.f, 0.f);
+        const int k0 = 2 * q, k1 = 2 * q + 1;
+        // the two lanes of pixel_alpha
+        const float2 offs = kPPT >= 4 ? make_float2(-(float)(k0 & 3), -(float)(k1 & 3))
+                                      : make_float2(base_off - (float)k0, base_off - (float)k1);
+        const float wg = w4[k0 >> 2];
+        const float2 w2 = __ffma2_rn(make_float2(col.x, col.x), offs, make_float2(wg, wg));
+        const float2 q2 = __ffma2_rn(w2, w2, make_float2(ct.adx2, ct.adx2));
+        const float aG0 = ex2_approx(-q2.x), aG1 = ex2_approx(-q2.y);
+        const float al0 = kClamp ? min_nan(0.99f, aG0) : aG0, al1 = kClamp ? min_nan(0.99f, aG1) : aG1;
+        // the forward's skip decision, NaN included, up to the pixel's last entry
+        const bool v0 = pos < last[k0] && al0 >= kAlphaMin, v1 = pos < last[k1] && al1 >= kAlphaMin;
+        if (!__any_sync(0xffffffffu, v0 || v1)) continue;
         contrib = true;
-        const float io = rcp_approx(__fsub_rn(1.0f, e.alpha));
-        T[k] = T[k] * io;  // transmittance in front of this entry
-        const float w = e.alpha * T[k];
-        gr += dC0[k] * w;
-        gg += dC1[k] * w;
-        gb += dC2[k] * w;
-        float Dc = dC0[k] * col.z + dC1[k] * col.w + dC2[k] * blue;  // dL/dX . x_i
-        if (kAux) {
-          Dc += dD[k] * zj + dO[k];
-          gz += dD[k] * w;
+        if (!finite) {  // an infinite or NaN gradient of a skipped pixel must not meet its zero weight: one at a time
+          auto pixel = [&](bool v, float al, float aG, float &t, float &dr, float n0, float n1, float n2, float nd,
+                           float no, float &sr, float &sg, float &sb, float &sz, float &gpk) {
+            if (!v) return;
+            const float io = rcp_approx(__fsub_rn(1.0f, al));
+            t = t * io;
+            const float nw = -al * t;
+            sr = __fmaf_rn(n0, nw, sr);
+            sg = __fmaf_rn(n1, nw, sg);
+            sb = __fmaf_rn(n2, nw, sb);
+            float nDc = __fmaf_rn(n2, blue, __fmaf_rn(n0, col.z, n1 * col.w));
+            if (kAux) {
+              nDc += __fmaf_rn(nd, zj, no);
+              sz = __fmaf_rn(nd, nw, sz);
+            }
+            if (!(kClamp && aG > 0.99f)) gpk = __fmaf_rn(t, nDc, io * dr) * -al;
+            dr = __fmaf_rn(nw, nDc, dr);
+          };
+          const float2 nd = kAux ? nD[q] : gz, no = kAux ? nO[q] : gz;
+          pixel(v0, al0, aG0, T[q].x, Dr[q].x, nC0[q].x, nC1[q].x, nC2[q].x, nd.x, no.x, gr.x, gg.x, gb.x, gz.x, gp[q].x);
+          pixel(v1, al1, aG1, T[q].y, Dr[q].y, nC0[q].y, nC1[q].y, nC2[q].y, nd.y, no.y, gr.y, gg.y, gb.y, gz.y, gp[q].y);
+          continue;
         }
-        const float g_alpha = T[k] * Dc - io * Dr[k];
-        Dr[k] += w * Dc;
-        if (!(kClamp && e.aG > 0.99f)) {  // min(0.99, .) is locally constant when clamped
-          const float gp = g_alpha * e.alpha;  // d alpha / d (natural-log power)
-          const float o = (float)(k & 3);
-          P0[k >> 2] += gp;
-          if (k & 3) {
-            P1[k >> 2] = __fmaf_rn(o, gp, P1[k >> 2]);
-            P2[k >> 2] = __fmaf_rn(o * o, gp, P2[k >> 2]);
-          }
+        const float2 na = make_float2(v0 ? -al0 : 0.0f, v1 ? -al1 : 0.0f);  // -alpha
+        const float2 om = __fadd2_rn(make_float2(1.0f, 1.0f), na);
+        const float2 io = make_float2(rcp_approx(om.x), rcp_approx(om.y));
+        T[q] = __fmul2_rn(T[q], io);               // transmittance in front of this entry
+        const float2 nw = __fmul2_rn(na, T[q]);    // -alpha T
+        gr = __ffma2_rn(nC0[q], nw, gr);
+        gg = __ffma2_rn(nC1[q], nw, gg);
+        gb = __ffma2_rn(nC2[q], nw, gb);
+        // -(dL/dX . x_i)
+        float2 nDc = __ffma2_rn(nC2[q], make_float2(blue, blue),
+                                __ffma2_rn(nC0[q], make_float2(col.z, col.z), __fmul2_rn(nC1[q], make_float2(col.w, col.w))));
+        if (kAux) {
+          nDc = __fadd2_rn(nDc, __ffma2_rn(nD[q], make_float2(zj, zj), nO[q]));
+          gz = __ffma2_rn(nD[q], nw, gz);
+        }
+        const float2 nga = __ffma2_rn(T[q], nDc, __fmul2_rn(io, Dr[q]));  // -dL/dalpha
+        Dr[q] = __ffma2_rn(nw, nDc, Dr[q]);
+        gp[q] = __fmul2_rn(nga, na);
+        if (kClamp) {  // min(0.99, .) is locally constant when clamped
+          if (aG0 > 0.99f) gp[q].x = 0.0f;
+          if (aG1 > 0.99f) gp[q].y = 0.0f;
         }
       }
-      if (!__any_sync(0xffffffffu, contrib)) return;
-      // the strip's moments S0 = sum gp, S1 = sum gp dy, S2 = sum gp dy^2
+      if (!contrib) return;
+      // Moments S_0 = sum gp, S_1 = sum gp dy, S_2 = sum gp dy^2 of the strip.
+      // Per row group dy = dyb - o with o the pixel's row in the group, so
+      // with P_n = sum o^n gp: S_1 = dyb P_0 - P_1, S_2 = dyb (dyb P_0 - 2
+      // P_1) + P_2.
       float S0 = 0.f, S1 = 0.f, S2 = 0.f;
 #pragma unroll
       for (int g = 0; g < kGroups; ++g) {
         const float dyb = dy4[g] + base_off;  // dy of the group's first row in the strip
-        S0 += P0[g];
-        S1 += dyb * P0[g] - P1[g];
-        S2 += dyb * (dyb * P0[g] - 2.0f * P1[g]) + P2[g];
+        float P0, P1, P2;
+        if (kPPT >= 4) {
+          const float2 ga = gp[2 * g], gc = gp[2 * g + 1 < kPairs ? 2 * g + 1 : 0];
+          P0 = ((ga.x + ga.y) + gc.x) + gc.y;
+          P1 = __fmaf_rn(3.0f, gc.y, __fmaf_rn(2.0f, gc.x, ga.y));
+          P2 = __fmaf_rn(9.0f, gc.y, __fmaf_rn(4.0f, gc.x, ga.y));
+        } else {
+          P0 = gp[0].x + gp[0].y;
+          P1 = P2 = gp[0].y;
+        }
+        S0 += P0;
+        S1 += __fmaf_rn(dyb, P0, -P1);
+        S2 += __fmaf_rn(dyb, __fmaf_rn(dyb, P0, -2.0f * P1), P2);
       }
-      const float dx = ct.dx;
-      // the natural-log conic (A, B, C) of the record's factors: A' = a1^2 +
-      // b1^2, B' = 2 b1 b2, C' = b2^2 in base 2
-      const float An = 2.0f * kLn2 * __fmaf_rn(geom.z, geom.z, geom.w * geom.w);
-      const float Bn = 2.0f * kLn2 * (geom.w * col.x), Cn = 2.0f * kLn2 * (col.x * col.x);
-      // g = (du, dv, dA', dB', dC', da, dr, dg), plus db.
-      float g[8] = {-(An * dx * S0 + Bn * S1), -(Cn * S1 + Bn * dx * S0), -0.5f * dx * dx * S0, -dx * S1,
-                    -0.5f * S2, S0 * ex2_approx(-col.y), gr, gg};
-      warp_sum8_transposed(g, lane);
-      gb = warp_sum(gb);
-      if (kAux) gz = warp_sum(gz);
-      // Lane 4k holds sum k: lanes 0 and 16 gather sums 0-3 and 4-7 and add
-      // them with one vector atomic each; lane 1 adds (db, dz).
-      const float s1 = __shfl_down_sync(0xffffffffu, g[0], 4);
-      const float s2 = __shfl_down_sync(0xffffffffu, g[0], 8);
-      const float s3 = __shfl_down_sync(0xffffffffu, g[0], 12);
-      const uint32_t slot = s_slot[j];
-      if (slot < A.vis_cap) {
-        float4 *dst = A.slot_grad + 3 * (size_t)slot;
-        if ((lane & 15) == 0) atomicAdd(dst + (lane >> 4), make_float4(g[0], s1, s2, s3));
-        else if (lane == 1) atomicAdd(reinterpret_cast<float2 *>(dst + 2), make_float2(gb, kAux ? gz : 0.0f));
-      }
+      float *dst = &red[buffered * kSums][lane];
+      dst[0 * kRedStride] = ct.dx * S0;
+      dst[1 * kRedStride] = S1;
+      dst[2 * kRedStride] = (ct.dx * ct.dx) * S0;
+      dst[3 * kRedStride] = ct.dx * S1;
+      dst[4 * kRedStride] = S2;
+      dst[5 * kRedStride] = S0;
+      dst[6 * kRedStride] = gr.x + gr.y;
+      dst[7 * kRedStride] = gg.x + gg.y;
+      dst[8 * kRedStride] = gb.x + gb.y;
+      if (kAux) dst[(kSums - 1) * kRedStride] = gz.x + gz.y;
+      if (lane == 0) jb[buffered] = j;
+      ++buffered;
     };
-    for (int j = nb - 1; j >= 0; --j) {
-      const uint32_t pos = base + j - range.x;  // entry index in the tile list
-      if (!__any_sync(0xffffffffu, pos < my_max)) continue;  // no pixel of this warp reached it
-      if (entry_clamps(s_col[j].y)) entry(j, pos, std::true_type());
-      else entry(j, pos, std::false_type());
+    const uint32_t pos0 = base - range.x;  // entry index of the batch's first entry
+    const int first = warp_max > pos0 ? (int)min(warp_max - pos0, (uint32_t)nb) - 1 : -1;
+    if (clamp_any) {
+      for (int j = first; j >= 0; --j) {
+        entry(j, pos0 + j, std::true_type());
+        if (buffered == kRedEntries) flush();
+      }
+    } else {
+      for (int j = first; j >= 0; --j) {
+        entry(j, pos0 + j, std::false_type());
+        if (buffered == kRedEntries) flush();
+      }
     }
+    if (buffered) flush();  // the batch's records are about to be replaced
   }
 }
 
@@ -693,8 +800,11 @@ cudaError_t launch_bwd_batch(const RenderBwdArgs &A, const RasterViews<MAXV> &rv
 template <int MAXV, int TILE, int PPT>
 cudaError_t launch_bwd_ppt(const RenderBwdArgs &A, const RasterViews<MAXV> &rv, unsigned grid, int batch,
                            cudaStream_t st) {
-  if (batch == 128) return launch_bwd_batch<MAXV, TILE, PPT, 128>(A, rv, grid, st);
-  return launch_bwd_batch<MAXV, TILE, PPT, 256>(A, rv, grid, st);
+  // Default 128: with the reduction rows a block of 64 threads then takes 13
+  // KB of shared memory instead of 18, so that shared memory does not bound
+  // the resident blocks below the registers' 16.
+  if (batch == 256) return launch_bwd_batch<MAXV, TILE, PPT, 256>(A, rv, grid, st);
+  return launch_bwd_batch<MAXV, TILE, PPT, 128>(A, rv, grid, st);
 }
 
 template <int MAXV>
