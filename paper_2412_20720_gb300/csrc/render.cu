@@ -109,12 +109,12 @@ __device__ __forceinline__ void stage_batch(const uint32_t *inst_val, const floa
 // no flag.  The update stays a branch: whole warps skip it for entries that
 // miss all their pixels.
 // Resident blocks per SM asked of the compiler for the image-only form of the
-// 64-thread 4-pixel-strip blocks: 20 (at most 51 registers a thread, 48 used,
-// no spills) instead of 18 at 56, for frames rendered concurrently.  The form
-// that keeps the backward's state (mode 0) loses with the same bound.
+// 64-thread 4-pixel-strip blocks: 18 (56 registers, no spills).  At 20 (48
+// registers) the pixel pairs spill: 16 views, 8 frames in flight, 3.32 ms
+// against 3.07.
 template <int TILE, int PPT, int kMode>
 constexpr int fwd_min_blocks() {
-  return (TILE == 16 && PPT == 4 && kMode == 3) ? 20 : 1;
+  return (TILE == 16 && PPT == 4 && kMode == 3) ? 18 : 1;
 }
 
 template <int MAXV, int TILE, int PPT, int kMode, int kBatch>
@@ -141,20 +141,30 @@ __global__ void __launch_bounds__(TILE *TILE / PPT, (fwd_min_blocks<TILE, PPT, k
   float gyc[kGroups];
 #pragma unroll
   for (int g = 0; g < kGroups; ++g) gyc[g] = row_group_centre(py0 + 4 * g);
-  float T[PPT], C0[PPT], C1[PPT], C2[PPT], off[PPT];
-  float X0[kAux ? PPT : 1], X1[kAux ? PPT : 1], X2[kAux ? PPT : 1];  // depth, flow_u, flow_v sums
-  uint32_t last[PPT];
-  uint32_t pend[kStats ? PPT : 1];  // evaluations since the pixel's last composited entry
+  // Pixel k is lane k & 1 of pair k >> 1 (a 1-pixel strip leaves the second
+  // lane outside the image).
+  constexpr int kPairs = (PPT + 1) / 2;
+  float2 T[kPairs], C0[kPairs], C1[kPairs], C2[kPairs], off[kPairs];
+  float2 X0[kAux ? kPairs : 1], X1[kAux ? kPairs : 1], X2[kAux ? kPairs : 1];  // depth, flow_u, flow_v sums
+  uint32_t last[2 * kPairs];
+  uint32_t pend[kStats ? 2 * kPairs : 1];  // evaluations since the pixel's last composited entry
   int nlive = 0;  // pixels of this thread still compositing
 #pragma unroll
-  for (int k = 0; k < PPT; ++k) {
-    const bool in = px < V.width && py0 + k < V.height;
+  for (int k = 0; k < 2 * kPairs; ++k) {
+    const bool in = k < PPT && px < V.width && py0 + k < V.height;
+    const int q = k >> 1;
     if (kStats) pend[k] = 0u;
-    T[k] = in ? 1.0f : -1.0f;
-    C0[k] = C1[k] = C2[k] = 0.f;
-    if (kAux) X0[k] = X1[k] = X2[k] = 0.f;
+    const float t = in ? 1.0f : -1.0f, o = in ? row_offset(py0 + k) : stopped_offset();
+    if (k & 1) {
+      T[q].y = t;
+      off[q].y = o;
+    } else {
+      T[q].x = t;
+      off[q].x = o;
+      C0[q] = C1[q] = C2[q] = make_float2(0.f, 0.f);
+      if (kAux) X0[q] = X1[q] = X2[q] = make_float2(0.f, 0.f);
+    }
     last[k] = 0u;
-    off[k] = in ? row_offset(py0 + k) : stopped_offset();
     nlive += in;
   }
   uint32_t n_eval = 0u, n_comp = 0u, n_evb = 0u;
@@ -174,9 +184,12 @@ __global__ void __launch_bounds__(TILE *TILE / PPT, (fwd_min_blocks<TILE, PPT, k
     }
     const bool clamp_any = __syncthreads_or(my_clamp) != 0;
     const uint32_t pos0 = base - range.x + 1u;
-    // One entry of the list at every pixel of the thread; the clamp case is a
-    // separate copy of the pixel loop.
+    // One entry of the list at every pixel of the thread, two pixels at a time
+    // with two-lane FP32 instructions (each lane rounds as the scalar one
+    // does); a skipped pixel takes part with alpha = 0, which changes nothing.
+    // The clamp case is a separate copy of the pixel loop.
     auto entry = [&](int j, auto clamp_tag) {
+      constexpr bool kClamp = decltype(clamp_tag)::value;
       const float4 geom = s_geom[j];
       const float4 col = s_col[j];
       const float blue = s_blue[j];
@@ -186,34 +199,70 @@ __global__ void __launch_bounds__(TILE *TILE / PPT, (fwd_min_blocks<TILE, PPT, k
 #pragma unroll
       for (int g = 0; g < kGroups; ++g) w4[g] = group_w(ct, geom.y, col.x, gyc[g]);
 #pragma unroll
-      for (int k = 0; k < PPT; ++k) {
-        const AlphaEval e = pixel_alpha<decltype(clamp_tag)::value>(ct, w4[k >> 2], col.x, off[k]);
+      for (int q = 0; q < kPairs; ++q) {
+        // the two lanes of pixel_alpha
+        const float wg = w4[q >> 1];
+        const float2 w2 = __ffma2_rn(make_float2(col.x, col.x), off[q], make_float2(wg, wg));
+        const float2 q2 = __ffma2_rn(w2, w2, make_float2(ct.adx2, ct.adx2));
+        const float aG0 = ex2_approx(-q2.x), aG1 = ex2_approx(-q2.y);
+        const float al0 = kClamp ? min_nan(0.99f, aG0) : aG0, al1 = kClamp ? min_nan(0.99f, aG1) : aG1;
         if (kStats) {
-          n_eval += T[k] > 0.0f;
-          pend[k] += T[k] > 0.0f;
+          n_eval += (T[q].x > 0.0f) + (T[q].y > 0.0f);
+          pend[2 * q] += T[q].x > 0.0f;
+          pend[2 * q + 1] += T[q].y > 0.0f;
         }
-        if (e.alpha >= kAlphaMin) {  // false for stopped pixels (row offset +inf)
-          const float w = __fmul_rn(e.alpha, T[k]);
-          const float Tn = __fsub_rn(T[k], w);
-          if (Tn < kTMin) {
-            T[k] = -T[k];
-            off[k] = stopped_offset();
-            --nlive;
-          } else {
-            C0[k] = __fmaf_rn(col.z, w, C0[k]);
-            C1[k] = __fmaf_rn(col.w, w, C1[k]);
-            C2[k] = __fmaf_rn(blue, w, C2[k]);
-            if (kAux) {
-              X0[k] = __fmaf_rn(xa.x, w, X0[k]);
-              X1[k] = __fmaf_rn(xa.y, w, X1[k]);
-              X2[k] = __fmaf_rn(xa.z, w, X2[k]);
+        // false for stopped pixels (row offset +inf)
+        const bool v0 = al0 >= kAlphaMin, v1 = al1 >= kAlphaMin;
+        if (v0 || v1) {
+          float2 w = __fmul2_rn(make_float2(v0 ? al0 : 0.0f, v1 ? al1 : 0.0f), T[q]);
+          float2 Tn = __ffma2_rn(w, make_float2(-1.0f, -1.0f), T[q]);  // T - w
+          bool c0 = v0, c1 = v1;
+          if ((v0 && Tn.x < kTMin) || (v1 && Tn.y < kTMin)) {
+            if (v0 && Tn.x < kTMin) {
+              Tn.x = -T[q].x;
+              w.x = 0.0f;
+              off[q].x = stopped_offset();
+              --nlive;
+              c0 = false;
             }
-            T[k] = Tn;
-            if (kTrack) last[k] = pos0 + (uint32_t)j;
-            if (kStats) {
+            if (v1 && Tn.y < kTMin) {
+              Tn.y = -T[q].y;
+              w.y = 0.0f;
+              off[q].y = stopped_offset();
+              --nlive;
+              c1 = false;
+            }
+          }
+          C0[q] = __ffma2_rn(make_float2(col.z, col.z), w, C0[q]);
+          C1[q] = __ffma2_rn(make_float2(col.w, col.w), w, C1[q]);
+          C2[q] = __ffma2_rn(make_float2(blue, blue), w, C2[q]);
+          if (kAux) {
+            X0[q] = __ffma2_rn(make_float2(xa.x, xa.x), w, X0[q]);
+            // a flow may overflow to infinity and must not meet a zero weight
+            if (c0) {
+              X1[q].x = __fmaf_rn(xa.y, w.x, X1[q].x);
+              X2[q].x = __fmaf_rn(xa.z, w.x, X2[q].x);
+            }
+            if (c1) {
+              X1[q].y = __fmaf_rn(xa.y, w.y, X1[q].y);
+              X2[q].y = __fmaf_rn(xa.z, w.y, X2[q].y);
+            }
+          }
+          T[q] = Tn;
+          if (kTrack) {
+            if (c0) last[2 * q] = pos0 + (uint32_t)j;
+            if (c1) last[2 * q + 1] = pos0 + (uint32_t)j;
+          }
+          if (kStats) {
+            if (c0) {
               ++n_comp;
-              n_evb += pend[k];
-              pend[k] = 0u;
+              n_evb += pend[2 * q];
+              pend[2 * q] = 0u;
+            }
+            if (c1) {
+              ++n_comp;
+              n_evb += pend[2 * q + 1];
+              pend[2 * q + 1] = 0u;
             }
           }
         }
@@ -256,19 +305,20 @@ __global__ void __launch_bounds__(TILE *TILE / PPT, (fwd_min_blocks<TILE, PPT, k
   for (int k = 0; k < PPT; ++k) {
     if (!(px < V.width && py0 + k < V.height)) continue;
     const int64_t p = (int64_t)(py0 + k) * V.width + px;
-    const float Tend = fabsf(T[k]);
-    img[p] = C0[k] + Tend * A.bg0;
-    img[HW + p] = C1[k] + Tend * A.bg1;
-    img[2 * HW + p] = C2[k] + Tend * A.bg2;
+    auto lane = [k](const float2 *v) { return k & 1 ? v[k >> 1].y : v[k >> 1].x; };
+    const float Tend = fabsf(lane(T));
+    img[p] = lane(C0) + Tend * A.bg0;
+    img[HW + p] = lane(C1) + Tend * A.bg1;
+    img[2 * HW + p] = lane(C2) + Tend * A.bg2;
     A.pix_T[V.pix_base + p] = Tend;
     A.pix_last[V.pix_base + p] = kTrack ? last[k] : 0u;
     if (A.out_T) A.out_T[V.pix_base + p] = Tend;
     if (kAux) {
       float *aux = A.out_aux + V.pix_base * 4;
-      aux[p] = X0[k];
+      aux[p] = lane(X0);
       aux[HW + p] = 1.0f - Tend;
-      aux[2 * HW + p] = X1[k];
-      aux[3 * HW + p] = X2[k];
+      aux[2 * HW + p] = lane(X1);
+      aux[3 * HW + p] = lane(X2);
     }
   }
 }
