@@ -58,10 +58,20 @@ struct RenderBwdArgs {
 };
 
 // Pixels per thread of the compositor kernels (the autotuned block shape):
-// 16x16 tiles take 2, 4 (default) or 8, 8x8 tiles 1 or 2 (default).
-inline int render_ppt(const fgs4d_settings *s) {
+// 16x16 tiles take 2, 4 or 8, 8x8 tiles 1 or 2.  Defaults for 16x16 tiles by
+// the tile count: 4; with few tiles, whose lists too few warps would walk, 2;
+// with many the adjoint of the image, whose per-entry work (moments and
+// reduction rows) is shared by a strip, 8.  Measured forward / adjoint (us)
+// with 2, 4 and 8 rows a thread: 48 tiles 12.0 / 26.7, 18.5 / 39.2, 35.0 /
+// 63.5; 690 tiles 26.8 / 63.7, 38.9 / 84.0, 70.6 / 123; 1200 tiles 32.3 / 76.4,
+// 33.1 / 74.6, 59.1 / 107; 3978 tiles 54.5 / 155, 56.7 / 139, 77.5 / 146; 5440
+// tiles 190 / 581, 186 / 454, 267 / 442.
+constexpr int64_t kFewTiles = 1024, kManyTiles = 5000;
+inline int render_ppt(const fgs4d_settings *s, const Layout &L, bool adjoint) {
   if (s->tile == 8) return s->pixels_per_thread == 1 ? 1 : 2;
-  return (s->pixels_per_thread == 2 || s->pixels_per_thread == 8) ? s->pixels_per_thread : 4;
+  if (s->pixels_per_thread) return s->pixels_per_thread;
+  if (L.total_tiles < kFewTiles) return 2;
+  return adjoint && L.total_tiles >= kManyTiles ? 8 : 4;
 }
 
 
@@ -830,10 +840,10 @@ cudaError_t render_fwd_typed(const Layout &L, const fgs4d_settings *s, const fgs
   if (L.total_tiles == 0) return cudaSuccess;
   const unsigned grid = (unsigned)L.total_tiles;
   if (s->tile == 8) {
-    if (render_ppt(s) == 1) return launch_fwd_ppt<MAXV, 8, 1>(A, rv, grid, stats, s->shared_batch, image_only, st);
+    if (render_ppt(s, L, false) == 1) return launch_fwd_ppt<MAXV, 8, 1>(A, rv, grid, stats, s->shared_batch, image_only, st);
     return launch_fwd_ppt<MAXV, 8, 2>(A, rv, grid, stats, s->shared_batch, image_only, st);
   }
-  switch (render_ppt(s)) {
+  switch (render_ppt(s, L, false)) {
     case 2: return launch_fwd_ppt<MAXV, 16, 2>(A, rv, grid, stats, s->shared_batch, image_only, st);
     case 8: return launch_fwd_ppt<MAXV, 16, 8>(A, rv, grid, stats, s->shared_batch, image_only, st);
     default: return launch_fwd_ppt<MAXV, 16, 4>(A, rv, grid, stats, s->shared_batch, image_only, st);
@@ -883,10 +893,10 @@ cudaError_t render_bwd_typed(const Layout &L, const fgs4d_settings *s, const fgs
   if (L.total_tiles == 0) return cudaSuccess;
   const unsigned grid = (unsigned)L.total_tiles;
   if (s->tile == 8) {
-    if (render_ppt(s) == 1) return launch_bwd_ppt<MAXV, 8, 1>(A, rv, grid, s->shared_batch, st);
+    if (render_ppt(s, L, dL_daux == nullptr) == 1) return launch_bwd_ppt<MAXV, 8, 1>(A, rv, grid, s->shared_batch, st);
     return launch_bwd_ppt<MAXV, 8, 2>(A, rv, grid, s->shared_batch, st);
   }
-  switch (render_ppt(s)) {
+  switch (render_ppt(s, L, dL_daux == nullptr)) {
     case 2: return launch_bwd_ppt<MAXV, 16, 2>(A, rv, grid, s->shared_batch, st);
     case 8: return launch_bwd_ppt<MAXV, 16, 8>(A, rv, grid, s->shared_batch, st);
     default: return launch_bwd_ppt<MAXV, 16, 4>(A, rv, grid, s->shared_batch, st);
