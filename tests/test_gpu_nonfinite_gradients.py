@@ -44,3 +44,49 @@ def test_colour_gradients(tile, ppt, value):
         return torch.cat([grads[k].reshape(1500, -1) for k in PARAM_KEYS], 1).cpu().numpy()
 
     _check(run, value, 1e-4)
+
+
+@pytest.mark.parametrize("D,tile", [(8, 16), (16, 8), (32, 16)])
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+def test_feature_gradients(D, tile, value):
+    import torch
+    p, r = _case(tile, 0)
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    feats = torch.randn((1500, D), device="cuda", generator=gen)
+    gate = torch.rand((D,), device="cuda", generator=gen)
+    base = torch.randn(D * r.total_pixels, device="cuda", generator=gen)
+
+    def run(v, s):
+        r.forward_features(p, feats, gate)
+        d = base * s
+        d[3 * 72 * 96 + 37 * 96 + 51] = v  # component 3 of pixel (51, 37)
+        g = torch.zeros_like(feats)
+        r.backward_features(feats, gate, d, g)
+        return g.cpu().numpy()
+
+    _check(run, value, 1e-4)
+
+
+@pytest.mark.parametrize("D", [8, 16, 32])
+def test_feature_map_of_a_feature_that_is_not_finite(D):
+    """NaN in one Gaussian's feature reaches only the pixels that composite it,
+    and only its component."""
+    import torch
+    p, r = _case(16, 0)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    feats = torch.randn((1500, D), device="cuda", generator=gen)
+    ref = r.forward_features(p, feats).view(D, -1).cpu().numpy()
+    # a Gaussian that the view shows: the one with the largest gradient
+    grad = torch.zeros_like(feats)
+    r.backward_features(feats, None, torch.ones(D * r.total_pixels, device="cuda"), grad)
+    g = int(grad.abs().sum(1).argmax())
+    alone = torch.zeros_like(feats)
+    alone[g] = 1.0
+    hit = r.forward_features(p, alone).view(D, -1)[5].cpu().numpy() != 0  # the pixels that composite it
+    bad = feats.clone()
+    bad[g, 5] = float("nan")
+    got = r.forward_features(p, bad).view(D, -1).cpu().numpy()
+    assert hit.any()
+    np.testing.assert_array_equal(np.isnan(got[5]), hit)
+    assert np.isfinite(got[np.arange(D) != 5]).all()
+    np.testing.assert_array_equal(got[:, ~hit], ref[:, ~hit])
