@@ -857,9 +857,37 @@ struct SplitArgs {
   float *o_logit, *o_sh;
 };
 
+// out[c width + k] = in[src[c] width + k] for c < n, k < width (zero rows
+// where src[c] < 0).
+template <typename T>
+__device__ __forceinline__ void copy_rows(const T *__restrict__ in, T *__restrict__ out, const int32_t *src, int n,
+                                          uint32_t width, T zero) {
+  constexpr int kBatch = 6;
+  const uint32_t total = (uint32_t)n * width;
+  for (uint32_t i0 = threadIdx.x; i0 < total; i0 += kBatch * blockDim.x) {
+    T v[kBatch];
+#pragma unroll
+    for (int b = 0; b < kBatch; ++b) {
+      const uint32_t i = i0 + b * blockDim.x;
+      v[b] = zero;
+      if (i < total) {
+        const uint32_t c = i / width;
+        const int32_t s = src[c];
+        if (s >= 0) v[b] = in[(int64_t)s * width + (i - c * width)];
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < kBatch; ++b) {
+      const uint32_t i = i0 + b * blockDim.x;
+      if (i < total) out[i] = v[b];
+    }
+  }
+}
+
 // One thread per child for the draw; the children's SH rows (the bulk of
-// the bytes) are then copied by whole warps, consecutive lanes on
-// consecutive floats of a row.
+// the bytes) are then copied by the whole block.  Bound by those bytes (and,
+// at a few ten thousand children, by their latency): 60k children of 144
+// coefficients took 21 us with a warp per row, two loads in flight per lane.
 __global__ void __launch_bounds__(128) split_kernel(SplitArgs A) {
   grid_dependency_sync();
   __shared__ int32_t s_src[128];  // parent of each child of the block, -1: none
@@ -907,21 +935,13 @@ __global__ void __launch_bounds__(128) split_kernel(SplitArgs A) {
   s_src[threadIdx.x] = src;
   __syncthreads();
   const int nchild = (int)min64((int64_t)blockDim.x, total - c0);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-  // float4 copies when rows of both arrays start on 16-byte boundaries
+  // The block's child rows are consecutive in the output: its threads copy
+  // them as one array, kBatch independent loads each before the stores.
+  // float4 copies when rows of both arrays start on 16-byte boundaries.
   const bool vec = (A.k3 & 3) == 0 && ((reinterpret_cast<uintptr_t>(A.sh) | reinterpret_cast<uintptr_t>(A.o_sh)) & 15) == 0;
-  const int width = vec ? A.k3 >> 2 : A.k3;
-  for (int c = warp; c < nchild; c += nwarps) {
-    const int32_t i = s_src[c];
-    const int64_t orow = (c0 + c) * A.k3, irow = (int64_t)(i >= 0 ? i : 0) * A.k3;
-    for (int k = lane; k < width; k += 32) {
-      if (vec)
-        reinterpret_cast<float4 *>(A.o_sh + orow)[k] =
-            i >= 0 ? reinterpret_cast<const float4 *>(A.sh + irow)[k] : make_float4(0.f, 0.f, 0.f, 0.f);
-      else
-        A.o_sh[orow + k] = i >= 0 ? A.sh[irow + k] : 0.f;
-    }
-  }
+  if (vec) copy_rows(reinterpret_cast<const float4 *>(A.sh), reinterpret_cast<float4 *>(A.o_sh) + c0 * (A.k3 >> 2),
+                     s_src, nchild, (uint32_t)A.k3 >> 2, make_float4(0.f, 0.f, 0.f, 0.f));
+  else copy_rows(A.sh, A.o_sh + c0 * A.k3, s_src, nchild, (uint32_t)A.k3, 0.f);
 }
 
 }  // namespace
