@@ -129,6 +129,7 @@ int compute_layout(const fgs4d_settings *s, int64_t n, const fgs4d_view *views, 
   // emission when other work shares the GPU (stage_blocks_per_sm = k).
   const int k = s->stage_blocks_per_sm;
   L.pre_grid = k ? std::min(L.pre_blocks, 152 * k) : L.pre_blocks;
+  L.pre_compact_grid = 152 * (k ? 2 * k : 8);
   L.sort_grid = 152 * (k ? k : 4);
   const int64_t segs = (L.inst_cap + kCellSeg - 1) / kCellSeg;
   L.cell_grid = (int32_t)std::min<int64_t>(segs, 152 * (k ? 2 * k : 8));
@@ -173,6 +174,9 @@ int compute_layout(const fgs4d_settings *s, int64_t n, const fgs4d_view *views, 
     L.cell_slot = take(ic * 4);
     L.cell_mask = take(ic * 8);
   }
+  L.pre_stage = L.inst_key[0];
+  L.pre_staged = L.pre_blocks >= kPreStagedMinBlocks &&
+                 off - L.pre_stage >= (size_t)L.pre_blocks * (kPreBlock * kPreStageBytes + sizeof(uint32_t));
   L.tile_state = take((size_t)L.tile_passes * L.tile_blocks * kRadixBins * sizeof(uint32_t));
   if (L.cells) {
     L.cell_ranges = take((size_t)L.total_cells * 8);

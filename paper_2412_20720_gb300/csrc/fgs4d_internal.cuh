@@ -12,6 +12,11 @@ namespace fgs4d {
 constexpr int kTile = 16;           // default tile edge in pixels (8 is the other supported size)
 constexpr int kTilePixels = kTile * kTile;
 constexpr int kPreBlock = 256;      // threads per preprocess block
+constexpr int kPreStageBytes = 56;  // a staged record
+// Logical preprocess blocks from which the staged form is taken (when the
+// staging area fits): about as many as run at once, so that blocks wait for
+// one another.
+constexpr int kPreStagedMinBlocks = 608;
 constexpr int kEmitBlock = 256;     // threads per pair-scan / emission block
 constexpr int kEmitChunk = 2048;    // (slot, rect tile) pairs per emission chunk
 constexpr int kSortThreads = 256;   // threads per radix block
@@ -142,6 +147,11 @@ struct Layout {
   int32_t chunk_cap;      // emission chunks of kEmitChunk (two-level binning: kCellChunk) pairs
   int32_t emit_grid;      // persistent emission blocks
   int32_t pre_grid;       // persistent preprocess blocks
+  // Preprocess through a staging area (see preprocess_kernel): it lies over
+  // the instance buffers, which bin_sort fills afterwards.
+  bool pre_staged;
+  size_t pre_stage;
+  int32_t pre_compact_grid;
   int32_t sort_grid;      // persistent radix-pass blocks (at most; one radix tile each at least)
   bool cells;             // two-level binning (cells.cuh) instead of the instance sort
   int32_t total_cells, cell_passes;

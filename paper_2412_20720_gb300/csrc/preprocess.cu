@@ -20,6 +20,8 @@
 // oracle uses the plain formula).
 #include <math.h>
 
+#include <algorithm>
+
 #include "fgs4d_internal.cuh"
 
 namespace fgs4d {
@@ -41,6 +43,12 @@ struct PreArgs {
   float *rec_blue, *rec_tau;
   int4 *rec_meta;
   uint32_t *depth_key;
+  // Staged form: per logical block its visible count and kPreBlock places for
+  // its records.
+  uint32_t *stage_count;
+  float4 *stage_geom, *stage_color;
+  int4 *stage_misc;  // (blue, tau, depth, Gaussian)
+  int2 *stage_rect;
 };
 
 struct BwdArgs {
@@ -330,7 +338,21 @@ __device__ __forceinline__ bool forward_chain(int32_t i, const float4 *__restric
   return true;
 }
 
-template <int L, int MAXV>
+// Sets the visible total (clamped to the capacity) and its overflow flag.
+__device__ __forceinline__ void set_visible_total(const PreArgs &A, uint64_t all) {
+  A.counters[kCtrNeedVisible] = (uint32_t)umin64(all, 0xffffffffull);
+  A.counters[kCtrVisible] = (uint32_t)umin64(all, (uint64_t)A.vis_cap);
+  if (all > (uint64_t)A.vis_cap) atomicOr(&A.counters[kCtrStatus], kStatusVisOverflow);
+}
+
+// kStaged: every logical block leaves its records, compacted, at its own
+// places of the staging area together with their count, and
+// preprocess_compact_kernel moves them to their slots.  Otherwise the block
+// finds its first slot by a decoupled look-back, for which it (its registers
+// and its eight warps) waits until the slowest of the blocks before it has
+// counted: 40 % of the kernel's time when the blocks are many.  1M Gaussians,
+// 8 views (2.2M visible): 904 us with the look-back, 531 without it.
+template <int L, int MAXV, bool kStaged>
 __global__ void __launch_bounds__(kPreBlock) preprocess_kernel(PreArgs A, PreViews<MAXV> views) {
   grid_dependency_sync();
   __shared__ uint32_t s_ticket;
@@ -340,62 +362,128 @@ __global__ void __launch_bounds__(kPreBlock) preprocess_kernel(PreArgs A, PreVie
   // Persistent: logical blocks of kPreBlock (view, Gaussian) pairs are taken
   // by ticket, so a logical block's look-back only waits on logical blocks
   // that running blocks hold.
-  while (true) {
-  if (threadIdx.x == 0) s_ticket = atomicAdd(&A.counters[kCtrTicketPre], 1u);
-  __syncthreads();
-  const int32_t w = (int32_t)s_ticket;
-  if (w >= nlogical) break;
-  const int32_t view = MAXV == 1 ? 0 : w / A.blocks_per_view;
-  const int32_t gb = MAXV == 1 ? w : w % A.blocks_per_view;
-  const int32_t i = gb * kPreBlock + (int32_t)threadIdx.x;
-  const PreView &cam = views.v[view];
-
-  Chain h;
-  // Compact-4DGS mask (Sec. 4.3): M_hat = 1{sigmoid(m) > eps} in value, so a
-  // Gaussian is either removed (zero scales and opacity) or unchanged.
-  bool kept = i < A.n;
-  if (kept && A.mask_logit) {
-    const float mk = A.mask_logit[i];
-    kept = isfinite(mk) && 1.0f / (1.0f + expf(-mk)) > A.mask_threshold;
-  }
-  const bool vis = kept && forward_chain<L>(i, A.mean, A.log_scale, A.q_l, A.q_r, A.logit, A.sh, A.t_order, A.k3,
-                                            A.period_inv, A.near_plane, A.dilation, A.p_t_min, cam, h);
-  uint32_t total;
-  const uint32_t local = block_exclusive_scan(vis ? 1u : 0u, s_scan, &total);
-  if (threadIdx.x < 32) {
-    const uint64_t prefix = lookback_u64_warp(A.lb, w, total, &A.counters[kCtrStatus]);
-    if (threadIdx.x == 0) s_base = prefix;
-    if (threadIdx.x == 0 && w == nlogical - 1) {
-      const uint64_t all = prefix + total;
-      A.counters[kCtrNeedVisible] = (uint32_t)umin64(all, 0xffffffffull);
-      A.counters[kCtrVisible] = (uint32_t)umin64(all, (uint64_t)A.vis_cap);
-      if (all > (uint64_t)A.vis_cap) atomicOr(&A.counters[kCtrStatus], kStatusVisOverflow);
+  for (int32_t w = blockIdx.x;; w += gridDim.x) {
+    if (!kStaged) {
+      if (threadIdx.x == 0) s_ticket = atomicAdd(&A.counters[kCtrTicketPre], 1u);
+      __syncthreads();
+      w = (int32_t)s_ticket;
     }
+    if (w >= nlogical) break;
+    const int32_t view = MAXV == 1 ? 0 : w / A.blocks_per_view;
+    const int32_t gb = MAXV == 1 ? w : w % A.blocks_per_view;
+    const int32_t i = gb * kPreBlock + (int32_t)threadIdx.x;
+    const PreView &cam = views.v[view];
+
+    Chain h;
+    // Compact-4DGS mask (Sec. 4.3): M_hat = 1{sigmoid(m) > eps} in value, so a
+    // Gaussian is either removed (zero scales and opacity) or unchanged.
+    bool kept = i < A.n;
+    if (kept && A.mask_logit) {
+      const float mk = A.mask_logit[i];
+      kept = isfinite(mk) && 1.0f / (1.0f + expf(-mk)) > A.mask_threshold;
+    }
+    const bool vis = kept && forward_chain<L>(i, A.mean, A.log_scale, A.q_l, A.q_r, A.logit, A.sh, A.t_order, A.k3,
+                                              A.period_inv, A.near_plane, A.dilation, A.p_t_min, cam, h);
+    uint32_t total;
+    const uint32_t local = block_exclusive_scan(vis ? 1u : 0u, s_scan, &total);
+    if (kStaged) {
+      if (threadIdx.x == 0) A.stage_count[w] = total;
+    } else {
+      if (threadIdx.x < 32) {
+        const uint64_t prefix = lookback_u64_warp(A.lb, w, total, &A.counters[kCtrStatus]);
+        if (threadIdx.x == 0) s_base = prefix;
+        if (threadIdx.x == 0 && w == nlogical - 1) set_visible_total(A, prefix + total);
+      }
+      __syncthreads();
+    }
+    const uint64_t slot = kStaged ? (uint64_t)w * kPreBlock + local : s_base + local;
+    if (vis && (kStaged || slot < (uint64_t)A.vis_cap)) {
+      // The exponent in base 2, q = (1/2) log2(e) d^T Sigma_2d^-1 d, as a sum of
+      // two squares: Sigma_2d^-1 = U U^T with U upper triangular gives
+      // q = (a1 dx)^2 + (b1 dx + b2 dy)^2, a1 = sqrt(k / Sa), b1 = -Sb sqrt(k /
+      // (Sa det)), b2 = Sa sqrt(k / (Sa det)), k = log2(e) / 2.  Evaluated this
+      // way q has no cancellation (the expanded conic form loses precision along
+      // the long axis of an elongated footprint, in proportion to its condition
+      // number); det is the Cauchy-Binet sum of squares.
+      const float kq = 0.5f * kLog2e;
+      const float a1 = sqrtf(kq / h.Sa);
+      const float rs = sqrtf(kq / (h.Sa * h.det));
+      // alpha = a 2^power2 >= 1/255 needs -power2 <= log2(255 a); the margin
+      // keeps the per-tile test of the instance emission conservative under
+      // rounding.
+      const float tau = log2f(255.0f * h.a) + kTauMargin;
+      const float4 geom = make_float4(h.uv[0], h.uv[1], a1, -h.Sb * rs);
+      const float4 color = make_float4(h.Sa * rs, log2f(h.a), h.rgb[0], h.rgb[1]);
+      const int2 rect = make_int2(h.rect[0] | (h.rect[1] << 16), h.rect[2] | (h.rect[3] << 16));
+      if (kStaged) {
+        A.stage_geom[slot] = geom;
+        A.stage_color[slot] = color;
+        A.stage_misc[slot] = make_int4(__float_as_int(h.rgb[2]), __float_as_int(tau), __float_as_int(h.pc[2]), i);
+        A.stage_rect[slot] = rect;
+      } else {
+        A.rec_geom[slot] = geom;
+        A.rec_color[slot] = color;
+        A.rec_blue[slot] = h.rgb[2];
+        A.rec_tau[slot] = tau;
+        A.rec_meta[slot] = make_int4(i, view, rect.x, rect.y);
+        A.depth_key[slot] = __float_as_uint(h.pc[2]);
+      }
+    }
+    if (!kStaged) __syncthreads();  // s_ticket and s_base are reused by the next logical block
   }
-  __syncthreads();
-  const uint64_t slot = s_base + local;
-  if (vis && slot < (uint64_t)A.vis_cap) {
-    // The exponent in base 2, q = (1/2) log2(e) d^T Sigma_2d^-1 d, as a sum of
-    // two squares: Sigma_2d^-1 = U U^T with U upper triangular gives
-    // q = (a1 dx)^2 + (b1 dx + b2 dy)^2, a1 = sqrt(k / Sa), b1 = -Sb sqrt(k /
-    // (Sa det)), b2 = Sa sqrt(k / (Sa det)), k = log2(e) / 2.  Evaluated this
-    // way q has no cancellation (the expanded conic form loses precision along
-    // the long axis of an elongated footprint, in proportion to its condition
-    // number); det is the Cauchy-Binet sum of squares.
-    const float kq = 0.5f * kLog2e;
-    const float a1 = sqrtf(kq / h.Sa);
-    const float rs = sqrtf(kq / (h.Sa * h.det));
-    A.rec_geom[slot] = make_float4(h.uv[0], h.uv[1], a1, -h.Sb * rs);
-    A.rec_color[slot] = make_float4(h.Sa * rs, log2f(h.a), h.rgb[0], h.rgb[1]);
-    A.rec_blue[slot] = h.rgb[2];
-    // alpha = a 2^power2 >= 1/255 needs -power2 <= log2(255 a); the margin
-    // keeps the per-tile test of the instance emission conservative under
-    // rounding.
-    A.rec_tau[slot] = log2f(255.0f * h.a) + kTauMargin;
-    A.rec_meta[slot] = make_int4(i, view, h.rect[0] | (h.rect[1] << 16), h.rect[2] | (h.rect[3] << 16));
-    A.depth_key[slot] = __float_as_uint(h.pc[2]);
-  }
-  __syncthreads();  // s_ticket and s_base are reused by the next logical block
+}
+
+// Moves the staged records to their slots, one warp per logical block: the
+// block's counts are scanned, its first slot comes from a decoupled look-back
+// over blocks of kCompactWarps counts (short: nothing but the counts is
+// loaded before it), and consecutive lanes copy consecutive records.
+constexpr int kCompactWarps = 8;
+static_assert(kCompactWarps * 32 == kPreBlock, "look-back words: one per logical block is enough");
+
+__global__ void __launch_bounds__(kCompactWarps * 32) preprocess_compact_kernel(PreArgs A) {
+  grid_dependency_sync();
+  __shared__ uint32_t s_ticket;
+  __shared__ uint64_t s_first[kCompactWarps];
+  const int32_t nlogical = A.nviews * A.blocks_per_view;
+  const int32_t ngroups = (nlogical + kCompactWarps - 1) / kCompactWarps;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  while (true) {
+    if (threadIdx.x == 0) s_ticket = atomicAdd(&A.counters[kCtrTicketPre], 1u);
+    __syncthreads();
+    const int32_t g = (int32_t)s_ticket;
+    if (g >= ngroups) break;
+    const int32_t w = g * kCompactWarps + warp;
+    const uint32_t count = w < nlogical ? min(A.stage_count[w], (uint32_t)kPreBlock) : 0u;
+    if (warp == 0) {
+      const int32_t wl = g * kCompactWarps + lane;
+      const uint32_t c = lane < kCompactWarps && wl < nlogical ? A.stage_count[wl] : 0u;
+      uint32_t inc = c;
+#pragma unroll
+      for (int o = 1; o < kCompactWarps; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+      }
+      const uint32_t total = __shfl_sync(0xffffffffu, inc, kCompactWarps - 1);
+      const uint64_t prefix = lookback_u64_warp(A.lb, g, total, &A.counters[kCtrStatus]);
+      if (lane < kCompactWarps) s_first[lane] = prefix + inc - c;
+      if (lane == 0 && g == ngroups - 1) set_visible_total(A, prefix + total);
+    }
+    __syncthreads();
+    const int32_t view = w / max(A.blocks_per_view, 1);
+    for (uint32_t k = lane; k < count; k += 32) {
+      const uint64_t slot = s_first[warp] + k, from = (uint64_t)w * kPreBlock + k;
+      if (slot < (uint64_t)A.vis_cap) {
+        const int4 misc = A.stage_misc[from];
+        const int2 rect = A.stage_rect[from];
+        A.rec_geom[slot] = A.stage_geom[from];
+        A.rec_color[slot] = A.stage_color[from];
+        A.rec_blue[slot] = __int_as_float(misc.x);
+        A.rec_tau[slot] = __int_as_float(misc.y);
+        A.rec_meta[slot] = make_int4(misc.w, view, rect.x, rect.y);
+        A.depth_key[slot] = (uint32_t)misc.z;
+      }
+    }
+    __syncthreads();  // s_ticket and s_first are reused by the next group
   }
 }
 
@@ -740,7 +828,20 @@ cudaError_t launch_pre_typed(const PreLaunch &p, const fgs4d_view *views, int32_
   A.rec_meta = reinterpret_cast<int4 *>(p.ws + Lo.rec_meta);
   A.depth_key = reinterpret_cast<uint32_t *>(p.ws + Lo.depth_key);
   if (Lo.pre_blocks == 0) return cudaSuccess;
-  return launch_pdl(preprocess_kernel<L, MAXV>, (unsigned)Lo.pre_grid, kPreBlock, p.stream, A, pv);
+  if (!Lo.pre_staged)
+    return launch_pdl(preprocess_kernel<L, MAXV, false>, (unsigned)Lo.pre_grid, kPreBlock, p.stream, A, pv);
+  const size_t places = (size_t)Lo.pre_blocks * kPreBlock;
+  unsigned char *st = p.ws + Lo.pre_stage;
+  A.stage_geom = reinterpret_cast<float4 *>(st);
+  A.stage_color = reinterpret_cast<float4 *>(st + 16 * places);
+  A.stage_misc = reinterpret_cast<int4 *>(st + 32 * places);
+  A.stage_rect = reinterpret_cast<int2 *>(st + 48 * places);
+  A.stage_count = reinterpret_cast<uint32_t *>(st + 56 * places);
+  cudaError_t e = launch_pdl(preprocess_kernel<L, MAXV, true>, (unsigned)Lo.pre_grid, kPreBlock, p.stream, A, pv);
+  if (e != cudaSuccess) return e;
+  const int groups = (Lo.pre_blocks + kCompactWarps - 1) / kCompactWarps;
+  return launch_pdl(preprocess_compact_kernel, (unsigned)std::min(groups, Lo.pre_compact_grid),
+                    (unsigned)(kCompactWarps * 32), p.stream, A);
 }
 
 template <int L, int MAXV>

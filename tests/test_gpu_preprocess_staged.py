@@ -1,0 +1,36 @@
+"""Preprocess through the staging area (many logical blocks, large instance
+buffers) against the look-back form (small instance buffers): the same slots,
+records and counts bit for bit."""
+import numpy as np
+import pytest
+
+from paper_2412_20720_gb300 import fgs4d
+from paper_2412_20720_gb300 import synthetic as sy
+from paper_2412_20720_gb300.render import RenderConfig, Renderer
+from helpers import to_device
+
+pytestmark = pytest.mark.gpu
+
+
+# 608 logical blocks of 256 (the smallest count staged), a ragged last block,
+# several views, lean grids; a visible capacity below the need
+@pytest.mark.parametrize("n,nviews,stage_blocks,vis_cap", [
+    (155_393, 1, 0, 0), (155_648, 1, 1, 0), (60_001, 3, 0, 0), (60_001, 3, 2, 0), (200_000, 1, 0, 20_000)])
+def test_same_records_as_with_the_look_back(n, nviews, stage_blocks, vis_cap):
+    import torch
+    params = to_device(sy.make_scene(n, 31, (-2, -2, -2), (2, 2, 2), sh_degree=1, t_order=1).as_dict())
+    views = [sy.tiny_view(400, 300, t=0.2 + 0.3 * k) for k in range(nviews)]
+    got = []
+    for inst_cap in (1 << 22, 1000):
+        r = Renderer(n, views, RenderConfig(sh_degree=1, t_order=1, inst_capacity=inst_cap, vis_capacity=vis_cap,
+                                            stage_blocks_per_sm=stage_blocks))
+        fgs4d.preprocess(r.gaussians(params), r.views, r.nviews, r.settings, r.ws.data_ptr(), r.ws_bytes, r.stream())
+        code, counts = r.status()
+        assert code == (fgs4d.ERR_CAPACITY if vis_cap else fgs4d.OK)
+        v, L = counts[0], r.layout
+        got.append([np.array(counts)] + [r.workspace_view(off, torch.int32, k * v).cpu().numpy()
+                                         for off, k in ((L.rec_geom, 4), (L.rec_color, 4), (L.rec_blue, 1), (L.rec_tau, 1),
+                                                        (L.rec_meta, 4), (L.depth_key, 1))])
+    assert got[0][0][0] > 10_000
+    for a, b in zip(*got):
+        np.testing.assert_array_equal(a, b)
