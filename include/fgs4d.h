@@ -368,6 +368,12 @@ typedef struct {
 int fgs4d_adam_update_set(const fgs4d_adam_tensor *tensors, int32_t ntensors, float beta1, float beta2, float eps,
                           const int32_t *step, int32_t zero_grad, void *stream);
 
+/* Clears ntensors float arrays (tensors[k], counts[k] elements) in one launch:
+ * the zeroed gradients a backward pass accumulates into.  Errors:
+ * FGS4D_ERR_ARG: ntensors outside [0, FGS4D_ADAM_MAX_TENSORS], a NULL table, a
+ * negative count, a NULL or misaligned (16 bytes) array of count > 0. */
+int fgs4d_zero_set(float *const *tensors, const int64_t *counts, int32_t ntensors, void *stream);
+
 /* Scale-gated feature rendering for 4D segmentation (Sec. 7, "Scale-gated
  * features"): Gaussian i carries features[i][0..D); at a scale s the caller
  * passes the gate vector S(s) (device float [D], values in [0, 1]; NULL =

@@ -513,6 +513,13 @@ int fgs4d_adam_update_set(const fgs4d_adam_tensor *tensors, int32_t ntensors, fl
                                      static_cast<cudaStream_t>(stream)));
 }
 
+int fgs4d_zero_set(float *const *tensors, const int64_t *counts, int32_t ntensors, void *stream) {
+  if (ntensors < 0 || ntensors > FGS4D_ADAM_MAX_TENSORS || (ntensors > 0 && (!tensors || !counts))) return FGS4D_ERR_ARG;
+  for (int32_t k = 0; k < ntensors; ++k)
+    if (counts[k] < 0 || (counts[k] > 0 && (!tensors[k] || !aligned16(tensors[k])))) return FGS4D_ERR_ARG;
+  return cuda_status(launch_zero_set(tensors, counts, ntensors, static_cast<cudaStream_t>(stream)));
+}
+
 int fgs4d_mask_loss(const float *mask_logit, int64_t n, float *loss_out, float *grad_out, void *stream) {
   if (n < 0 || (n > 0 && (!mask_logit || !loss_out || !grad_out))) return FGS4D_ERR_ARG;
   return cuda_status(launch_mask_loss(mask_logit, n, loss_out, grad_out, static_cast<cudaStream_t>(stream)));

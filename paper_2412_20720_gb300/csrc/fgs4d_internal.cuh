@@ -501,6 +501,7 @@ struct AdamTensorDev {
 };
 cudaError_t launch_adam_set(const AdamTensorDev *tensors, int32_t n, float b1, float b2, float eps,
                             const int32_t *step, bool zero_grad, cudaStream_t stream);
+cudaError_t launch_zero_set(float *const *tensors, const int64_t *counts, int32_t n, cudaStream_t stream);
 cudaError_t launch_mask_loss(const float *mask_logit, int64_t n, float *loss, float *grad, cudaStream_t stream);
 cudaError_t launch_aux_records(const PreLaunch &p, const fgs4d_view *views, int32_t nviews, float flow_dt);
 cudaError_t launch_split(const fgs4d_gaussians *src, const int32_t *idx, int64_t m, int32_t k_children,

@@ -771,6 +771,29 @@ __global__ void adam_set_kernel(AdamSetArgs A) {
   }
 }
 
+// Clears a set of tensors in one launch (units as in adam_set_kernel): six
+// fills of a small model's gradients took six launches of the host's time.
+struct ZeroSetArgs {
+  float *p[kAdamMaxTensors];
+  int64_t count[kAdamMaxTensors], first[kAdamMaxTensors + 1];
+  int32_t n;
+};
+
+__global__ void zero_set_kernel(ZeroSetArgs A) {
+  grid_dependency_sync();
+  const int64_t total = A.first[A.n], stride = (int64_t)gridDim.x * blockDim.x;
+  int k = 0;
+  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < total; u += stride) {
+    while (u >= A.first[k + 1]) ++k;  // units only grow along the loop
+    const int64_t i = 4 * (u - A.first[k]);
+    if (i + 4 <= A.count[k]) {
+      *reinterpret_cast<float4 *>(A.p[k] + i) = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {
+      for (int64_t e = i; e < A.count[k]; ++e) A.p[k][e] = 0.f;
+    }
+  }
+}
+
 __global__ void adam_tick_kernel(int32_t *step) {
   grid_dependency_sync();
   if (threadIdx.x == 0) *step += 1;
@@ -946,6 +969,19 @@ cudaError_t launch_adam_set(const AdamTensorDev *tensors, int32_t n, float b1, f
   if (total == 0) return cudaSuccess;
   const int blocks = (int)std::min<int64_t>((total + 255) / 256, 152 * 8);
   return launch_pdl(adam_set_kernel, (unsigned)blocks, 256u, stream, A);
+}
+
+cudaError_t launch_zero_set(float *const *tensors, const int64_t *counts, int32_t n, cudaStream_t stream) {
+  ZeroSetArgs A{};
+  A.n = n;
+  for (int32_t k = 0; k < n; ++k) {
+    A.p[k] = tensors[k];
+    A.count[k] = counts[k];
+    A.first[k + 1] = A.first[k] + (counts[k] + 3) / 4;
+  }
+  if (A.first[n] == 0) return cudaSuccess;
+  const int blocks = (int)std::min<int64_t>((A.first[n] + 255) / 256, 152 * 8);
+  return launch_pdl(zero_set_kernel, (unsigned)blocks, 256u, stream, A);
 }
 
 cudaError_t launch_adam_tick(int32_t *step, cudaStream_t stream) {

@@ -33,7 +33,7 @@ EXPORTED = ("fgs4d_workspace_size", "fgs4d_workspace_layout", "fgs4d_preprocess"
             "fgs4d_render_stats", "fgs4d_render_bwd", "fgs4d_render_bwd_composite",
             "fgs4d_render_bwd_preprocess", "fgs4d_render_aux_bwd", "fgs4d_split_gaussians",
             "fgs4d_mask_loss", "fgs4d_adam_tick", "fgs4d_adam_update", "fgs4d_adam_update_set",
-            "fgs4d_render_features",
+            "fgs4d_zero_set", "fgs4d_render_features",
             "fgs4d_render_features_bwd", "fgs4d_l1_loss", "fgs4d_l1_loss_part", "fgs4d_sort_depth_static",
             "fgs4d_sort_depth_static_status", "fgs4d_wait_selftest", "fgs4d_get_status", "fgs4d_status_string")
 STATIC_SORT_MAX = 1 << 20
@@ -135,6 +135,7 @@ def load():
     lib.fgs4d_adam_tick.argtypes = [vp, vp]
     lib.fgs4d_adam_update.argtypes = [vp, vp, vp, vp, i64, C.c_float, C.c_float, C.c_float, C.c_float, vp, vp]
     lib.fgs4d_adam_update_set.argtypes = [P(AdamTensor), i32, C.c_float, C.c_float, C.c_float, vp, i32, vp]
+    lib.fgs4d_zero_set.argtypes = [P(vp), P(i64), i32, vp]
     lib.fgs4d_l1_loss.argtypes = [vp, vp, i64, vp, vp, vp]
     lib.fgs4d_l1_loss_part.argtypes = [vp, vp, i64, i64, vp, vp, vp]
     lib.fgs4d_sort_depth_static.argtypes = [vp, i64, vp, vp]
@@ -327,6 +328,14 @@ def adam_update_set(tensors, beta1: float, beta2: float, eps: float, step: int, 
         arr[k] = AdamTensor(p, g, m, v, int(count), float(lr))
     _check(load().fgs4d_adam_update_set(arr, len(tensors), float(beta1), float(beta2), float(eps), step,
                                         1 if zero_grad else 0, stream), "fgs4d_adam_update_set")
+
+
+def zero_set(tensors, stream: int):
+    """tensors: sequence of (device pointer, float count) to clear in one launch."""
+    n = len(tensors)
+    ptrs = (C.c_void_p * max(1, n))(*(p for p, _ in tensors))
+    counts = (C.c_int64 * max(1, n))(*(int(c) for _, c in tensors))
+    _check(load().fgs4d_zero_set(ptrs, counts, n, stream), "fgs4d_zero_set")
 
 
 def l1_loss(img: int, target: int, count: int, loss_out: int, dL_dimg: int, stream: int):

@@ -512,7 +512,8 @@ class Render4DGS(torch.autograd.Function):
     def backward(ctx, grad_out):
         saved = ctx.saved_tensors
         params = dict(zip(PARAM_KEYS, saved))
-        grads = {k: torch.zeros_like(v) for k, v in params.items()}
+        grads = {k: torch.empty_like(v) for k, v in params.items()}
+        fgs4d.zero_set([(_ptr(g), g.numel()) for g in grads.values()], ctx.renderer.stream())
         ctx.renderer.backward(params, grad_out, grads)
         return (None,) + tuple(grads[k] for k in PARAM_KEYS)
 
