@@ -134,7 +134,9 @@ int compute_layout(const fgs4d_settings *s, int64_t n, const fgs4d_view *views, 
   const int64_t segs = (L.inst_cap + kCellSeg - 1) / kCellSeg;
   L.cell_grid = (int32_t)std::min<int64_t>(segs, 152 * (k ? 2 * k : 8));
   L.emit_grid = std::max(1, std::min(L.chunk_cap, 152 * (k ? 2 * k : 8)));
-  L.depth_blocks = (int32_t)((L.vis_cap + kDepthSortTile - 1) / kDepthSortTile);
+  L.depth_items = L.vis_cap >= kDepthSortLargeMin ? kDepthSortItemsLarge : kDepthSortItems;
+  const int64_t depth_tile = (int64_t)kSortThreads * L.depth_items;
+  L.depth_blocks = (int32_t)((L.vis_cap + depth_tile - 1) / depth_tile);
   L.tile_blocks = (int32_t)((L.inst_cap + kInstSortTile - 1) / kInstSortTile);
 
   size_t off = 0;

@@ -22,8 +22,10 @@ constexpr int kEmitChunk = 2048;    // (slot, rect tile) pairs per emission chun
 constexpr int kSortThreads = 256;   // threads per radix block
 constexpr int kSortItems = 8;       // keys per thread per radix block (instance sort)
 constexpr int kSortTile = kSortThreads * kSortItems;
-constexpr int kDepthSortItems = 4;  // keys per thread per radix block of the depth sort
-constexpr int kDepthSortTile = kSortThreads * kDepthSortItems;
+// Keys per thread per radix block of the depth sort: 4, so that 80k keys
+// occupy more SMs, or 8 (half the look-backs) from this capacity on.
+constexpr int kDepthSortItems = 4, kDepthSortItemsLarge = 8;
+constexpr int64_t kDepthSortLargeMin = int64_t(1) << 20;
 constexpr int kInstSortItems = 8;   // keys per thread per radix block of the instance (tile-id) sort
 constexpr int kInstSortTile = kSortThreads * kInstSortItems;
 // Two-level binning (cells.cuh).
@@ -39,6 +41,10 @@ constexpr int kCellPrefixThreads = 512;
 // cells (8 views, 1.9M) 168 / 194; 48,000 over 352 cells (8-pixel tiles) 91 /
 // 120; the 6-view street call (5.4M over 810 cells, 685M) 20,900 / 4,100.
 constexpr int64_t kCellsMinVisible = 65536, kCellsMinPerCell = 1024;
+// Instance capacity from which cell_write takes its form for dense masks:
+// bin_sort 4425 -> 4140 us at 741M instances (with the depth sort's larger
+// tickets), 110 -> 116 us at 1.7M.
+constexpr int64_t kCellDenseMinCap = int64_t(1) << 26;
 // Visible slots up to which the depth sort ranks by counting.
 constexpr int64_t kRankSortMax = 8192;
 constexpr int64_t kPairScanWideMin = int64_t(1) << 19;
@@ -156,6 +162,7 @@ struct Layout {
   bool cells;             // two-level binning (cells.cuh) instead of the instance sort
   int32_t total_cells, cell_passes;
   int32_t cell_grid;      // persistent count / write blocks
+  int32_t depth_items;    // keys per thread of the depth sort's blocks
   int32_t depth_blocks, tile_blocks;
   int32_t depth_passes, tile_passes;
   int32_t tile_bits;

@@ -842,7 +842,40 @@ cudaError_t bin_cells(const Layout &L, const EmitArgs &ea_in, const RasterViews<
   if (e != cudaSuccess) return e;
   e = launch_pdl(cell_prefix_kernel<MAXV>, (unsigned)std::min(L.total_cells, 152 * 8), kCellPrefixThreads, st, C, rv);
   if (e != cudaSuccess) return e;
-  return launch_pdl(cell_write_kernel<MAXV>, (unsigned)L.cell_grid, kCellBlock, st, C, rv);
+  return launch_pdl(L.inst_cap >= kCellDenseMinCap ? cell_write_kernel<MAXV, true> : cell_write_kernel<MAXV, false>,
+                    (unsigned)L.cell_grid, kCellBlock, st, C, rv);
+}
+
+// Depth sort of the visible slots (31 key bits: depth > near > 0); the
+// per-slot keys stay intact, the passes ping-pong between two buffers.
+template <int kItems>
+cudaError_t depth_sort(const Layout &L, unsigned char *ws, uint32_t *sorted, cudaStream_t st) {
+  uint32_t *ctr = reinterpret_cast<uint32_t *>(ws + L.counters);
+  const uint32_t *dkey = reinterpret_cast<const uint32_t *>(ws + L.depth_key);
+  uint32_t *dk[2] = {reinterpret_cast<uint32_t *>(ws + L.dsort_key[0]), reinterpret_cast<uint32_t *>(ws + L.dsort_key[1])};
+  uint32_t *dv[2] = {reinterpret_cast<uint32_t *>(ws + L.dsort_val[0]), reinterpret_cast<uint32_t *>(ws + L.dsort_val[1])};
+  uint32_t *dstate = reinterpret_cast<uint32_t *>(ws + L.depth_state);
+  uint32_t *hist = reinterpret_cast<uint32_t *>(ws + L.hist_depth);
+  const int pb = std::min(L.depth_blocks, L.sort_grid);
+  // the first pass ranks few keys 32 at a time: blocks beyond its own for those
+  const int pb0 = std::max(pb, (int)std::min<int64_t>((std::min(L.vis_cap, kRankSortMax) + 31) / 32, 152));
+  constexpr size_t smem = radix_smem_bytes<kItems>();
+  cudaError_t e = launch_pdl(radix_hist_kernel<kItems>, (unsigned)pb, kSortThreads, st, dkey,
+                             (const uint32_t *)(ctr + kCtrVisible), (int64_t)L.vis_cap, (int32_t)L.depth_passes, hist,
+                             dstate, (int32_t)L.depth_blocks, (uint2 *)nullptr, (int64_t)0, kRankSortMax);
+  if (e != cudaSuccess) return e;
+  for (int p = 0; p < L.depth_passes; ++p) {
+    const int out = p & 1, in = out ^ 1;
+    e = launch_pdl_smem(p == 0 ? radix_pass_kernel<true, kItems> : radix_pass_kernel<false, kItems>,
+                        (unsigned)(p == 0 ? pb0 : pb), kSortThreads, smem, st, p == 0 ? dkey : (const uint32_t *)dk[in],
+                        p == 0 ? (const uint32_t *)nullptr : (const uint32_t *)dv[in], dk[out], dv[out],
+                        (const uint32_t *)(ctr + kCtrVisible), (int64_t)L.vis_cap, (int32_t)(kRadixBits * p),
+                        (const uint32_t *)(hist + p * kRadixBins), dstate + (size_t)p * L.depth_blocks * kRadixBins,
+                        ctr + kCtrTicketDepth + p, ctr + kCtrStatus, (uint2 *)nullptr, (int64_t)0, kRankSortMax,
+                        p == 0 ? sorted : (uint32_t *)nullptr);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 template <int MAXV>
@@ -854,14 +887,8 @@ cudaError_t bin_sort_typed(const Layout &L, const fgs4d_view *views, int32_t nvi
   uint32_t *status = ctr + kCtrStatus;
   cudaError_t e = cudaMemsetAsync(ws + kSortControlStart, 0, L.control_end - kSortControlStart, st);
   if (e != cudaSuccess) return e;
-  // 1. Depth sort of the visible slots (31 key bits: depth > near > 0); the
-  // per-slot keys stay intact, the passes ping-pong between two buffers.
-  const uint32_t *dkey = reinterpret_cast<const uint32_t *>(ws + L.depth_key);
-  uint32_t *dk[2] = {reinterpret_cast<uint32_t *>(ws + L.dsort_key[0]), reinterpret_cast<uint32_t *>(ws + L.dsort_key[1])};
-  uint32_t *dv[2] = {reinterpret_cast<uint32_t *>(ws + L.dsort_val[0]), reinterpret_cast<uint32_t *>(ws + L.dsort_val[1])};
-  uint32_t *dstate = reinterpret_cast<uint32_t *>(ws + L.depth_state);
-  uint32_t *hist_d = reinterpret_cast<uint32_t *>(ws + L.hist_depth);
-  uint32_t *sorted = dv[(L.depth_passes - 1) & 1];
+  // 1. Depth sort of the visible slots.
+  uint32_t *sorted = reinterpret_cast<uint32_t *>(ws + L.dsort_val[(L.depth_passes - 1) & 1]);
   uint32_t *tstate = reinterpret_cast<uint32_t *>(ws + L.tile_state);
   uint32_t *hist_t = reinterpret_cast<uint32_t *>(ws + L.hist_tile);
   uint2 *ranges = reinterpret_cast<uint2 *>(ws + L.ranges);
@@ -896,28 +923,9 @@ cudaError_t bin_sort_typed(const Layout &L, const fgs4d_view *views, int32_t nvi
     if (e != cudaSuccess) return e;
   } else {
     if (L.depth_blocks > 0) {
-      const int hb = std::min(L.depth_blocks, L.sort_grid);
-      const int pb = std::min(L.depth_blocks, L.sort_grid);
-      // the first pass ranks few keys 32 at a time: blocks beyond its own for those
-      const int pb0 = std::max(pb, (int)std::min<int64_t>((std::min(L.vis_cap, kRankSortMax) + 31) / 32, 152));
-      constexpr size_t smem = radix_smem_bytes<kDepthSortItems>();
-      e = launch_pdl(radix_hist_kernel<kDepthSortItems>, (unsigned)hb, kSortThreads, st, dkey,
-                     (const uint32_t *)(ctr + kCtrVisible), (int64_t)L.vis_cap, (int32_t)L.depth_passes, hist_d,
-                     dstate, (int32_t)L.depth_blocks, (uint2 *)nullptr, (int64_t)0, kRankSortMax);
+      e = L.depth_items == kDepthSortItems ? depth_sort<kDepthSortItems>(L, ws, sorted, st)
+                                           : depth_sort<kDepthSortItemsLarge>(L, ws, sorted, st);
       if (e != cudaSuccess) return e;
-      for (int p = 0; p < L.depth_passes; ++p) {
-        const int out = p & 1, in = out ^ 1;
-        uint32_t *state = dstate + (size_t)p * L.depth_blocks * kRadixBins;
-        const uint32_t *kin = p == 0 ? dkey : dk[in];
-        const uint32_t *vin = p == 0 ? nullptr : dv[in];
-        e = launch_pdl_smem(p == 0 ? radix_pass_kernel<true, kDepthSortItems>
-                                   : radix_pass_kernel<false, kDepthSortItems>,
-                            (unsigned)(p == 0 ? pb0 : pb), kSortThreads, smem, st, kin, vin, dk[out], dv[out],
-                       (const uint32_t *)(ctr + kCtrVisible), (int64_t)L.vis_cap, (int32_t)(kRadixBits * p),
-                       (const uint32_t *)(hist_d + p * kRadixBins), state, ctr + kCtrTicketDepth + p, status,
-                       (uint2 *)nullptr, (int64_t)0, kRankSortMax, p == 0 ? sorted : (uint32_t *)nullptr);
-        if (e != cudaSuccess) return e;
-      }
     }
     // 2. Instances in depth order.
     if (L.cells) return bin_cells<MAXV>(L, ea, rv, ws, st);
