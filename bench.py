@@ -415,8 +415,9 @@ def run_ours(args, rank, world, local):
     st = stream.cuda_stream
     npx = W_IMG * H_IMG
     imgs = [torch.empty(3 * npx, dtype=torch.float32, device=dev) for _ in range(pipe.depth)]
-    # preprocess; bin_sort (as the library reports it); render.
-    launches_per_frame = 1 + fgs4d.bin_sort_kernels(scene.n, vv[0][0], vv[0][1], s) + 1
+    # preprocess and bin_sort (as the library reports them); render.
+    launches_per_frame = (fgs4d.preprocess_kernels(scene.n, vv[0][0], vv[0][1], s)
+                          + fgs4d.bin_sort_kernels(scene.n, vv[0][0], vv[0][1], s) + 1)
 
     # Capacity and work counts over the whole sweep (outside the timed region).
     stats = torch.zeros(3, dtype=torch.int64, device=dev)  # fgs4d_render_stats adds three counters

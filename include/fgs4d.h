@@ -207,6 +207,13 @@ int fgs4d_preprocess(const fgs4d_gaussians *gaussians, const fgs4d_view *views, 
 int fgs4d_bin_sort(int64_t n, const fgs4d_view *views, int32_t nviews, const fgs4d_settings *settings,
                    void *workspace, size_t workspace_bytes, void *stream);
 
+/* Diagnostic: *count_out = the number of kernels fgs4d_preprocess launches for
+ * these arguments (two where the records pass through a staging area, which
+ * lies over the instance buffers that fgs4d_bin_sort fills afterwards).
+ * Launches nothing; has no counterpart in the paper. */
+int fgs4d_preprocess_kernels(int64_t n, const fgs4d_view *views, int32_t nviews, const fgs4d_settings *settings,
+                             int32_t *count_out);
+
 /* Diagnostic: *count_out = the number of kernels fgs4d_bin_sort launches for
  * these arguments (the count depends on the tile grid's size, which sets the
  * number of tile-sort passes).  Launches nothing; has no counterpart in the

@@ -155,6 +155,7 @@ int compute_layout(const fgs4d_settings *s, int64_t n, const fgs4d_view *views, 
   L.pair_prefix = take(((size_t)L.vis_cap + 1) * sizeof(uint32_t));
   L.emit_rec = take((size_t)L.vis_cap * 48);
   L.rec_aux = take((size_t)L.vis_cap * sizeof(float4));
+  L.block_first = take((size_t)L.pre_blocks * sizeof(uint32_t));
   L.chunk_first = take((size_t)L.chunk_cap * sizeof(uint32_t));
   const size_t vc = (size_t)L.vis_cap, ic = (size_t)L.inst_cap;
   L.rec_geom = take(vc * 16);
@@ -265,6 +266,16 @@ int fgs4d_bin_sort(int64_t n, const fgs4d_view *views, int32_t nviews, const fgs
   if (rc) return rc;
   return cuda_status(launch_bin_sort(L, views, nviews, static_cast<unsigned char *>(workspace),
                                      static_cast<cudaStream_t>(stream)));
+}
+
+int fgs4d_preprocess_kernels(int64_t n, const fgs4d_view *views, int32_t nviews, const fgs4d_settings *settings,
+                             int32_t *count_out) {
+  if (!count_out) return FGS4D_ERR_ARG;
+  Layout L;
+  const int rc = compute_layout(settings, n, views, nviews, &L);
+  if (rc) return rc;
+  *count_out = L.pre_blocks == 0 ? 0 : (L.pre_staged ? 2 : 1);
+  return FGS4D_OK;
 }
 
 int fgs4d_bin_sort_kernels(int64_t n, const fgs4d_view *views, int32_t nviews, const fgs4d_settings *settings,

@@ -127,6 +127,7 @@ struct Layout {
   size_t pair_prefix;   // uint32 [vis_cap + 1]: exclusive prefix of rect areas in depth order
   size_t emit_rec;      // 3 x 16 B [vis_cap]: emission record per depth-sorted position
   size_t rec_aux;       // float4 [vis_cap]: (camera depth, flow_u, flow_v, 0) per slot (auxiliary render)
+  size_t block_first;   // uint32 [pre_blocks]: first slot of each logical preprocess block
   size_t chunk_first;   // uint32 [chunk_cap]: depth-sorted position holding each chunk's first pair
   size_t control_end;
   size_t rec_geom, rec_color, rec_blue, rec_tau, rec_meta;

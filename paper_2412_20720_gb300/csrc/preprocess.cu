@@ -43,6 +43,7 @@ struct PreArgs {
   float *rec_blue, *rec_tau;
   int4 *rec_meta;
   uint32_t *depth_key;
+  uint32_t *block_first;  // first slot of each logical block
   // Staged form: per logical block its visible count and kPreBlock places for
   // its records.
   uint32_t *stage_count;
@@ -61,6 +62,11 @@ struct BwdArgs {
   int64_t vis_cap;
   const uint32_t *counters;
   const int4 *rec_meta;
+  const float4 *rec_color;
+  const float *rec_blue;
+  int32_t blocks_per_view;
+  bool grouped;  // blocks take groups of logical blocks, views fastest
+  const uint32_t *block_first;
   const float4 *slot_grad;
   float4 *g_mean, *g_log_scale, *g_q_l, *g_q_r;
   float *g_logit, *g_sh;
@@ -174,7 +180,9 @@ struct Chain {
   float a;
 };
 
-template <int L>
+// kColour false: without the SH sum (h.raw, h.rgb unset); the caller knows the
+// slot's colour to be finite.
+template <int L, bool kColour = true>
 __device__ __forceinline__ bool forward_chain(int32_t i, const float4 *__restrict__ mean,
                                               const float4 *__restrict__ log_scale, const float4 *__restrict__ q_l,
                                               const float4 *__restrict__ q_r, const float *__restrict__ logit,
@@ -303,6 +311,7 @@ __device__ __forceinline__ bool forward_chain(int32_t i, const float4 *__restric
     h.cn[nn] = h.cn[nn - 1] * c1 - h.sn[nn - 1] * s1;
     h.sn[nn] = h.sn[nn - 1] * c1 + h.cn[nn - 1] * s1;
   }
+  if (!kColour) return true;
   float acc[3] = {0.f, 0.f, 0.f};
   const float *shg = sh + (size_t)i * k3;
 #pragma unroll
@@ -369,8 +378,12 @@ __global__ void __launch_bounds__(kPreBlock) preprocess_kernel(PreArgs A, PreVie
       w = (int32_t)s_ticket;
     }
     if (w >= nlogical) break;
-    const int32_t view = MAXV == 1 ? 0 : w / A.blocks_per_view;
-    const int32_t gb = MAXV == 1 ? w : w % A.blocks_per_view;
+    // Staged blocks wait for no other, so they run view by view over the same
+    // Gaussians: a Gaussian's SH row then comes from L2 for all views but the
+    // first.
+    const int32_t view = MAXV == 1 ? 0 : (kStaged ? w % A.nviews : w / A.blocks_per_view);
+    const int32_t gb = MAXV == 1 ? w : (kStaged ? w / A.nviews : w % A.blocks_per_view);
+    const int32_t lw = view * A.blocks_per_view + gb;  // logical block: (view, Gaussian) order
     const int32_t i = gb * kPreBlock + (int32_t)threadIdx.x;
     const PreView &cam = views.v[view];
 
@@ -387,16 +400,17 @@ __global__ void __launch_bounds__(kPreBlock) preprocess_kernel(PreArgs A, PreVie
     uint32_t total;
     const uint32_t local = block_exclusive_scan(vis ? 1u : 0u, s_scan, &total);
     if (kStaged) {
-      if (threadIdx.x == 0) A.stage_count[w] = total;
+      if (threadIdx.x == 0) A.stage_count[lw] = total;
     } else {
       if (threadIdx.x < 32) {
         const uint64_t prefix = lookback_u64_warp(A.lb, w, total, &A.counters[kCtrStatus]);
         if (threadIdx.x == 0) s_base = prefix;
+        if (threadIdx.x == 0) A.block_first[w] = (uint32_t)umin64(prefix, (uint64_t)A.vis_cap);
         if (threadIdx.x == 0 && w == nlogical - 1) set_visible_total(A, prefix + total);
       }
       __syncthreads();
     }
-    const uint64_t slot = kStaged ? (uint64_t)w * kPreBlock + local : s_base + local;
+    const uint64_t slot = kStaged ? (uint64_t)lw * kPreBlock + local : s_base + local;
     if (vis && (kStaged || slot < (uint64_t)A.vis_cap)) {
       // The exponent in base 2, q = (1/2) log2(e) d^T Sigma_2d^-1 d, as a sum of
       // two squares: Sigma_2d^-1 = U U^T with U upper triangular gives
@@ -466,6 +480,7 @@ __global__ void __launch_bounds__(kCompactWarps * 32) preprocess_compact_kernel(
       const uint32_t total = __shfl_sync(0xffffffffu, inc, kCompactWarps - 1);
       const uint64_t prefix = lookback_u64_warp(A.lb, g, total, &A.counters[kCtrStatus]);
       if (lane < kCompactWarps) s_first[lane] = prefix + inc - c;
+      if (lane < kCompactWarps && wl < nlogical) A.block_first[wl] = (uint32_t)umin64(prefix + inc - c, (uint64_t)A.vis_cap);
       if (lane == 0 && g == ngroups - 1) set_visible_total(A, prefix + total);
     }
     __syncthreads();
@@ -499,9 +514,8 @@ __device__ __forceinline__ void red_add4(float4 *p, float x, float y, float z, f
 // between consecutive frames).  mu_xyz|t moves with velocity
 // Sigma_{1:3,4} / Sigma_44 = (B u) / sqrt(Sigma_44) in the factored form, so the
 // displaced camera-space centre is pc + W v flow_dt; the flow is 0 when that
-// point is not in front of the near plane.  The chain is re-run with the
-// colour basis cut to degree 0 (the slot is known to be visible; only its
-// geometry is used).
+// point is not in front of the near plane.  The chain is re-run without the
+// colour (the slot is known to be visible; only its geometry is used).
 struct AuxArgs {
   const float4 *mean, *log_scale, *q_l, *q_r;
   const float *logit, *sh;
@@ -523,7 +537,7 @@ __global__ void __launch_bounds__(128) aux_records_kernel(AuxArgs A, PreViews<MA
   const PreView &cam = views.v[MAXV == 1 ? 0 : meta.y];
   Chain h;
   float4 out = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (forward_chain<0>(meta.x, A.mean, A.log_scale, A.q_l, A.q_r, A.logit, A.sh, A.t_order, A.k3, A.period_inv,
+  if (forward_chain<0, false>(meta.x, A.mean, A.log_scale, A.q_l, A.q_r, A.logit, A.sh, A.t_order, A.k3, A.period_inv,
                        A.near_plane, A.dilation, A.p_t_min, cam, h)) {
     const float k = A.flow_dt / h.sqc;  // velocity = B u / sqrt(Sigma_44)
     const float d0 = h.Bu[0] * k, d1 = h.Bu[1] * k, d2 = h.Bu[2] * k;
@@ -539,24 +553,21 @@ __global__ void __launch_bounds__(128) aux_records_kernel(AuxArgs A, PreViews<MA
   A.rec_aux[slot] = out;
 }
 
+// Adjoint of one slot.
 template <int L, int MAXV>
-__global__ void __launch_bounds__(128) preprocess_bwd_kernel(BwdArgs A, PreViews<MAXV> views) {
-  grid_dependency_sync();
-  const int64_t nvis = min64((int64_t)A.counters[kCtrVisible], A.vis_cap);
-  const int64_t slot = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (slot >= nvis) return;
+__device__ __forceinline__ void slot_adjoint(const BwdArgs &A, const PreViews<MAXV> &views, int64_t slot) {
   const int4 meta = A.rec_meta[slot];
   const int32_t i = meta.x, view = meta.y;
   if (i < 0 || i >= A.n || view < 0 || view >= A.nviews) return;  // only after a recorded timeout
-  const PreView &cam = views.v[view];
-  Chain h;
-  if (!forward_chain<L>(i, A.mean, A.log_scale, A.q_l, A.q_r, A.logit, A.sh, A.t_order, A.k3, A.period_inv,
-                        A.near_plane, A.dilation, A.p_t_min, cam, h))
-    return;  // cannot happen for a slot the forward produced with the same inputs
+  const PreView &cam = views.v[MAXV == 1 ? 0 : view];
   const float4 g0 = A.slot_grad[3 * slot + 0];  // du, dv, dA, dB
   const float4 g1 = A.slot_grad[3 * slot + 1];  // dC, da, dr, dg
   const float4 g2 = A.slot_grad[3 * slot + 2];  // db, dz
   const float gu = g0.x, gv = g0.y, gA = g0.z, gB = g0.w, gC = g1.x, ga = g1.y;
+  // The colour's clamp is open where the record's colour is above 0: the SH
+  // row is read once, for the gradient, and not for the colour again.
+  const float4 col = A.rec_color[slot];
+  const bool open[3] = {col.z > 0.0f, col.w > 0.0f, A.rec_blue[slot] > 0.0f};
   const float grgb[3] = {g1.z, g1.w, g2.x};
 
   float g_mu[3] = {0.f, 0.f, 0.f}, g_dt = 0.f;
@@ -564,15 +575,18 @@ __global__ void __launch_bounds__(128) preprocess_bwd_kernel(BwdArgs A, PreViews
   constexpr int NLM = (L + 1) * (L + 1);
   float graw[3];
 #pragma unroll
-  for (int ch = 0; ch < 3; ++ch) graw[ch] = (h.raw[ch] + 0.5f > 0.0f) ? grgb[ch] : 0.0f;
-  float Y[NLM], gY[NLM];
-  sh_basis<L>(h.dir[0], h.dir[1], h.dir[2], Y);
-#pragma unroll
-  for (int k = 0; k < NLM; ++k) gY[k] = 0.f;
+  for (int ch = 0; ch < 3; ++ch) graw[ch] = open[ch] ? grgb[ch] : 0.0f;
   const float *shg = A.sh + (size_t)i * A.k3;
   float *gsh = A.g_sh + (size_t)i * A.k3;
   const bool any_col = graw[0] != 0.f || graw[1] != 0.f || graw[2] != 0.f;
   if (any_col) {
+    Chain h;  // the sliced mean and the view direction (the rest is dropped by the compiler)
+    (void)forward_chain<L, false>(i, A.mean, A.log_scale, A.q_l, A.q_r, A.logit, A.sh, A.t_order, A.k3, A.period_inv,
+                                  A.near_plane, A.dilation, A.p_t_min, cam, h);
+    float Y[NLM], gY[NLM];
+    sh_basis<L>(h.dir[0], h.dir[1], h.dir[2], Y);
+#pragma unroll
+    for (int k = 0; k < NLM; ++k) gY[k] = 0.f;
 #pragma unroll
     for (int nn = 0; nn <= FGS4D_MAX_T_ORDER; ++nn) {
       if (nn > A.t_order) break;
@@ -615,6 +629,14 @@ __global__ void __launch_bounds__(128) preprocess_bwd_kernel(BwdArgs A, PreViews
 #pragma unroll
     for (int x = 0; x < 3; ++x) g_mu[x] += (gdir[x] - h.dir[x] * dd) * irw;
   }
+  // ---- geometry.  The chain is evaluated again behind an opaque index: kept
+  // from the colour above, its 80 values would be live through the SH row.
+  int32_t ig = i;
+  asm volatile("" : "+r"(ig));
+  Chain h;
+  if (!forward_chain<L, false>(ig, A.mean, A.log_scale, A.q_l, A.q_r, A.logit, A.sh, A.t_order, A.k3, A.period_inv,
+                               A.near_plane, A.dilation, A.p_t_min, cam, h))
+    return;  // cannot happen for a slot the forward produced with the same inputs
   // ---- opacity a = sigmoid(logit) p_t.
   const float g_sig = ga * h.pt;
   float g_pt = ga * h.sig;
@@ -765,6 +787,30 @@ __global__ void __launch_bounds__(128) preprocess_bwd_kernel(BwdArgs A, PreViews
            (gqr[3] - s * dr) * ir);
 }
 
+constexpr int64_t kBwdGroupedMinBytes = int64_t(96) << 20;
+constexpr int kBwdGroup = 4;  // logical blocks whose slots one block takes (about 290 of 1024 at 28 % visible)
+
+template <int L, int MAXV>
+__global__ void __launch_bounds__(128, 4) preprocess_bwd_kernel(BwdArgs A, PreViews<MAXV> views) {
+  grid_dependency_sync();
+  const int64_t nvis = min64((int64_t)A.counters[kCtrVisible], A.vis_cap);
+  if (MAXV == 1 || !A.grouped) {
+    const int64_t slot = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (slot < nvis) slot_adjoint<L, MAXV>(A, views, slot);
+    return;
+  }
+  // Block (group of kBwdGroup logical blocks, view), views fastest: the slots
+  // of one view for a range of Gaussians are consecutive, and the views'
+  // adjoints of one range run together, so that the SH rows and their
+  // gradients stay in L2 from view to view.
+  const int32_t view = blockIdx.x % A.nviews, g0 = blockIdx.x / A.nviews * kBwdGroup;
+  const int32_t w0 = view * A.blocks_per_view + g0;
+  const int32_t w1 = view * A.blocks_per_view + min(g0 + kBwdGroup, A.blocks_per_view);
+  const int64_t s0 = min64(A.block_first[w0], nvis);
+  const int64_t s1 = w1 < A.nviews * A.blocks_per_view ? min64(A.block_first[w1], nvis) : nvis;
+  for (int64_t slot = s0 + threadIdx.x; slot < s1; slot += blockDim.x) slot_adjoint<L, MAXV>(A, views, slot);
+}
+
 template <int MAXV>
 bool fill_pre_views(const fgs4d_view *views, int32_t nviews, int32_t tile, PreViews<MAXV> *pv) {
   if (nviews > MAXV) return false;
@@ -827,6 +873,7 @@ cudaError_t launch_pre_typed(const PreLaunch &p, const fgs4d_view *views, int32_
   A.rec_tau = reinterpret_cast<float *>(p.ws + Lo.rec_tau);
   A.rec_meta = reinterpret_cast<int4 *>(p.ws + Lo.rec_meta);
   A.depth_key = reinterpret_cast<uint32_t *>(p.ws + Lo.depth_key);
+  A.block_first = reinterpret_cast<uint32_t *>(p.ws + Lo.block_first);
   if (Lo.pre_blocks == 0) return cudaSuccess;
   if (!Lo.pre_staged)
     return launch_pdl(preprocess_kernel<L, MAXV, false>, (unsigned)Lo.pre_grid, kPreBlock, p.stream, A, pv);
@@ -868,6 +915,8 @@ cudaError_t launch_bwd_typed(const PreLaunch &p, const fgs4d_view *views, int32_
   A.vis_cap = Lo.vis_cap;
   A.counters = reinterpret_cast<const uint32_t *>(p.ws + Lo.counters);
   A.rec_meta = reinterpret_cast<const int4 *>(p.ws + Lo.rec_meta);
+  A.rec_color = reinterpret_cast<const float4 *>(p.ws + Lo.rec_color);
+  A.rec_blue = reinterpret_cast<const float *>(p.ws + Lo.rec_blue);
   A.slot_grad = reinterpret_cast<const float4 *>(p.ws + Lo.slot_grad);
   A.g_mean = reinterpret_cast<float4 *>(gr->mean);
   A.g_log_scale = reinterpret_cast<float4 *>(gr->log_scale);
@@ -878,7 +927,13 @@ cudaError_t launch_bwd_typed(const PreLaunch &p, const fgs4d_view *views, int32_
   A.mask_logit = p.g->mask_logit;
   A.g_mask = gr->mask_logit;
   A.densify_stats = reinterpret_cast<float4 *>(gr->densify_stats);
-  const int64_t blocks = (Lo.vis_cap + 127) / 128;
+  A.blocks_per_view = Lo.pre_blocks_per_view;
+  A.block_first = reinterpret_cast<const uint32_t *>(p.ws + Lo.block_first);
+  // Several views whose SH rows and gradients do not fit L2 together (129 MB)
+  // take the grouped order; otherwise slots in their own order fill the blocks.
+  A.grouped = MAXV > 1 && p.g->n * A.k3 * (int64_t)(2 * sizeof(float)) > kBwdGroupedMinBytes;
+  const int64_t blocks = A.grouped ? (int64_t)((Lo.pre_blocks_per_view + kBwdGroup - 1) / kBwdGroup) * nviews
+                                   : (Lo.vis_cap + 127) / 128;
   if (blocks == 0) return cudaSuccess;
   return launch_pdl(preprocess_bwd_kernel<L, MAXV>, (unsigned)blocks, 128u, p.stream, A, pv);
 }
