@@ -68,6 +68,136 @@ struct FeatArgs {
   float *g_gate;      // backward: [D] or null
 };
 
+constexpr int kScalarPPT = 2;
+
+// Stages entry `k` of the batch: geometry, opacity and normalised gated
+// feature (rows padded to D + 1 floats against bank conflicts).
+template <int D>
+__device__ __forceinline__ void stage_feature(const FeatArgs &A, const float *s_gate, uint32_t idx, int k,
+                                              float4 *s_geom, float2 *s_ca, float *s_fhat) {
+  const uint32_t s = A.inst_val[idx];
+  float4 geom = make_float4(0.f, 0.f, 0.f, 0.f);
+  float2 ca = make_float2(0.f, kLogAlphaNone);  // (b2, log2 a): every pixel skips the entry
+  int32_t gi = -1;
+  if (s < A.vis_cap) {
+    geom = A.rec_geom[s];
+    const float4 c = A.rec_color[s];
+    ca = make_float2(c.x, c.y);
+    gi = A.rec_meta[s].x;
+    if (gi < 0 || (int64_t)gi >= A.n) {
+      gi = -1;
+      ca.y = kLogAlphaNone;
+    }
+  }
+  s_geom[k] = geom;
+  s_ca[k] = ca;
+  float g[D];
+  float nn = 0.f;
+  if (gi >= 0) {
+    const float4 *row = reinterpret_cast<const float4 *>(A.feat + (int64_t)gi * D);
+#pragma unroll
+    for (int c4 = 0; c4 < D / 4; ++c4) {
+      const float4 v = row[c4];
+      g[4 * c4 + 0] = v.x;
+      g[4 * c4 + 1] = v.y;
+      g[4 * c4 + 2] = v.z;
+      g[4 * c4 + 3] = v.w;
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < D; ++c) g[c] = 0.f;
+  }
+#pragma unroll
+  for (int c = 0; c < D; ++c) {
+    g[c] *= s_gate[c];
+    nn += g[c] * g[c];
+  }
+  const float norm = sqrtf(nn);
+  const float inv = norm > 0.f ? 1.0f / norm : 0.f;
+#pragma unroll
+  for (int c = 0; c < D; ++c) s_fhat[k * (D + 1) + c] = g[c] * inv;
+}
+
+// Feature map with a multiply-add per component, pixel and entry, a thread on a
+// vertical pair of pixels.  For D <= 16 it beats the matrix form below, whose
+// weights cost a thread per pixel: 300k Gaussians at 1352x1014 (us, this /
+// matrix form) D = 8 331 / 409, D = 16 486 / 488, D = 32 900 / 717; a street
+// view of 14 entries a tile D = 16 44 / 63.
+template <int MAXV, int TILE, int D>
+__global__ void __launch_bounds__(TILE *TILE / kScalarPPT)
+    render_features_scalar_kernel(FeatArgs A, RasterViews<MAXV> rv) {
+  grid_dependency_sync();
+  constexpr int kBatch = TILE * TILE / kScalarPPT;
+  __shared__ float4 s_geom[kBatch];
+  __shared__ float2 s_ca[kBatch];
+  __shared__ float s_fhat[kBatch * (D + 1)];
+  __shared__ float s_gate[D];
+  const int32_t gt = blockIdx.x;
+  const RasterView &V = rv.v[find_view<MAXV>(rv, gt)];
+  const int32_t lt = gt - V.tile_base;
+  const int32_t tx = lt % V.gw, ty = lt / V.gw;
+  const int32_t px = tx * TILE + (threadIdx.x & (TILE - 1));
+  const int32_t py0 = ty * TILE + (threadIdx.x / TILE) * kScalarPPT;
+  const uint2 range = tile_range(A.ranges, gt);
+  const float pxc = (float)px + 0.5f;
+  if (threadIdx.x < D) s_gate[threadIdx.x] = A.gate ? A.gate[threadIdx.x] : 1.0f;
+  static_assert(kScalarPPT <= 4, "a strip inside one row group");
+  const float gyc = row_group_centre(py0);
+  float T[kScalarPPT], off[kScalarPPT], F[kScalarPPT][D];
+  bool live = false;
+#pragma unroll
+  for (int k = 0; k < kScalarPPT; ++k) {
+    const bool in = px < V.width && py0 + k < V.height;
+    T[k] = in ? 1.0f : -1.0f;
+    off[k] = in ? row_offset(py0 + k) : stopped_offset();
+#pragma unroll
+    for (int c = 0; c < D; ++c) F[k][c] = 0.f;
+    live = live || in;
+  }
+  for (uint32_t base = range.x; base < range.y; base += kBatch) {
+    if (__syncthreads_count(live) == 0) break;
+    if (base + threadIdx.x < range.y)
+      stage_feature<D>(A, s_gate, base + threadIdx.x, threadIdx.x, s_geom, s_ca, s_fhat);
+    __syncthreads();
+    const int nb = (int)min(range.y - base, (uint32_t)kBatch);
+    for (int j = 0; j < nb && live; ++j) {
+      const float4 geom = s_geom[j];
+      const float2 ca = s_ca[j];
+      const ColumnTerms ct = column_terms(geom, pxc, ca.y);
+      const float w4 = group_w(ct, geom.y, ca.x, gyc);
+      const bool clamp = entry_clamps(ca.y);
+#pragma unroll
+      for (int k = 0; k < kScalarPPT; ++k) {
+        const AlphaEval e = pixel_alpha(ct, w4, ca.x, off[k], clamp);
+        if (e.alpha >= kAlphaMin) {  // false for stopped pixels (row offset +inf)
+          const float w = __fmul_rn(e.alpha, T[k]);
+          const float Tn = __fsub_rn(T[k], w);
+          if (Tn < kTMin) {
+            T[k] = -T[k];
+            off[k] = stopped_offset();
+          } else {
+#pragma unroll
+            for (int c = 0; c < D; ++c) F[k][c] = __fmaf_rn(s_fhat[j * (D + 1) + c], w, F[k][c]);
+            T[k] = Tn;
+          }
+        }
+      }
+      live = false;
+#pragma unroll
+      for (int k = 0; k < kScalarPPT; ++k) live = live || T[k] > 0.0f;
+    }
+  }
+  const int64_t HW = (int64_t)V.width * V.height;
+  float *out = A.out + V.pix_base * D;
+#pragma unroll
+  for (int k = 0; k < kScalarPPT; ++k) {
+    if (!(px < V.width && py0 + k < V.height)) continue;
+    const int64_t p = (int64_t)(py0 + k) * V.width + px;
+#pragma unroll
+    for (int c = 0; c < D; ++c) out[c * HW + p] = F[k][c];
+  }
+}
+
 __device__ __forceinline__ float tf32_round(float x) {
   uint32_t r;
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
@@ -339,29 +469,33 @@ __global__ void __launch_bounds__(feat_threads<TILE>()) render_features_bwd_kern
   }
   if (threadIdx.x < 2) s_poison[threadIdx.x] = s_has[threadIdx.x] = 0u;
   // Upstream gradients as operands: pixel 8 ks + lane % 4 (+ 4) of the warp,
-  // component 8 n + lane / 4.  A value that is not finite becomes 0 and marks
-  // its pixel.
-  const int64_t HW = (int64_t)V.width * V.height;
+  // component 8 n + lane / 4, from coalesced loads (lane = pixel) through the
+  // warp's buffer.  A value that is not finite becomes 0 and marks its pixel.
+  const int64_t HW = (int64_t)V.width * V.height, pixel = (int64_t)py * V.width + px;
   const float *dF = A.dL_dF + V.pix_base * D;
   uint32_t Gh[4][kN][2], Gl[4][kN][2];
-  uint32_t bad_pixels = 0u;  // of the warp
+  float up[D];  // all in flight before the first is used
 #pragma unroll
-  for (int ks = 0; ks < 4; ++ks)
+  for (int c = 0; c < D; ++c) up[c] = in ? dF[c * HW + pixel] : 0.f;
+  bool bad = false;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int q = 32 * warp + 8 * ks + lc + 4 * h;  // pixel of the tile
-      const int32_t x = tx0 + (q & (TILE - 1)), y = ty0 + q / TILE;
+  for (int n = 0; n < kN; ++n) {
+    __syncwarp();
 #pragma unroll
-      for (int n = 0; n < kN; ++n) {
-        float v = x < V.width && y < V.height ? dF[(8 * n + lr) * HW + (int64_t)y * V.width + x] : 0.f;
-        if (!isfinite(v)) {
-          bad_pixels |= 1u << (8 * ks + lc + 4 * h);
-          v = 0.f;
-        }
-        tf32_split(v, &Gh[ks][n][h], &Gl[ks][n][h]);
-      }
+    for (int c = 0; c < 8; ++c) {
+      const bool ok = isfinite(up[8 * n + c]);
+      bad = bad || !ok;
+      s_buf[warp][c * kWBwd + lane] = ok ? up[8 * n + c] : 0.f;
     }
-  bad_pixels = __reduce_or_sync(0xffffffffu, bad_pixels);
+    __syncwarp();
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        tf32_split(s_buf[warp][lr * kWBwd + 8 * ks + lc + 4 * h], &Gh[ks][n][h], &Gl[ks][n][h]);
+  }
+  const uint32_t bad_pixels = __ballot_sync(0xffffffffu, bad);  // of the warp
+  __syncwarp();
   FeatPixel P(px, py, in);
   float ggate = 0.f;  // of component lane % D
   int buf = 0;
@@ -385,7 +519,7 @@ __global__ void __launch_bounds__(feat_threads<TILE>()) render_features_bwd_kern
           w[j * kWBwd + lane] = x;
         }
         if (bad_pixels) {
-          const uint32_t e = __reduce_or_sync(0xffffffffu, (bad_pixels >> lane) & 1u ? hit : 0u);
+          const uint32_t e = __reduce_or_sync(0xffffffffu, bad ? hit : 0u);
           if (lane == 0 && e) atomicOr(&s_poison[buf], e);
         }
         some = __any_sync(0xffffffffu, hit != 0u);
@@ -463,7 +597,10 @@ cudaError_t launch_feat_tile(const FeatArgs &A, const RasterViews<MAXV> &rv, uns
   constexpr unsigned NT = feat_threads<TILE>();
   if (backward)
     return launch_pdl(render_features_bwd_kernel<MAXV, TILE, D>, grid, NT, st, A, rv);
-  return launch_pdl(render_features_kernel<MAXV, TILE, D>, grid, NT, st, A, rv);
+  if constexpr (D <= 16)
+    return launch_pdl(render_features_scalar_kernel<MAXV, TILE, D>, grid, (unsigned)(TILE * TILE / kScalarPPT), st, A, rv);
+  else
+    return launch_pdl(render_features_kernel<MAXV, TILE, D>, grid, NT, st, A, rv);
 }
 
 template <int MAXV, int D>
