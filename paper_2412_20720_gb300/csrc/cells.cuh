@@ -416,15 +416,16 @@ __global__ void __launch_bounds__(kCellPrefixThreads) cell_prefix_kernel(CellArg
 // the set bits of its words, from the tile's offset in the run plus the counts
 // of the warps before -- and then written, consecutive threads on consecutive
 // staged bits, to each tile's place in the instance list (the tile's start
-// plus the cell's earlier runs).  kDense: words with many bits set are walked
-// bit by bit without a search, about 8 instructions a step for both words
-// against 10 a set bit of the fullest lane (street call of 685M instances: see
-// kCellDenseMinCap); the unrolled walk costs registers, so that smaller calls
-// take the other form.
-template <int MAXV, bool kDense>
-__global__ void __launch_bounds__(kCellBlock) cell_write_kernel(CellArgs C, RasterViews<MAXV> rv) {
+// plus the cell's earlier runs).  The explicit minimum of one resident block
+// lets the compiler take more registers than its own choice: bin_sort (us)
+// without / with it 725 / 664 at 2.3M visible slots and 15M instances (8
+// views), 112 / 112 at 94k and 1.7M.  Walking words of many set bits by an
+// unrolled loop over all 32 gave 4165 us without the minimum and 4219 with it
+// at 741M instances; the plain walk with the minimum 4018.
+template <int MAXV>
+__global__ void __launch_bounds__(kCellBlock, 1) cell_write_kernel(CellArgs C, RasterViews<MAXV> rv) {
   grid_dependency_sync();
-  constexpr int kWarps = kCellBlock / 32, kDenseBits = 32;
+  constexpr int kWarps = kCellBlock / 32;
   static_assert(kCellSeg <= 256, "a pair's place in its segment fits a byte");
   __shared__ uint32_t s_key[kCellSeg], s_slot[kCellSeg];
   __shared__ uint16_t s_cnt[kWarps][kCellTiles];  // then: the warp's first staged position of the tile
@@ -492,16 +493,8 @@ __global__ void __launch_bounds__(kCellBlock) cell_write_kernel(CellArgs C, Rast
       // (tile, pair) of this lane's first pair in each word
       const uint32_t v0 = (uint32_t)((lane << 8) | (32 * warp)), v1 = v0 + (32u << 8);
       uint32_t p0 = s_cnt[warp][lane], p1 = s_cnt[warp][32 + lane];
-      if (kDense && __any_sync(0xffffffffu, __popc(w[0]) + __popc(w[1]) > kDenseBits)) {
-#pragma unroll
-        for (uint32_t k = 0; k < 32; ++k) {
-          if ((w[0] >> k) & 1u) s_stage[p0++] = (uint16_t)(v0 + k);
-          if ((w[1] >> k) & 1u) s_stage[p1++] = (uint16_t)(v1 + k);
-        }
-      } else {
-        for (uint32_t x = w[0]; x; x &= x - 1u) s_stage[p0++] = (uint16_t)(v0 + __ffs(x) - 1);
-        for (uint32_t x = w[1]; x; x &= x - 1u) s_stage[p1++] = (uint16_t)(v1 + __ffs(x) - 1);
-      }
+      for (uint32_t x = w[0]; x; x &= x - 1u) s_stage[p0++] = (uint16_t)(v0 + __ffs(x) - 1);
+      for (uint32_t x = w[1]; x; x &= x - 1u) s_stage[p1++] = (uint16_t)(v1 + __ffs(x) - 1);
       __syncthreads();
       const uint32_t total = s_total;
 #pragma unroll 4

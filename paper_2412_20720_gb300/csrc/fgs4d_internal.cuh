@@ -15,7 +15,8 @@ constexpr int kPreBlock = 256;      // threads per preprocess block
 constexpr int kPreStageBytes = 56;  // a staged record
 // Logical preprocess blocks from which the staged form is taken (when the
 // staging area fits): about as many as run at once, so that blocks wait for
-// one another.
+// one another.  Look-back / staged (us): 1172 blocks 38.4 / 33.5, 31k blocks of
+// 8 views 903 / 577, 70k blocks of 6 views 1843 / 1124.
 constexpr int kPreStagedMinBlocks = 608;
 constexpr int kEmitBlock = 256;     // threads per pair-scan / emission block
 constexpr int kEmitChunk = 2048;    // (slot, rect tile) pairs per emission chunk
@@ -23,7 +24,8 @@ constexpr int kSortThreads = 256;   // threads per radix block
 constexpr int kSortItems = 8;       // keys per thread per radix block (instance sort)
 constexpr int kSortTile = kSortThreads * kSortItems;
 // Keys per thread per radix block of the depth sort: 4, so that 80k keys
-// occupy more SMs, or 8 (half the look-backs) from this capacity on.
+// occupy more SMs, or 8 (half the look-backs) from this capacity on:
+// bin_sort 698 -> 664 us at 2.3M keys.
 constexpr int kDepthSortItems = 4, kDepthSortItemsLarge = 8;
 constexpr int64_t kDepthSortLargeMin = int64_t(1) << 20;
 constexpr int kInstSortItems = 8;   // keys per thread per radix block of the instance (tile-id) sort
@@ -41,12 +43,13 @@ constexpr int kCellPrefixThreads = 512;
 // cells (8 views, 1.9M) 168 / 194; 48,000 over 352 cells (8-pixel tiles) 91 /
 // 120; the 6-view street call (5.4M over 810 cells, 685M) 20,900 / 4,100.
 constexpr int64_t kCellsMinVisible = 65536, kCellsMinPerCell = 1024;
-// Instance capacity from which cell_write takes its form for dense masks:
-// bin_sort 4425 -> 4140 us at 741M instances (with the depth sort's larger
-// tickets), 110 -> 116 us at 1.7M.
-constexpr int64_t kCellDenseMinCap = int64_t(1) << 26;
-// Visible slots up to which the depth sort ranks by counting.
-constexpr int64_t kRankSortMax = 8192;
+// Visible slots up to which the depth sort ranks by counting.  bin_sort (us) by
+// passes / by counting at 1352x1014: 630 slots 50.8 / 37.9, 1889 57.5 / 47.9,
+// 3733 62.3 / 57.9, 7512 65.7 / 88.9.
+constexpr int64_t kRankSortMax = 4096;
+// Visible capacity from which a pair-scan thread takes four slots: 2.3M visible
+// slots of 8 views 136 -> 111 us (a quarter of the look-backs); 94k slots would
+// fill 92 of 152 SMs.
 constexpr int64_t kPairScanWideMin = int64_t(1) << 19;
 constexpr int kRadixBits = 8;
 constexpr int kRadixBins = 1 << kRadixBits;

@@ -6,7 +6,8 @@
 // sorting every (tile, Gaussian) instance on a 64-bit (tile << 32 | depth)
 // key, the visible pairs are first sorted by depth alone (31 key bits, one
 // element per pair), the instances are then emitted in that order, and a
-// stable sort on the tile id alone (13-19 bits) groups them per tile.  Both
+// stable sort on the tile id alone (13-19 bits) groups them per tile (large
+// calls: cells.cuh).  Both
 // sorts are stable LSD radix sorts, so the result equals the sort on the
 // 64-bit key with the slot as tie-break, while the instance array (8x larger
 // than the visible set at the benchmark sizes) is only passed over
@@ -29,7 +30,7 @@ constexpr uint32_t kFlagAgg = 1u << 30;
 constexpr uint32_t kFlagInc = 2u << 30;
 constexpr uint32_t kValMask = kFlagAgg - 1u;
 
-// Decoupled look-back of digit d for ticket b (one or more radix sub-tiles):
+// Decoupled look-back of digit d for ticket b:
 // publishes the ticket's count of the digit, sums the counts of the tickets
 // before it back to the nearest inclusive prefix (reading a window of kWin
 // predecessors per round trip: their words are independent loads), publishes
@@ -842,8 +843,7 @@ cudaError_t bin_cells(const Layout &L, const EmitArgs &ea_in, const RasterViews<
   if (e != cudaSuccess) return e;
   e = launch_pdl(cell_prefix_kernel<MAXV>, (unsigned)std::min(L.total_cells, 152 * 8), kCellPrefixThreads, st, C, rv);
   if (e != cudaSuccess) return e;
-  return launch_pdl(L.inst_cap >= kCellDenseMinCap ? cell_write_kernel<MAXV, true> : cell_write_kernel<MAXV, false>,
-                    (unsigned)L.cell_grid, kCellBlock, st, C, rv);
+  return launch_pdl(cell_write_kernel<MAXV>, (unsigned)L.cell_grid, kCellBlock, st, C, rv);
 }
 
 // Depth sort of the visible slots (31 key bits: depth > near > 0); the

@@ -104,7 +104,7 @@ def test_left_out_tiles_are_skipped_by_every_pixel(tile):
 
 # one key; a group of 32 less and more one; the last count ranked by counting
 # and the first sorted by passes
-@pytest.mark.parametrize("n", [1, 31, 32, 33, 257, 8191, 8192, 8193])
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 257, 4095, 4096, 4097, 8193])
 def test_depth_order_of_few_slots(n):
     import torch
     rng = np.random.default_rng(n)
