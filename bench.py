@@ -873,14 +873,14 @@ def tgt_scene_seed() -> int:
 
 
 def bin_sort_bytes(vis: int, inst: int, total_tiles: int) -> float:
-    """Algorithmic DRAM bytes of fgs4d_bin_sort: the depth sort's four 8-bit
-    passes over the visible pairs (key and value read and written, 16 B), the
-    pair scan (52 B read and 52 B written per pair), the emission (8 B per
-    instance) and the tile sort's ceil(bits / 8) passes (16 B per instance),
-    plus the ranges (8 B per tile)."""
-    import math
-    passes = max(1, math.ceil(max(1, math.ceil(math.log2(max(total_tiles, 2)))) / 8))
-    return vis * (4 * 16 + 104) + inst * (8 + 16 * passes) + 8 * total_tiles
+    """A lower bound on the DRAM bytes of fgs4d_bin_sort on either route: the
+    depth sort's four 8-bit passes over the visible pairs (key and value read
+    and written, 16 B), the pair scan (52 B read and 52 B written per pair),
+    the instance list written once (8 B per instance) and the ranges (8 B per
+    tile).  Left out: the 28 B per (cell, slot) pair of the two-level binning,
+    whose count stays on the device, and the 16 B per instance and pass of the
+    instance sort that smaller calls take."""
+    return vis * (4 * 16 + 104) + inst * 8 + 8 * total_tiles
 
 
 def run_batched(dev, scene, views, label, steps, group, plain=True, tiles=(16,), hbm=6800.0):
@@ -975,8 +975,8 @@ def run_batched(dev, scene, views, label, steps, group, plain=True, tiles=(16,),
                            "the %d calls of a step" % len(rs),
            "bin_sort_roofline": {"bound": "hbm", "achieved": bs_gbs, "peak": hbm, "unit": "GB/s",
                                  "frac": bs_gbs / hbm, "bytes_per_step": bs_bytes,
-                                 "bytes_basis": "bin_sort_bytes(): depth sort, pair scan, emission, tile-sort "
-                                                "passes and ranges",
+                                 "bytes_basis": "bin_sort_bytes(), a lower bound: depth sort, pair scan, the instance "
+                                                "list written once and ranges",
                                  "peak_basis": "measured hbm_gbs"}}
     del graph
     # The same groups as calls on parallel streams (lean grids for their
