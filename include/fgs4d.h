@@ -84,9 +84,10 @@ typedef struct fgs4d_settings {
   float bg[3];           /* background colour composited behind the Gaussians */
   int64_t vis_capacity;  /* max visible (view, Gaussian) pairs; 0 = n * nviews */
   int64_t inst_capacity; /* max (tile, Gaussian) instances over all views, > 0 */
-  int32_t pixels_per_thread; /* compositor block shape: 0 (default 4), 2, 4 or 8 pixels
-                                of one tile column per thread; results are identical */
-  int32_t shared_batch;      /* records the compositors stage per shared-memory batch: 0 (= 256), 128 or 256 */
+  int32_t pixels_per_thread; /* compositor block shape: 2, 4 or 8 pixels of one tile column per
+                                thread, or 0 (chosen by the tile count); results are identical */
+  int32_t shared_batch;      /* records the compositors stage per shared-memory batch: 128 or 256, or
+                                0 (256 forward, 128 adjoint); results are identical */
   int32_t stage_blocks_per_sm; /* grids of the latency-bound stages: 0 = full-GPU grids (the lowest
                                   latency for one frame alone); k in 1..8 = at most k resident blocks
                                   per SM for preprocess and the radix passes and 2k for the instance

@@ -5,7 +5,8 @@
 // colour of Eq. 6 (zero background).  The geometry is that of a pre-trained
 // 4DGS, so the backward pass returns dL/df and dL/dS(s) only.
 //
-// Both directions are contractions: the map is F[p][c] = sum_j w[p][j]
+// Both directions are contractions (for D <= 16 the forward stays scalar, see
+// render_features_scalar_kernel): the map is F[p][c] = sum_j w[p][j]
 // fhat[j][c], and the adjoint needs v[j][c] = sum_p w[p][j] dL/dF[p][c].  One
 // CTA per (view, tile), one pixel per thread; a warp computes the weights of
 // its 32 pixels for kChunk entries (pixel_alpha's skip/stop decisions, so the
@@ -15,8 +16,8 @@
 // lo hi, so a product is within 2^-22; FP32 accumulators that start at zero
 // every chunk and are added up in FP32).  The warp-level instruction is taken
 // rather than tcgen05 because the weights come out of a per-pixel recurrence
-// 32 pixels at a time and the contraction is the small part: per chunk of 16
-// entries and 32 pixels about 50 of 450 issued instructions at D = 32.
+// 32 pixels at a time and the contraction is the small part: 48 products of
+// some 800 issued instructions per chunk of 16 entries and 32 pixels at D = 32.
 //
 // Backward: a warp's product sums over its own 32 pixels; the warps' sums of
 // an entry are added through shared memory, the normalisation Jacobian is
@@ -24,9 +25,11 @@
 // dL/df = S (.) dL/dg is added with one atomic per component, and dL/dS(s) =
 // f (.) dL/dg is summed per block.
 //
-// Measured at 300k Gaussians, one 1352x1014 view, D = 32 (forward / backward):
-// scalar multiply-adds with a shuffle butterfly per (warp, entry) 0.856 / 1.413
-// ms.
+// Measured at 300k Gaussians, one 1352x1014 view, before (multiply-adds with a
+// shuffle butterfly and D atomics per (warp, entry)) -> now, us: D = 32 forward
+// 900 -> 716, backward 1492 -> 860; D = 16 backward 933 -> 586; D = 8 663 -> 512.
+// Bound by issue (57 and 62 % of the slots at a quarter of the warps: the
+// accumulators or operands take 128 registers a thread).
 #include <algorithm>
 
 #include "fgs4d_internal.cuh"
@@ -232,7 +235,7 @@ struct FeatEntries {
 
 // Stages records [base, base + nb) of a tile's list, four threads per entry,
 // each with D / 4 components: `put(k, c, f, fhat)` receives component c of the
-// raw gated-by-nothing feature and of the normalised gated one (0 where it is
+// raw feature and of the normalised gated one (0 where it is
 // not finite; `bad` then has the component's bit).  Entries up to the next
 // multiple of kChunk are staged as skipped by every pixel with zero features.
 // Returns whether any component of the thread's entries was not finite.

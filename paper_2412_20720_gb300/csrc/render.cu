@@ -5,7 +5,7 @@
 // kPPT pixels of one column, so the per-entry work that does not depend on the
 // row (shared-memory loads, dx, (a1 dx)^2, b1 dx) is done once for kPPT pixels.
 // The tile's depth-sorted list is staged through shared memory in batches of
-// 256 records; the CTA stops loading once every pixel has reached the
+// 128 or 256 records; the CTA stops loading once every pixel has reached the
 // transmittance cutoff (__syncthreads_count).  alpha = min(0.99, a 2^-q),
 // skip when alpha < 1/255, stop before the entry that would take T below 1e-4
 // -- evaluated by pixel_alpha, shared with the backward pass so both take
@@ -15,9 +15,9 @@
 //
 // Backward: the same tiles traversed back to front from each pixel's last
 // composited entry, recomputing T_i = T_{i+1} / (1 - alpha_i) from the final
-// transmittance.  A thread first sums its strip's contributions; the sums are
-// then reduced across the warp by shuffles and added with two float4 and one
-// float2 atomic per warp and entry.
+// transmittance.  A thread first sums its strip's contributions; the lanes' sums
+// then meet in shared memory (render_bwd_kernel) and are added with one atomic
+// per sum, warp and entry.
 #include <algorithm>
 #include <type_traits>
 
@@ -369,7 +369,9 @@ constexpr int bwd_min_blocks() {
 // kRedEntries entries are rows, and each lane then adds up one row (8 float4
 // loads) and adds it with one atomic -- about 25 warp instructions an entry
 // where the transposed shuffle butterfly and its operands took about 70.
-// Train call of 4 views: see launch_bwd_batch for the measured times.
+// 4 views of 1352x1014, 349k visible, 6.3M instances: 1.85 -> 1.11 G warp
+// instructions, 1.755 -> 1.399 ms (8 rows a thread; 1.525 with 4); it now issues
+// in 67 % of the slots with 28 % of the warps resident.
 //
 // kAux: the loss also has gradients dL/dD, dL/dO with respect to the depth
 // and opacity channels (zero background, x_i = z_i resp. 1 in the colour
