@@ -224,9 +224,16 @@ class Renderer:
         """Adds dL/dparams into ``grads`` for the last forward of this renderer;
         with ``densify_stats`` ([n, 4]) also accumulates, per visible (view,
         Gaussian), (|dL/dmu_2d|, |dL/dmu_t|, 1, 0)."""
+        self._backward(params, dL_drgb, grads, densify_stats)
+
+    def _backward(self, params: dict, dL_drgb: torch.Tensor, grads: dict, densify_stats=None, clear: bool = False):
+        """backward(); with ``clear`` the gradients are cleared first, in one
+        launch made after every tensor has been checked."""
         g = self.gaussians(params)
         gg = self._grads(grads, densify_stats)
         dL = dL_drgb.contiguous()
+        if clear:
+            fgs4d.zero_set([(_ptr(grads[k]), grads[k].numel()) for k in PARAM_KEYS], self.stream())
         fgs4d.render_bwd(g, self.views, self.nviews, self.settings, _ptr(self.ws), self.ws_bytes, _ptr(dL), gg,
                          self.stream())
 
@@ -512,9 +519,10 @@ class Render4DGS(torch.autograd.Function):
     def backward(ctx, grad_out):
         saved = ctx.saved_tensors
         params = dict(zip(PARAM_KEYS, saved))
+        # Saved-tensor hooks may hand back other tensors than were saved: the
+        # renderer checks them before anything is written.
         grads = {k: torch.empty_like(v) for k, v in params.items()}
-        fgs4d.zero_set([(_ptr(g), g.numel()) for g in grads.values()], ctx.renderer.stream())
-        ctx.renderer.backward(params, grad_out, grads)
+        ctx.renderer._backward(params, grad_out, grads, clear=True)
         return (None,) + tuple(grads[k] for k in PARAM_KEYS)
 
 
