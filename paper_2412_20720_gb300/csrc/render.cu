@@ -75,15 +75,26 @@ inline int render_ppt(const fgs4d_settings *s, const Layout &L, bool adjoint) {
 }
 
 
+// Magnitudes up to which products of gradients with colours and depths, and
+// their sums, stay far below the largest float (render_bwd_kernel).
+constexpr float kMagMax = 1152921504606846976.0f;  // 2^60
+
+// What the records a thread staged ask of the pixel loop.
+struct StagedFlags {
+  bool clamp;  // some entry can reach the 0.99 clamp
+  bool large;  // some colour or depth is above kMagMax (or not a number)
+};
+
 // Stages records [base, min(base + kBatch, end)) of the tile list into shared
 // memory; slots out of range (only possible after a recorded timeout) stage a
 // record that every pixel skips.
 template <int NT, int kBatch>
-__device__ __forceinline__ void stage_batch(const uint32_t *inst_val, const float4 *rec_geom,
-                                            const float4 *rec_color, const float *rec_blue, uint32_t vis_cap,
-                                            uint32_t base, uint32_t end, float4 *s_geom, float4 *s_col,
-                                            float *s_blue, uint32_t *s_slot, const float4 *rec_aux = nullptr,
-                                            float4 *s_aux = nullptr) {
+__device__ __forceinline__ StagedFlags stage_batch(const uint32_t *inst_val, const float4 *rec_geom,
+                                                   const float4 *rec_color, const float *rec_blue, uint32_t vis_cap,
+                                                   uint32_t base, uint32_t end, float4 *s_geom, float4 *s_col,
+                                                   float *s_blue, uint32_t *s_slot, const float4 *rec_aux = nullptr,
+                                                   float4 *s_aux = nullptr) {
+  StagedFlags f = {false, false};
 #pragma unroll
   for (int i = 0; i < kBatch / NT; ++i) {
     const int k = threadIdx.x + i * NT;
@@ -91,19 +102,23 @@ __device__ __forceinline__ void stage_batch(const uint32_t *inst_val, const floa
     if (idx < end) {
       const uint32_t s = inst_val[idx];
       if (s_slot) s_slot[k] = s;
+      float4 geom = make_float4(0.f, 0.f, 0.f, 0.f), col = make_float4(0.f, kLogAlphaNone, 0.f, 0.f), aux = geom;
+      float blue = 0.f;
       if (s < vis_cap) {
-        s_geom[k] = rec_geom[s];
-        s_col[k] = rec_color[s];
-        s_blue[k] = rec_blue[s];
-        if (s_aux) s_aux[k] = rec_aux[s];
-      } else {
-        s_geom[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        s_col[k] = make_float4(0.f, kLogAlphaNone, 0.f, 0.f);
-        s_blue[k] = 0.f;
-        if (s_aux) s_aux[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        geom = rec_geom[s];
+        col = rec_color[s];
+        blue = rec_blue[s];
+        if (s_aux) aux = rec_aux[s];
       }
+      s_geom[k] = geom;
+      s_col[k] = col;
+      s_blue[k] = blue;
+      if (s_aux) s_aux[k] = aux;
+      f.clamp = f.clamp || entry_clamps(col.y);
+      f.large = f.large || !(fabsf(col.z) + fabsf(col.w) + fabsf(blue) + fabsf(aux.x) <= kMagMax);
     }
   }
+  return f;
 }
 
 // kMode 0: image (and the per-pixel state of the backward pass); 3: image
@@ -180,19 +195,13 @@ __global__ void __launch_bounds__(TILE *TILE / PPT, (fwd_min_blocks<TILE, PPT, k
   uint32_t n_eval = 0u, n_comp = 0u, n_evb = 0u;
   for (uint32_t base = range.x; base < range.y; base += kBatch) {
     if (__syncthreads_count(nlive > 0) == 0) break;
-    stage_batch<NT, kBatch>(A.inst_val, A.rec_geom, A.rec_color, A.rec_blue, A.vis_cap, base, range.y, s_geom, s_col,
-                    s_blue, nullptr, kAux ? A.rec_aux : nullptr, kAux ? s_aux : nullptr);
+    const StagedFlags staged =
+        stage_batch<NT, kBatch>(A.inst_val, A.rec_geom, A.rec_color, A.rec_blue, A.vis_cap, base, range.y, s_geom, s_col,
+                                s_blue, nullptr, kAux ? A.rec_aux : nullptr, kAux ? s_aux : nullptr);
     const int nb = (int)min(range.y - base, (uint32_t)kBatch);
     // Whether any staged entry can reach the 0.99 clamp (opacity > 0.98, rare):
-    // each thread checks the entries it staged, and the barrier that
-    // publishes the batch ORs the answers.
-    bool my_clamp = false;
-#pragma unroll
-    for (int i = 0; i < kBatch / NT; ++i) {
-      const int k = threadIdx.x + i * NT;
-      if (k < nb) my_clamp = my_clamp || entry_clamps(s_col[k].y);
-    }
-    const bool clamp_any = __syncthreads_or(my_clamp) != 0;
+    // the barrier that publishes the batch ORs the threads' answers.
+    const bool clamp_any = __syncthreads_or(staged.clamp) != 0;
     const uint32_t pos0 = base - range.x + 1u;
     // One entry of the list at every pixel of the thread, two pixels at a time
     // with two-lane FP32 instructions (each lane rounds as the scalar one
@@ -415,7 +424,11 @@ __global__ void __launch_bounds__(TILE *TILE / kPPT, (bwd_min_blocks<TILE, kPPT,
   uint32_t last[2 * kPairs];
   uint32_t my_max = 0u;
   const float *g = A.dL_drgb + V.pix_base * 3;
-  bool finite = true;  // every upstream gradient of the thread, then of the warp (see entry())
+  // Whether no product of the thread's (then the warp's) upstream gradients can
+  // overflow: a skipped pixel takes part with weight 0, which must not meet an
+  // infinity (see entry()).  With gradients, colours and depths up to kMagMax
+  // the sums below stay under 2^124.
+  bool tame = true;
 #pragma unroll
   for (int k = 0; k < 2 * kPairs; ++k) {
     float t = 1.0f, c0 = 0.f, c1 = 0.f, c2 = 0.f, d = 0.f, o = 0.f;
@@ -433,8 +446,9 @@ __global__ void __launch_bounds__(TILE *TILE / kPPT, (bwd_min_blocks<TILE, kPPT,
         o = ga[HW + p];
       }
     }
-    finite = finite && isfinite(c0) && isfinite(c1) && isfinite(c2) && isfinite(d) && isfinite(o);
     const float dr = t * (c0 * A.bg0 + c1 * A.bg1 + c2 * A.bg2);  // the background behind all
+    tame = tame && fabsf(c0) <= kMagMax && fabsf(c1) <= kMagMax && fabsf(c2) <= kMagMax && fabsf(d) <= kMagMax &&
+           fabsf(o) <= kMagMax && fabsf(dr) <= kMagMax * kMagMax;
     auto lane = [k](float2 &v, float x) { (k & 1 ? v.y : v.x) = x; };
     lane(T[k >> 1], t);
     lane(nC0[k >> 1], -c0);
@@ -453,7 +467,7 @@ __global__ void __launch_bounds__(TILE *TILE / kPPT, (bwd_min_blocks<TILE, kPPT,
   __syncthreads();
   const uint32_t end = range.x + min(s_maxlast, range.y - range.x);
   const uint32_t warp_max = __reduce_max_sync(0xffffffffu, my_max);  // past the last entry of the warp's pixels
-  finite = __all_sync(0xffffffffu, finite);
+  tame = __all_sync(0xffffffffu, tame);
   const int lane = threadIdx.x & 31;
   float(*red)[kRedStride] = s_red[threadIdx.x >> 5];
   int buffered = 0;  // entries in `red` (the same in every lane)
@@ -507,19 +521,17 @@ __global__ void __launch_bounds__(TILE *TILE / kPPT, (bwd_min_blocks<TILE, kPPT,
   for (int bi = nbatch - 1; bi >= 0; --bi) {
     const uint32_t base = range.x + (uint32_t)bi * kBatch;
     __syncthreads();
-    stage_batch<kRenderThreads, kBatch>(A.inst_val, A.rec_geom, A.rec_color, A.rec_blue, A.vis_cap, base, end, s_geom,
-                                s_col, s_blue, s_slot, kAux ? A.rec_aux : nullptr, kAux ? s_aux : nullptr);
+    const StagedFlags staged =
+        stage_batch<kRenderThreads, kBatch>(A.inst_val, A.rec_geom, A.rec_color, A.rec_blue, A.vis_cap, base, end, s_geom,
+                                            s_col, s_blue, s_slot, kAux ? A.rec_aux : nullptr, kAux ? s_aux : nullptr);
     const int nb = (int)min(end - base, (uint32_t)kBatch);
     // Whether any staged entry can reach the 0.99 clamp (rare): then the batch
-    // takes the clamping copy of the pixel loop, which gives the entries that
-    // cannot clamp the same alpha.
-    bool my_clamp = false;
-#pragma unroll
-    for (int i = 0; i < kBatch / kRenderThreads; ++i) {
-      const int k = threadIdx.x + i * kRenderThreads;
-      if (k < nb) my_clamp = my_clamp || entry_clamps(s_col[k].y);
-    }
-    const bool clamp_any = __syncthreads_or(my_clamp) != 0;
+    // takes the careful copy of the pixel loop, which gives the entries that
+    // cannot clamp the same alpha.  So does every batch of a warp whose
+    // products may overflow: from its upstream gradients, or from the first
+    // batch on that holds a colour or depth above kMagMax.
+    const bool clamp_any = __syncthreads_or(staged.clamp || staged.large) != 0;
+    if (clamp_any && __syncthreads_or(staged.large)) tame = false;
     // One list entry.
     auto entry = [&](int j, uint32_t pos, auto clamp_tag) {
       constexpr bool kClamp = decltype(clamp_tag)::value;
@@ -556,7 +568,7 @@ __global__ void __launch_bounds__(TILE *TILE / kPPT, (bwd_min_blocks<TILE, kPPT,
         const bool v0 = pos < last[k0] && al0 >= kAlphaMin, v1 = pos < last[k1] && al1 >= kAlphaMin;
         if (!__any_sync(0xffffffffu, v0 || v1)) continue;
         contrib = true;
-        if (!finite) {  // an infinite or NaN gradient of a skipped pixel must not meet its zero weight: one at a time
+        if (kClamp && !tame) {  // an infinity or NaN of a skipped pixel must not meet its zero weight: one at a time
           auto pixel = [&](bool v, float al, float aG, float &t, float &dr, float n0, float n1, float n2, float nd,
                            float no, float &sr, float &sg, float &sb, float &sz, float &gpk) {
             if (!v) return;
@@ -641,7 +653,7 @@ __global__ void __launch_bounds__(TILE *TILE / kPPT, (bwd_min_blocks<TILE, kPPT,
     };
     const uint32_t pos0 = base - range.x;  // entry index of the batch's first entry
     const int first = warp_max > pos0 ? (int)min(warp_max - pos0, (uint32_t)nb) - 1 : -1;
-    if (clamp_any) {
+    if (clamp_any || !tame) {
       for (int j = first; j >= 0; --j) {
         entry(j, pos0 + j, std::true_type());
         if (buffered == kRedEntries) flush();

@@ -90,3 +90,51 @@ def test_feature_map_of_a_feature_that_is_not_finite(D):
     np.testing.assert_array_equal(np.isnan(got[5]), hit)
     assert np.isfinite(got[np.arange(D) != 5]).all()
     np.testing.assert_array_equal(got[:, ~hit], ref[:, ~hit])
+
+
+@pytest.mark.parametrize("tile,ppt", [(16, 2), (16, 4), (16, 8), (8, 1), (8, 2)])
+def test_products_that_overflow_stay_with_their_pixel(tile, ppt):
+    """A finite gradient so large that its products with the colours overflow
+    reaches only the Gaussians its pixel composites."""
+    import torch
+    p, r = _case(tile, ppt)
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    base = torch.randn(3 * r.total_pixels, device="cuda", generator=gen)
+
+    def run(v, s):
+        r.forward(p)
+        d = base * s
+        d[[c * 72 * 96 + 37 * 96 + 51 for c in range(3)]] = v  # all channels of pixel (51, 37)
+        grads = {k: torch.zeros_like(p[k]) for k in PARAM_KEYS}
+        r.backward(p, d, grads)
+        return torch.cat([grads[k].reshape(1500, -1) for k in PARAM_KEYS], 1).cpu().numpy()
+
+    _check(run, 3.4e38, 1e-4)
+
+
+@pytest.mark.parametrize("tile,ppt", [(16, 2), (16, 4), (16, 8), (8, 1), (8, 2)])
+def test_a_colour_near_the_largest_float_stays_with_its_pixels(tile, ppt):
+    """One Gaussian's colour of 8e37 makes the products with ordinary gradients
+    overflow at the pixels that composite it and nowhere else."""
+    import torch
+    p, r = _case(tile, ppt)
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    base = 8.0 * torch.randn(3 * r.total_pixels, device="cuda", generator=gen)
+
+    def run(q, d):
+        img = r.forward(q).clone()
+        grads = {k: torch.zeros_like(p[k]) for k in PARAM_KEYS}
+        r.backward(q, d, grads)
+        return img, torch.cat([grads[k].reshape(1500, -1) for k in PARAM_KEYS], 1).cpu().numpy()
+
+    img, ref = run(p, base)
+    g = int(np.argsort(np.abs(ref).sum(1))[-100])  # a Gaussian that the view shows
+    q = {k: v.clone() for k, v in p.items()}
+    q["sh"][g] = 0.0
+    q["sh"][g, 0] = 3e38  # times Y_00: colour 8.5e37 in every channel
+    hit = (r.forward(q) != img).view(3, -1).any(0).repeat(3)
+    touched = (run(p, base * hit)[1] != 0).any(1)
+    bad = run(q, base)[1]
+    assert touched[g] and not touched.all() and not np.isfinite(bad).all()
+    assert np.isfinite(bad[~touched]).all()
+    assert np.abs(bad[~touched] - ref[~touched]).max() <= 1e-4 * np.abs(ref).max()
