@@ -256,13 +256,14 @@ __global__ void __launch_bounds__(TILE *TILE / PPT, (fwd_min_blocks<TILE, PPT, k
           C1[q] = __ffma2_rn(make_float2(col.w, col.w), w, C1[q]);
           C2[q] = __ffma2_rn(make_float2(blue, blue), w, C2[q]);
           if (kAux) {
-            X0[q] = __ffma2_rn(make_float2(xa.x, xa.x), w, X0[q]);
-            // a flow may overflow to infinity and must not meet a zero weight
+            // a depth or flow may overflow to infinity and must not meet a zero weight
             if (c0) {
+              X0[q].x = __fmaf_rn(xa.x, w.x, X0[q].x);
               X1[q].x = __fmaf_rn(xa.y, w.x, X1[q].x);
               X2[q].x = __fmaf_rn(xa.z, w.x, X2[q].x);
             }
             if (c1) {
+              X0[q].y = __fmaf_rn(xa.x, w.y, X0[q].y);
               X1[q].y = __fmaf_rn(xa.y, w.y, X1[q].y);
               X2[q].y = __fmaf_rn(xa.z, w.y, X2[q].y);
             }

@@ -138,3 +138,28 @@ def test_a_colour_near_the_largest_float_stays_with_its_pixels(tile, ppt):
     assert touched[g] and not touched.all() and not np.isfinite(bad).all()
     assert np.isfinite(bad[~touched]).all()
     assert np.abs(bad[~touched] - ref[~touched]).max() <= 1e-4 * np.abs(ref).max()
+
+
+def test_depth_that_overflows_stays_with_its_pixels():
+    """A Gaussian whose camera depth overflows to infinity reaches the depth
+    plane of the pixels that composite it and no other."""
+    import torch
+    params = sy.make_scene(1500, 23, (-1, -1, -1), (1, 1, 1), sh_degree=1, t_order=1).as_dict()
+    p = to_device(params)
+    # looking along (1, 1, 1): a mean of 3.4e38 in all coordinates has depth 5.9e38 and projects to the image centre
+    view = sy.look_at((-2.0, -2.0, -2.0), (0, 0, 0), (0, -1, 0), 96, 72, 0.5)
+    p["opacity_logit"] -= 3.0  # faint: the last Gaussian still shows
+    p["mean"][7] = torch.tensor([3.4e38, 3.4e38, 3.4e38, 0.5], device="cuda")
+    p["opacity_logit"][7] = 3.0
+    for tile, ppt in ((16, 2), (16, 4), (16, 8), (8, 1), (8, 2)):
+        r = Renderer(1500, [view], RenderConfig(sh_degree=1, t_order=1, inst_capacity=1 << 18, tile=tile,
+                                                pixels_per_thread=ppt))
+        rgb, aux = r.forward_aux(p, 0.1)
+        q = dict(p, opacity_logit=p["opacity_logit"].clone())
+        q["opacity_logit"][7] = -30.0
+        rgb0, aux0 = r.forward_aux(q, 0.1)
+        d, d0 = aux.view(4, -1)[0], aux0.view(4, -1)[0]
+        hit = (aux.view(4, -1)[1] != aux0.view(4, -1)[1]) | (rgb != rgb0).view(3, -1).any(0)
+        assert 0 < int(hit.sum()) < 100 and torch.isfinite(d0).all()
+        assert torch.isinf(d[hit]).all()
+        assert torch.equal(d[~hit], d0[~hit])
