@@ -214,6 +214,15 @@ __device__ __forceinline__ void tf32_split(float x, uint32_t *hi, uint32_t *lo) 
   *lo = __float_as_uint(tf32_round(__fsub_rn(x, h)));
 }
 
+// The same for values up to the largest float: where hi would round to
+// infinity it is cut off instead (x = hi + lo to about 2^-21 there).
+__device__ __forceinline__ void tf32_split_any(float x, uint32_t *hi, uint32_t *lo) {
+  float h = tf32_round(x);
+  if (isinf(h)) h = __uint_as_float(__float_as_uint(x) & 0xffffe000u);
+  *hi = __float_as_uint(h);
+  *lo = __float_as_uint(tf32_round(__fsub_rn(x, h)));
+}
+
 // c += a b: a 16 x 8 (row = lane / 4, + 8; column = lane % 4, + 4), b 8 x 8
 // (row = lane % 4, + 4; column = lane / 4), c 16 x 8 (row = lane / 4, + 8;
 // columns 2 (lane % 4), + 1).
@@ -495,7 +504,7 @@ __global__ void __launch_bounds__(feat_threads<TILE>()) render_features_bwd_kern
     for (int ks = 0; ks < 4; ++ks)
 #pragma unroll
       for (int h = 0; h < 2; ++h)
-        tf32_split(s_buf[warp][lr * kWBwd + 8 * ks + lc + 4 * h], &Gh[ks][n][h], &Gl[ks][n][h]);
+        tf32_split_any(s_buf[warp][lr * kWBwd + 8 * ks + lc + 4 * h], &Gh[ks][n][h], &Gl[ks][n][h]);
   }
   const uint32_t bad_pixels = __ballot_sync(0xffffffffu, bad);  // of the warp
   __syncwarp();

@@ -163,3 +163,28 @@ def test_depth_that_overflows_stays_with_its_pixels():
         assert 0 < int(hit.sum()) < 100 and torch.isfinite(d0).all()
         assert torch.isinf(d[hit]).all()
         assert torch.equal(d[~hit], d0[~hit])
+
+
+@pytest.mark.parametrize("D,tile", [(8, 16), (16, 8), (32, 16)])
+def test_feature_gradients_near_the_largest_float(D, tile):
+    """The adjoint is linear in the upstream gradient up to the largest floats:
+    a component of 3.4025e38 (which rounds to infinity with 11 significant
+    bits) gives that multiple of the gradient of 1, to 1e-3."""
+    import torch
+    p, r = _case(tile, 0)
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    feats = torch.randn((1500, D), device="cuda", generator=gen)
+
+    def run(v):
+        r.forward_features(p, feats)
+        d = torch.zeros(D * r.total_pixels, device="cuda")
+        d[3 * 72 * 96 + 37 * 96 + 51] = v
+        g = torch.zeros_like(feats)
+        r.backward_features(feats, None, d, g)
+        return g.cpu().numpy().astype(np.float64)
+
+    one, big = run(1.0) * 3.4025e38, run(3.4025e38)
+    below = np.abs(one).max(1) < 3e38  # the others may overflow
+    assert (one[below] != 0).any()
+    assert np.isfinite(big[below]).all()
+    assert np.abs(big[below] - one[below]).max() <= 1e-3 * np.abs(one[below]).max()
