@@ -91,6 +91,22 @@ __device__ __forceinline__ uint64_t cell_mask(float u, float v, float a1, float 
   return mask;
 }
 
+// The tiles of all slots' rects: the instances that a call whose pairs
+// outnumber the pair capacity may need.  Added up here, only then, so that the
+// pair scan carries one sum.
+__device__ __forceinline__ void add_rect_tiles(const EmitArgs &A, int64_t nvis) {
+  uint64_t sum = 0ull;
+  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < nvis; j += (int64_t)gridDim.x * blockDim.x) {
+    const int4 r = A.emit_rec[3 * j + 2];
+    const int w = (r.w & 0xffff) - (r.z & 0xffff), h = (int)((uint32_t)r.w >> 16) - (int)((uint32_t)r.z >> 16);
+    sum += (uint64_t)max(w, 0) * (uint64_t)max(h, 0);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if ((threadIdx.x & 31) == 0 && sum)
+    atomicAdd(reinterpret_cast<unsigned long long *>(&A.counters[kCtrRectTiles64]), (unsigned long long)sum);
+}
+
 // Pair emission, one candidate (slot, cell) pair per thread and kCellChunk
 // pairs per chunk: the pair's slot is found by a binary search of the pair
 // prefix and its mask computed.  When the candidates fit the pair buffers (the
@@ -120,6 +136,7 @@ __global__ void __launch_bounds__(kCellChunk) cell_emit_kernel(CellArgs C, Raste
     if (blockIdx.x == 0 && threadIdx.x == 0) A.counters[kCtrCellPairs] = 0u;
     return;
   }
+  if (A.counters[kCtrPairOverflow]) add_rect_tiles(A, nvis);
   for (int p = 0; p < C.cell_passes; ++p) s_hist[p][threadIdx.x] = 0u;
   const bool direct = (int64_t)npairs <= A.inst_cap;
   if (direct && blockIdx.x == 0 && threadIdx.x == 0) A.counters[kCtrCellPairs] = npairs;
@@ -407,8 +424,12 @@ __global__ void __launch_bounds__(kCellPrefixThreads) cell_prefix_kernel(CellArg
     }
     base += total;
   }
-  if (threadIdx.x == 0)
+  if (threadIdx.x == 0) {
+    if (A.counters[kCtrPairOverflow])
+      A.counters[kCtrNeedInstances] = (uint32_t)umin64(
+          *reinterpret_cast<const volatile unsigned long long *>(&A.counters[kCtrRectTiles64]), 0xffffffffull);
     set_instance_total(A, *reinterpret_cast<const volatile unsigned long long *>(&A.counters[kCtrInstances64]));
+  }
 }
 
 // Expands every run into its tiles' lists.  The run's (tile, pair) bits are

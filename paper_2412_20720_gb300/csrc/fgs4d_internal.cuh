@@ -83,6 +83,8 @@ enum Counter : int {
   kCtrPairs = 19,        // (slot, rect tile) pairs of all visible slots, or (slot, cell) pairs
   kCtrInstances64 = 20,  // 64-bit instance count of the two-level binning
   kCtrCellDone = 22,     // finished blocks of cell_prefix_kernel
+  kCtrPairOverflow = 23, // two-level binning: more pairs than the pair capacity
+  kCtrRectTiles64 = 24,  // then the tiles of all slots' rects (64 bits)
   kCtrCount = 64
 };
 constexpr size_t kSortControlStart = 32;

@@ -473,14 +473,16 @@ __device__ __forceinline__ void mark_chunks(const EmitArgs &A, int64_t j, uint64
 }
 
 // Sets the pair total (clamped to the pair capacity) and, when pairs are lost
-// to the clamp, the instance bound and the overflow flag.
-__device__ __forceinline__ void set_pair_total(const EmitArgs &A, int64_t nvis, uint64_t all, uint32_t per_pair) {
+// to the clamp, the overflow flag and a bound on the instances needed: the
+// (slot, tile) pairs of the rects.  The two-level binning counts (slot, cell)
+// pairs here and has cell_emit_kernel add up the tiles.
+template <bool kCells>
+__device__ __forceinline__ void set_pair_total(const EmitArgs &A, int64_t nvis, uint64_t all) {
   A.pair_prefix[nvis] = (uint32_t)umin64(all, (uint64_t)A.pair_cap);
   A.counters[kCtrPairs] = (uint32_t)umin64(all, (uint64_t)A.pair_cap);
   if (all > (uint64_t)A.pair_cap) {
-    // Some pairs cannot be examined: report the bound on the instances needed
-    // (per_pair: the most instances of one pair).
-    A.counters[kCtrNeedInstances] = (uint32_t)umin64(all * per_pair, 0xffffffffull);
+    if (kCells) A.counters[kCtrPairOverflow] = 1u;
+    else A.counters[kCtrNeedInstances] = (uint32_t)umin64(all, 0xffffffffull);
     atomicOr(&A.counters[kCtrStatus], kStatusInstOverflow);
   }
 }
@@ -529,7 +531,7 @@ __global__ void __launch_bounds__(kEmitBlock) pair_scan_kernel(EmitArgs A, Raste
   if (threadIdx.x < 32) {
     const uint64_t prefix = lookback_u64_warp(A.lb_scan, (int32_t)b, sum, &A.counters[kCtrStatus]);
     if (threadIdx.x == 0) s_base = prefix;
-    if (threadIdx.x == 0 && j0 + kEmitBlock * kItems >= nvis) set_pair_total(A, nvis, prefix + sum, kCells ? 64u : 1u);
+    if (threadIdx.x == 0 && j0 + kEmitBlock * kItems >= nvis) set_pair_total<kCells>(A, nvis, prefix + sum);
   }
   __syncthreads();
 #pragma unroll

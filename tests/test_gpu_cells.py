@@ -114,3 +114,31 @@ def test_depth_order_of_few_slots(n):
         assert code == fgs4d.OK
         got = r.workspace_view(r.layout.sorted_slots, torch.int32, n).cpu().numpy()
         np.testing.assert_array_equal(got, np.argsort(rec["depth"], kind="stable"))
+
+
+def _lists(r, counts, ntiles):
+    tiles, slots, gr = _read_instances(r, counts[1], ntiles)
+    return tiles, slots, canonical_ranges(gr)
+
+
+@pytest.mark.parametrize("n,cap", [(16_384, 8192), (16_385, 300)])
+def test_pair_overflow_reports_a_need_that_fits(n, cap):
+    """More candidate (slot, cell) pairs than 8 x inst_capacity: the reported
+    need is the tiles of the rects (here each holds an instance), and a call
+    with that capacity succeeds."""
+    W, H, gw, gh = 640, 480, 40, 30
+    rec = _synthetic_records(np.random.default_rng(n), n, W, H, 34, tau=KEEP_ALL)
+    r0 = rec["rect"].astype(np.int64)
+    cells = (((r0[:, 2] - 1) >> 3) - (r0[:, 0] >> 3) + 1) * (((r0[:, 3] - 1) >> 3) - (r0[:, 1] >> 3) + 1)
+    cells[(r0[:, 2] <= r0[:, 0]) | (r0[:, 3] <= r0[:, 1])] = 0
+    assert cells.sum() > 8 * cap
+    keys, vals, ranges = oracle.sort_instances(rec["rect"], rec["depth"], gw, gh)
+    m = keys.shape[0]
+    _, (code, counts) = _run(rec, [sy.tiny_view(W, H)], 16, cap)
+    assert code == fgs4d.ERR_CAPACITY and counts[1] == cap and counts[3] == m
+    r, (code, counts) = _run(rec, [sy.tiny_view(W, H)], 16, counts[3])
+    assert code == fgs4d.OK and counts[1] == m and counts[3] == m
+    tiles, slots, gr = _lists(r, counts, gw * gh)
+    np.testing.assert_array_equal(tiles, (keys >> np.uint64(32)).astype(np.int64))
+    np.testing.assert_array_equal(slots, vals)
+    np.testing.assert_array_equal(gr, ranges)
