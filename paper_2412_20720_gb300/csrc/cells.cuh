@@ -16,7 +16,7 @@
 //   cell_write    per segment: (tile id, slot) of every set bit, in list order
 //
 // The result -- instances ordered by (tile, depth, slot), and their ranges --
-// is that of the instance sort.  Reads and writes per instance drop from the
+// is that of the instance sort, instance for instance.  Reads and writes per instance drop from the
 // sort's 16 bytes a pass to the 8 bytes of the final list; the passes over
 // pairs move 28 bytes a pair.
 
@@ -40,55 +40,89 @@ struct CellArgs {
 // Cells a tile rect [x0, x1) x [y0, y1) touches, by row of cells.
 __device__ __forceinline__ int cell_span(int lo, int hi) { return ((hi - 1) >> kCellShift) - (lo >> kCellShift) + 1; }
 
-// The tiles [tx0, tx1) x [ty0, ty1) of one cell whose pixel-centre box meets
-// the ellipse q <= tau of a record, as bits (ty & 7) * 8 + (tx & 7).  Per row
-// of tiles the ellipse's x extent over the row's band of pixel centres is an
-// interval: with q = (a1 x)^2 + (b1 x + b2 y)^2 and n = a1^2 + b1^2, the
-// rightmost point is x = r / a1 at y = kx r / a1 (r^2 = tau, kx = -b1 / b2);
-// when that y lies outside the band the extreme is on the nearest edge y = Y,
-// x = ky Y + sqrt(tau - (a1 b2 Y)^2 / n) / sqrt(n) (ky = -b1 b2 / n), and the
-// left end is the mirror image.  tau is widened by 1e-3 (0.07 % in alpha) and
-// the interval by 0.03 px plus 1e-5 of its terms, which covers the FP32 error
-// of both, so a tile left out has alpha < 1/255 at every pixel.  A row costs
-// about 35 instructions instead of up to 8 ellipse-box tests of 40.
+// sqrt within an ulp or two (the intervals below have room for that).
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// The tiles [tx0, tx1) x [ty0, ty1) of one cell that ellipse_meets_box accepts
+// for a record, as bits (ty & 7) * 8 + (tx & 7): the instance sort's test, bit
+// for bit, mostly without making it.  Per row of tiles the ellipse's x extent
+// over the row's band of pixel centres is an interval: with q = (a1 x)^2 +
+// (b1 x + b2 y)^2 and n = a1^2 + b1^2, the rightmost point of q <= t lies at
+// y = kx r / a1 (r^2 = t, kx = -b1 / b2); clamped to the band as y = Y its row
+// ends at x = ky Y + sqrt((t - (a1 b2 Y)^2 / n) / n) (ky = -b1 b2 / n), and the
+// left end is the mirror image.  With t = tau + margin and the interval
+// widened by `slack` no tile outside it can pass the test; with t = tau -
+// margin and the interval narrowed every tile that it meets does; the few
+// between (about 0.1 % of a cell's tiles) are tested.  margin covers the FP32
+// error of q, whose terms are up to |b1| / a1 times larger than tau, in the test
+// and here; slack that of the coordinates and of the interval's terms.  Records
+// outside the bounds for which that holds (or not finite) have all tiles
+// tested.  A row costs about 45 instructions instead of up to 8 tests of 40.
 __device__ __forceinline__ uint64_t cell_mask(float u, float v, float a1, float b1, float b2, float kx, float ky,
                                               float tau, const RasterView &V, int tx0, int tx1, int ty0, int ty1) {
   const float T = (float)V.tile, iT = 1.0f / T;
   const float xmax = (float)V.width - 0.5f - u, ymax = (float)V.height - 0.5f - v;  // last pixel centre
   const uint32_t cols = (((1u << (tx1 - tx0)) - 1u) << (tx0 & (kCellEdge - 1)));
-  uint64_t mask = 0ull;
-  // all corners inside: the whole (convex) box is
-  const float lx = (float)tx0 * T + 0.5f - u, hx = fminf((float)tx1 * T - 0.5f - u, xmax);
-  const float by0 = (float)ty0 * T + 0.5f - v, by1 = fminf((float)ty1 * T - 0.5f - v, ymax);
-  if (sum_sq(a1, b1, b2, lx, by0) <= tau && sum_sq(a1, b1, b2, hx, by0) <= tau &&
-      sum_sq(a1, b1, b2, lx, by1) <= tau && sum_sq(a1, b1, b2, hx, by1) <= tau) {
-    for (int ty = ty0; ty < ty1; ++ty) mask |= (uint64_t)cols << ((ty & (kCellEdge - 1)) * kCellEdge);
-    return mask;
+  const float aspect = __fdividef(fabsf(b1), a1), ab = a1 * b2;
+  const float margin = 2e-5f + 2e-6f * tau * (1.0f + aspect);
+  const float t = tau + margin;
+  const float n = __fmaf_rn(a1, a1, b1 * b1);
+  const bool ok = tau >= 0.0f && t < 1e9f && a1 > 1e-12f && b2 > 1e-12f && b2 < 1e9f && ab > 1e-18f &&
+                  aspect < 1e6f && n < 1e18f && fabsf(u) < 1e9f && fabsf(v) < 1e9f;
+  uint64_t sure = 0ull, maybe = 0ull;
+  if (ok) {
+    // all corners inside: the whole (convex) box is
+    const float lx = (float)tx0 * T + 0.5f - u, hx = fminf((float)tx1 * T - 0.5f - u, xmax);
+    const float by0 = (float)ty0 * T + 0.5f - v, by1 = fminf((float)ty1 * T - 0.5f - v, ymax);
+    const float tin = tau - margin;
+    if (sum_sq(a1, b1, b2, lx, by0) <= tin && sum_sq(a1, b1, b2, hx, by0) <= tin &&
+        sum_sq(a1, b1, b2, lx, by1) <= tin && sum_sq(a1, b1, b2, hx, by1) <= tin) {
+      for (int ty = ty0; ty < ty1; ++ty) sure |= (uint64_t)cols << ((ty & (kCellEdge - 1)) * kCellEdge);
+      return sure;
+    }
+    const float in = __fdividef(1.0f, n), r = sqrt_approx(t);
+    const float ym = kx * __fdividef(r, a1);  // y of the rightmost point
+    const float slack = 2e-7f * (fabsf(u) + fabsf(v) + (float)V.width + (float)V.height);
+    const float ry = __fdividef(r * sqrt_approx(n), ab) * 1.00001f + slack;  // vertical half-extent
+    const float c2 = ab * ab * in;
+    // tile columns that [l, h] meets
+    auto columns = [&](float l, float h) -> uint32_t {
+      const float flo = ceilf((l + u - (T - 0.5f)) * iT), fhi = floorf((h + u - 0.5f) * iT);
+      const int lo = (int)fmaxf(flo, (float)tx0), hi = (int)fminf(fhi, (float)(tx1 - 1));
+      if (l > xmax || lo > hi || lo >= tx1 || hi < tx0) return 0u;
+      return (((2u << (hi - lo)) - 1u) << (lo & (kCellEdge - 1))) & cols;
+    };
+    for (int ty = ty0; ty < ty1; ++ty) {
+      const float ly = (float)ty * T + 0.5f - v, hy = fminf((float)ty * T + (T - 0.5f) - v, ymax);
+      if (ly > ry || hy < -ry) continue;
+      // right end: the rightmost point's y clamped to the band; left end: its mirror's
+      const float yr = fminf(fmaxf(ym, ly), hy), yl = fminf(fmaxf(-ym, ly), hy);
+      const float kr = ky * yr, kl = ky * yl;
+      const float dr = __fmaf_rn(-c2 * yr, yr, t), dl = __fmaf_rn(-c2 * yl, yl, t);
+      const float xr = kr + sqrt_approx(fmaxf(dr, 0.0f) * in), xl = kl - sqrt_approx(fmaxf(dl, 0.0f) * in);
+      const float er = slack + 4e-6f * (fabsf(kr) + fabsf(xr)), el = slack + 4e-6f * (fabsf(kl) + fabsf(xl));
+      const uint32_t outer = columns(xl - el, xr + er);
+      const float ir = dr - 2.0f * margin, il = dl - 2.0f * margin;
+      const float xri = kr + sqrt_approx(fmaxf(ir, 0.0f) * in) - er, xli = kl - sqrt_approx(fmaxf(il, 0.0f) * in) + el;
+      const uint32_t inner = ir >= 0.0f && il >= 0.0f && xli <= xri ? columns(xli, xri) & outer : 0u;
+      const int row = (ty & (kCellEdge - 1)) * kCellEdge;
+      sure |= (uint64_t)inner << row;
+      maybe |= (uint64_t)(outer & ~inner) << row;
+    }
+  } else {
+    for (int ty = ty0; ty < ty1; ++ty) maybe |= (uint64_t)cols << ((ty & (kCellEdge - 1)) * kCellEdge);
   }
-  const float t = tau + 1e-3f;
-  const float n = a1 * a1 + b1 * b1, in = 1.0f / n;
-  const float r = sqrtf(t);
-  const float xm = r / a1, ym = kx * xm;             // rightmost point
-  const float ry = r * sqrtf(n) / (a1 * b2) * 1.00001f + 0.03f;  // vertical half-extent
-  const float c2 = (a1 * b2) * (a1 * b2) * in;
-  for (int ty = ty0; ty < ty1; ++ty) {
-    const float ly = (float)ty * T + 0.5f - v, hy = fminf((float)ty * T + (T - 0.5f) - v, ymax);
-    if (ly > ry || hy < -ry) continue;
-    // right end: the rightmost point's y clamped to the band; left end: its mirror's
-    const float yr = fminf(fmaxf(ym, ly), hy), yl = fminf(fmaxf(-ym, ly), hy);
-    const float kr = ky * yr, kl = ky * yl;
-    float xr = yr == ym ? xm : kr + sqrtf(fmaxf(t - c2 * yr * yr, 0.0f) * in);
-    float xl = yl == -ym ? -xm : kl - sqrtf(fmaxf(t - c2 * yl * yl, 0.0f) * in);
-    xr += 0.03f + 1e-5f * (fabsf(kr) + fabsf(xr));
-    xl -= 0.03f + 1e-5f * (fabsf(kl) + fabsf(xl));
-    if (xl > xmax) continue;
-    const float flo = ceilf((xl + u - (T - 0.5f)) * iT), fhi = floorf((xr + u - 0.5f) * iT);
-    const int lo = (int)fmaxf(flo, (float)tx0), hi = (int)fminf(fhi, (float)(tx1 - 1));
-    if (lo > hi || lo >= tx1 || hi < tx0) continue;
-    const uint32_t bits = ((2u << (hi - lo)) - 1u) << (lo & (kCellEdge - 1));
-    mask |= (uint64_t)(bits & cols) << ((ty & (kCellEdge - 1)) * kCellEdge);
+  while (maybe) {
+    const int bit = __ffsll((long long)maybe) - 1;
+    maybe &= maybe - 1ull;
+    const int tx = (tx0 & ~(kCellEdge - 1)) + (bit & (kCellEdge - 1)), ty = (ty0 & ~(kCellEdge - 1)) + (bit >> kCellShift);
+    if (tile_meets(u, v, a1, b1, b2, kx, ky, tau, V, tx, ty)) sure |= 1ull << bit;
   }
-  return mask;
+  return sure;
 }
 
 // The tiles of all slots' rects: the instances that a call whose pairs

@@ -384,6 +384,16 @@ __device__ __forceinline__ bool ellipse_meets_box(float u, float v, float a1, fl
   return m <= tau;
 }
 
+// ellipse_meets_box for a tile's box of pixel centres.
+__device__ __forceinline__ bool tile_meets(float u, float v, float a1, float b1, float b2, float kx, float ky,
+                                           float tau, const RasterView &V, int tx, int ty) {
+  const int T = V.tile;
+  const float bx0 = (float)(tx * T) + 0.5f, by0 = (float)(ty * T) + 0.5f;
+  const float bx1 = (float)min(tx * T + T - 1, V.width - 1) + 0.5f;
+  const float by1 = (float)min(ty * T + T - 1, V.height - 1) + 0.5f;
+  return ellipse_meets_box(u, v, a1, b1, b2, kx, ky, tau, bx0, bx1, by0, by1);
+}
+
 struct EmitArgs {
   const uint32_t *sorted_slots;
   const int4 *meta;
@@ -654,12 +664,7 @@ __device__ __forceinline__ void walk_next(const EmitArgs &A, const EmitChunkSmem
 
 template <int MAXV>
 __device__ __forceinline__ bool walk_keep(const RasterViews<MAXV> &rv, const PairWalk &w) {
-  const RasterView &V = rv.v[MAXV == 1 ? 0 : w.view];
-  const int T = V.tile;
-  const float bx0 = (float)(w.tx * T) + 0.5f, by0 = (float)(w.ty * T) + 0.5f;
-  const float bx1 = (float)min(w.tx * T + T - 1, V.width - 1) + 0.5f;
-  const float by1 = (float)min(w.ty * T + T - 1, V.height - 1) + 0.5f;
-  return ellipse_meets_box(w.u, w.v, w.a1, w.b1, w.b2, w.kx, w.ky, w.tau, bx0, bx1, by0, by1);
+  return tile_meets(w.u, w.v, w.a1, w.b1, w.b2, w.kx, w.ky, w.tau, rv.v[MAXV == 1 ? 0 : w.view], w.tx, w.ty);
 }
 
 template <int MAXV>

@@ -142,3 +142,61 @@ def test_pair_overflow_reports_a_need_that_fits(n, cap):
     np.testing.assert_array_equal(tiles, (keys >> np.uint64(32)).astype(np.int64))
     np.testing.assert_array_equal(slots, vals)
     np.testing.assert_array_equal(gr, ranges)
+
+
+def _stretched(rec, rng, lo, hi):
+    """Ellipses of widths lo..hi along one axis and 0.55..hi along the other."""
+    n = rec["rect"].shape[0]
+    ang = rng.uniform(0, np.pi, n)
+    ang[::9] = rng.integers(0, 4, ang[::9].size) * (np.pi / 4)
+    s1 = np.exp(rng.uniform(np.log(lo), np.log(hi), n))
+    s2 = np.exp(rng.uniform(np.log(0.55), np.log(hi), n))
+    c, s, k = np.cos(ang), np.sin(ang), 0.5 * np.log2(np.e)
+    rec["conic2"] = np.stack([k * (c * c / s1 ** 2 + s * s / s2 ** 2), k * 2 * c * s * (1 / s1 ** 2 - 1 / s2 ** 2),
+                              k * (s * s / s1 ** 2 + c * c / s2 ** 2)], 1)
+
+
+# round and elongated ellipses of many sizes, on both tile edges; needles (their q is a difference of terms 1e4
+# times as large); centres on pixel centres
+@pytest.mark.parametrize("tile,W,H,lo,hi", [(16, 723, 597, 0.55, 30.0), (8, 363, 301, 0.55, 30.0),
+                                            (16, 1352, 1014, 20.0, 500.0), (16, 1280, 720, 1e3, 1e5),
+                                            (8, 640, 480, 100.0, 1e4)])
+def test_lists_equal_the_instance_sorts(tile, W, H, lo, hi):
+    """The same list, counts and ranges by both routes (visible capacity below
+    and above 65,536), at a capacity of exactly the instances."""
+    n, ntiles = 30_000, ((W + tile - 1) // tile) * ((H + tile - 1) // tile)
+    rng = np.random.default_rng(W + tile)
+    rec = _synthetic_records(rng, n, W, H, 24, tile=tile)
+    _stretched(rec, rng, lo, hi)
+    rec["uv"][::5] = np.floor(rec["uv"][::5]) + np.float32(0.5)
+    views = [sy.tiny_view(W, H)]
+    a, (code, want) = _run(rec, views, tile, 1 << 23, vis_cap=n)
+    assert code == fgs4d.OK and want[1] > n
+    b, (code, got) = _run(rec, views, tile, want[1])
+    assert code == fgs4d.OK and got == want
+    for x, y in zip(_lists(a, want, ntiles), _lists(b, got, ntiles)):
+        np.testing.assert_array_equal(x, y)
+
+
+@pytest.mark.parametrize("stage_blocks", [0, 1])
+def test_pairs_beyond_the_capacity_whose_masks_are_empty(stage_blocks):
+    """Circles of radius 4 px centred (3, 3) px from the corner of four cells:
+    four candidate pairs, three with a tile.  At a capacity of exactly the
+    instances (fewer than the candidates) the pairs are compacted."""
+    n, W, H = 16_384, 640, 512
+    rng = np.random.default_rng(9)
+    rec = _synthetic_records(rng, n, W, H, 2)
+    cx, cy = rng.integers(1, 5, n) * 128.0, rng.integers(1, 4, n) * 128.0
+    sx, sy_ = rng.choice([-1.0, 1.0], n), rng.choice([-1.0, 1.0], n)
+    rec["uv"] = np.stack([cx + 3 * sx, cy + 3 * sy_], 1).astype(np.float32)
+    rec["rect"] = np.stack([cx / 16 - 1, cy / 16 - 1, cx / 16 + 1, cy / 16 + 1], 1).astype(np.int32)
+    rec["tau"][:] = 8.0
+    k = 8.0 / 4.0 ** 2
+    rec["conic2"] = np.tile(np.float32([k, 0.0, k]), (n, 1))
+    views, ntiles = [sy.tiny_view(W, H)], 40 * 32
+    a, (code, want) = _run(rec, views, 16, 1 << 20, vis_cap=n)
+    assert code == fgs4d.OK and want[1] == 3 * n  # of the 4 n candidate pairs
+    b, (code, got) = _run(rec, views, 16, want[1], stage_blocks=stage_blocks)
+    assert code == fgs4d.OK and got == want
+    for x, y in zip(_lists(a, want, ntiles), _lists(b, got, ntiles)):
+        np.testing.assert_array_equal(x, y)
