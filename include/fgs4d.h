@@ -209,8 +209,8 @@ int fgs4d_bin_sort(int64_t n, const fgs4d_view *views, int32_t nviews, const fgs
                    void *workspace, size_t workspace_bytes, void *stream);
 
 /* Diagnostic: *count_out = the number of kernels fgs4d_preprocess launches for
- * these arguments (two where the records pass through a staging area, which
- * lies over the instance buffers that fgs4d_bin_sort fills afterwards).
+ * these arguments (two where the records pass through a staging area in scratch
+ * of fgs4d_bin_sort; results of earlier calls other than its own stay).
  * Launches nothing; has no counterpart in the paper. */
 int fgs4d_preprocess_kernels(int64_t n, const fgs4d_view *views, int32_t nviews, const fgs4d_settings *settings,
                              int32_t *count_out);

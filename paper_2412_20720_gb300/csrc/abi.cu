@@ -151,44 +151,53 @@ int compute_layout(const fgs4d_settings *s, int64_t n, const fgs4d_view *views, 
   L.hist_tile = take(kMaxPasses * kRadixBins * sizeof(uint32_t));
   L.lb_emit = take((size_t)L.emit_blocks * sizeof(uint64_t));
   L.control_end = off;
-  L.lb_chunk = take((size_t)L.chunk_cap * sizeof(uint64_t));
-  L.pair_prefix = take(((size_t)L.vis_cap + 1) * sizeof(uint32_t));
-  L.emit_rec = take((size_t)L.vis_cap * 48);
-  L.rec_aux = take((size_t)L.vis_cap * sizeof(float4));
-  L.block_first = take((size_t)L.pre_blocks * sizeof(uint32_t));
-  L.chunk_first = take((size_t)L.chunk_cap * sizeof(uint32_t));
   const size_t vc = (size_t)L.vis_cap, ic = (size_t)L.inst_cap;
+  // Results that later calls read.
+  const int fin = L.tile_passes & 1;           // instance buffers that hold the sorted list
+  const int dfin = (L.depth_passes - 1) & 1;   // and the depth-sorted slots
   L.rec_geom = take(vc * 16);
   L.rec_color = take(vc * 16);
   L.rec_blue = take(vc * 4);
   L.rec_tau = take(vc * 4);
   L.rec_meta = take(vc * 16);
+  L.rec_aux = take(vc * sizeof(float4));
   L.depth_key = take(vc * 4);
-  for (int k = 0; k < 2; ++k) {
-    L.dsort_key[k] = take(vc * 4);
-    L.dsort_val[k] = take(vc * 4);
-  }
-  L.depth_state = take((size_t)L.depth_passes * L.depth_blocks * kRadixBins * sizeof(uint32_t));
-  for (int k = 0; k < 2; ++k) {
-    L.inst_key[k] = take(ic * 4);
-    L.inst_val[k] = take(ic * 4);
-  }
-  if (L.cells) {
-    L.cell_slot = take(ic * 4);
-    L.cell_mask = take(ic * 8);
-  }
-  L.pre_stage = L.inst_key[0];
-  L.pre_staged = L.pre_blocks >= kPreStagedMinBlocks &&
-                 off - L.pre_stage >= (size_t)L.pre_blocks * (kPreBlock * kPreStageBytes + sizeof(uint32_t));
-  L.tile_state = take((size_t)L.tile_passes * L.tile_blocks * kRadixBins * sizeof(uint32_t));
-  if (L.cells) {
-    L.cell_ranges = take((size_t)L.total_cells * 8);
-    L.cell_rows = take((size_t)(segs + L.total_cells) * 64 * 4);
-  }
+  L.block_first = take((size_t)L.pre_blocks * sizeof(uint32_t));
+  L.dsort_val[dfin] = take(vc * 4);
   L.ranges = take((size_t)L.total_tiles * 8);
   L.pix_T = take((size_t)L.total_pixels * 4);
   L.pix_last = take((size_t)L.total_pixels * 4);
   L.slot_grad = take(vc * kSlotGradFloats * sizeof(float));
+  L.inst_key[fin] = take(ic * 4);
+  L.inst_val[fin] = take(ic * 4);
+  // Scratch of bin_sort, free between its calls: preprocess stages its records
+  // here, so that it leaves all results but its own as they are.
+  L.pre_stage = off;
+  L.inst_key[fin ^ 1] = take(ic * 4);
+  L.inst_val[fin ^ 1] = take(ic * 4);
+  if (L.cells) {
+    L.cell_slot = take(ic * 4);
+    L.cell_mask = take(ic * 8);
+  }
+  L.tile_state = take((size_t)L.tile_passes * L.tile_blocks * kRadixBins * sizeof(uint32_t));
+  if (L.cells) {
+    L.cell_ranges = take(((size_t)L.total_cells << kCellRangeShift) * 8);
+    L.cell_rows = take((size_t)(segs + L.total_cells) * 64 * 4);
+  }
+  L.lb_chunk = take((size_t)L.chunk_cap * sizeof(uint64_t));
+  L.pair_prefix = take((vc + 1) * sizeof(uint32_t));
+  L.emit_rec = take(vc * 48);
+  L.chunk_first = take((size_t)L.chunk_cap * sizeof(uint32_t));
+  L.dsort_key[0] = take(vc * 4);
+  L.dsort_key[1] = take(vc * 4);
+  L.dsort_val[dfin ^ 1] = take(vc * 4);
+  L.depth_state = take((size_t)L.depth_passes * L.depth_blocks * kRadixBins * sizeof(uint32_t));
+  // Staged where the instance buffers are at least as large as the staging
+  // area: the workspace then grows by a part of them at most.
+  const size_t stage = (size_t)L.pre_blocks * (kPreBlock * kPreStageBytes + sizeof(uint32_t));
+  const size_t inst_bytes = 4 * align_up(ic * 4) + (L.cells ? align_up(ic * 4) + align_up(ic * 8) : 0);
+  L.pre_staged = L.pre_blocks >= kPreStagedMinBlocks && inst_bytes >= stage;
+  if (L.pre_staged) off = std::max(off, align_up(L.pre_stage + stage));
   L.total = off;
   *out = L;
   return FGS4D_OK;

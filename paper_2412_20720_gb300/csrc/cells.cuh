@@ -33,7 +33,7 @@ struct CellArgs {
   uint2 *mask;           // tile mask per pair, in depth order (low word: tile rows 0-3)
   const uint32_t *skey;  // sorted cell ids
   const uint32_t *sidx;  // sorted pairs (indices into slot and mask)
-  uint2 *cell_ranges;    // [start, end) of each cell's sorted pairs
+  uint2 *cell_ranges;    // [start, end) of each cell's sorted pairs (entry c << kCellRangeShift)
   uint32_t *rows;        // instances per tile of each (segment, cell) run; after cell_prefix their exclusive prefix
 };
 
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kCellChunk) cell_emit_kernel(CellArgs C, Raste
   const EmitArgs &A = C.e;
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < C.total_cells;
        r += (int64_t)gridDim.x * blockDim.x)
-    C.cell_ranges[r] = make_uint2(0xffffffffu, 0u);
+    C.cell_ranges[r << kCellRangeShift] = make_uint2(0xffffffffu, 0u);
   const int64_t nvis = min64((int64_t)A.counters[kCtrVisible], A.vis_cap);
   const uint32_t npairs = A.counters[kCtrPairs];
   const uint32_t nchunks = (uint32_t)min64(((int64_t)npairs + kCellChunk - 1) / kCellChunk, A.chunk_cap);
@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(kCellPrefixThreads) cell_prefix_kernel(CellArg
   const int64_t npairs = min64((int64_t)A.counters[kCtrCellPairs], A.inst_cap);
   const int t = threadIdx.x & (kCellTiles - 1), g = threadIdx.x / kCellTiles;
   for (int32_t c = blockIdx.x; c < C.total_cells; c += gridDim.x) {
-    const uint2 r = C.cell_ranges[c];
+    const uint2 r = C.cell_ranges[(int64_t)c << kCellRangeShift];
     int64_t s0 = 0, s1 = 0;  // rows [s0, s1) of the cell
     if (r.x < r.y && (int64_t)r.y <= npairs) {
       s0 = (int64_t)(r.x / kCellSeg) + c;

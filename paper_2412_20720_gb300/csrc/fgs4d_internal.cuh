@@ -35,6 +35,11 @@ constexpr int kCellChunk = 256;          // candidate (slot, cell) pairs per emi
 constexpr int kCellSeg = 256;            // sorted pairs per segment, one per thread
 constexpr int kCellBlock = kCellSeg;     // threads of the count and write kernels: one warp per row of a cell's tiles
 constexpr int kCellPrefixThreads = 512;
+// A cell's range has a 128-byte line of its own: the cell sort's blocks update
+// the ranges by atomics, and eight or sixteen cells a line cost 75 or 105 us a
+// pass by the array's offset (135 cells, 115M instances; bin_sort 654 or 680,
+// now 627).
+constexpr int kCellRangeShift = 4;
 // Two-level binning is taken from these visible capacities on (in all, and per
 // cell): it launches three more kernels than the instance sort and works a
 // cell's list at a time.  bin_sort (us) instance sort / two-level, at 1352x1014
@@ -160,7 +165,7 @@ struct Layout {
   int32_t emit_grid;      // persistent emission blocks
   int32_t pre_grid;       // persistent preprocess blocks
   // Preprocess through a staging area (see preprocess_kernel): it lies over
-  // the instance buffers, which bin_sort fills afterwards.
+  // scratch that only bin_sort uses, and only during its call.
   bool pre_staged;
   size_t pre_stage;
   int32_t pre_compact_grid;

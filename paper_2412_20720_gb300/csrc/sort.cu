@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(kSortThreads) radix_pass_kernel(
     const uint32_t *__restrict__ keys_in, const uint32_t *__restrict__ vals_in, uint32_t *__restrict__ keys_out,
     uint32_t *__restrict__ vals_out, const uint32_t *__restrict__ count_ptr, int64_t cap, int32_t shift,
     const uint32_t *__restrict__ hist, uint32_t *state, uint32_t *ticket, uint32_t *status, uint2 *ranges,
-    int64_t total_tiles, int64_t small, uint32_t *__restrict__ small_out) {
+    int64_t total_tiles, int64_t small, uint32_t *__restrict__ small_out, int32_t range_shift) {
   static_assert(kItems % 4 == 0, "whole 16-byte copies per warp segment");
   grid_dependency_sync();
   constexpr int kTileKeys = kSortThreads * kItems;
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(kSortThreads) radix_pass_kernel(
         vals_out[gpos] = S.vals[p];
         if (ranges) {
           if ((int64_t)kk < total_tiles) {
-            uint32_t *r = reinterpret_cast<uint32_t *>(&ranges[kk]);
+            uint32_t *r = reinterpret_cast<uint32_t *>(&ranges[(int64_t)kk << range_shift]);
             if (p == 0 || S.keys[p - 1] != kk) atomicMin(&r[0], gpos);
             if (p == nvalid - 1 || S.keys[p + 1] != kk) atomicMax(&r[1], gpos + 1u);
           } else {
@@ -843,7 +843,7 @@ cudaError_t bin_cells(const Layout &L, const EmitArgs &ea_in, const RasterViews<
                         (const uint32_t *)(ea.hist_tile + p * kRadixBins),
                         ea.tile_state + (size_t)p * L.tile_blocks * kRadixBins, ctr + kCtrTicketTile + p,
                         ctr + kCtrStatus, p == P - 1 ? C.cell_ranges : (uint2 *)nullptr, (int64_t)L.total_cells,
-                        (int64_t)-1, (uint32_t *)nullptr);
+                        (int64_t)-1, (uint32_t *)nullptr, (int32_t)kCellRangeShift);
     if (e != cudaSuccess) return e;
   }
   e = launch_pdl(cell_count_kernel, (unsigned)L.cell_grid, kCellBlock, st, C);
@@ -879,7 +879,7 @@ cudaError_t depth_sort(const Layout &L, unsigned char *ws, uint32_t *sorted, cud
                         (const uint32_t *)(ctr + kCtrVisible), (int64_t)L.vis_cap, (int32_t)(kRadixBits * p),
                         (const uint32_t *)(hist + p * kRadixBins), dstate + (size_t)p * L.depth_blocks * kRadixBins,
                         ctr + kCtrTicketDepth + p, ctr + kCtrStatus, (uint2 *)nullptr, (int64_t)0, kRankSortMax,
-                        p == 0 ? sorted : (uint32_t *)nullptr);
+                        p == 0 ? sorted : (uint32_t *)nullptr, (int32_t)0);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -953,7 +953,7 @@ cudaError_t bin_sort_typed(const Layout &L, const fgs4d_view *views, int32_t nvi
                         (const uint32_t *)iv[in], ik[out], iv[out], (const uint32_t *)(ctr + kCtrInstances),
                         (int64_t)L.inst_cap, (int32_t)(kRadixBits * p), (const uint32_t *)(hist_t + p * kRadixBins),
                         state, ctr + kCtrTicketTile + p, status, last ? ranges : (uint2 *)nullptr,
-                        (int64_t)L.total_tiles, (int64_t)-1, (uint32_t *)nullptr);
+                        (int64_t)L.total_tiles, (int64_t)-1, (uint32_t *)nullptr, (int32_t)0);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -1106,11 +1106,11 @@ extern "C" int fgs4d_sort_depth_static(const uint32_t *depth_keys, int64_t n, ui
     if (p == 0)
       radix_pass_kernel<true, kSortItems><<<blocks, kSortThreads, smem, st>>>(kin, nullptr, s->keys[out], vout, &s->ctl[0],
                                                                FGS4D_STATIC_SORT_MAX, kRadixBits * p, s->hist[p],
-                                                               &s->state[p][0][0], &s->ctl[8 + p], &s->ctl[1], nullptr, 0, -1, nullptr);
+                                                               &s->state[p][0][0], &s->ctl[8 + p], &s->ctl[1], nullptr, 0, -1, nullptr, 0);
     else
       radix_pass_kernel<false, kSortItems><<<blocks, kSortThreads, smem, st>>>(kin, s->vals[in], s->keys[out], vout, &s->ctl[0],
                                                                 FGS4D_STATIC_SORT_MAX, kRadixBits * p, s->hist[p],
-                                                                &s->state[p][0][0], &s->ctl[8 + p], &s->ctl[1], nullptr, 0, -1, nullptr);
+                                                                &s->state[p][0][0], &s->ctl[8 + p], &s->ctl[1], nullptr, 0, -1, nullptr, 0);
   }
   return cudaGetLastError() == cudaSuccess ? FGS4D_OK : FGS4D_ERR_CUDA;
 }

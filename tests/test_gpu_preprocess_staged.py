@@ -34,3 +34,23 @@ def test_same_records_as_with_the_look_back(n, nviews, stage_blocks, vis_cap):
     assert got[0][0][0] > 10_000
     for a, b in zip(*got):
         np.testing.assert_array_equal(a, b)
+
+
+# one view and several; capacities that stage the records (two kernels)
+@pytest.mark.parametrize("n,nviews,inst_cap", [(155_648, 1, 1 << 20), (60_001, 3, 1 << 20)])
+def test_a_second_preprocess_keeps_the_lists(n, nviews, inst_cap):
+    """Preprocess with other colours leaves the sorted lists in place: the
+    compositor then gives the image of a whole render with them."""
+    import torch
+    params = to_device(sy.make_scene(n, 31, (-2, -2, -2), (2, 2, 2), sh_degree=1, t_order=1).as_dict())
+    views = [sy.tiny_view(400, 300, t=0.2 + 0.3 * k) for k in range(nviews)]
+    r = Renderer(n, views, RenderConfig(sh_degree=1, t_order=1, inst_capacity=inst_cap))
+    assert fgs4d.preprocess_kernels(n, r.views, r.nviews, r.settings) == 2
+    other = dict(params, sh=params["sh"].flip(0).contiguous())
+    want = r.forward(other).clone()
+    first = r.forward(params).clone()
+    ws = r.ws.data_ptr()
+    fgs4d.preprocess(r.gaussians(other), r.views, r.nviews, r.settings, ws, r.ws_bytes, r.stream())
+    got = torch.empty_like(want)
+    fgs4d.render_fwd(n, r.views, r.nviews, r.settings, ws, r.ws_bytes, got.data_ptr(), None, r.stream())
+    assert not torch.equal(first, want) and torch.equal(got, want)
