@@ -131,6 +131,8 @@ int compute_layout(const fgs4d_settings *s, int64_t n, const fgs4d_view *views, 
   L.pre_grid = k ? std::min(L.pre_blocks, 152 * k) : L.pre_blocks;
   L.pre_compact_grid = 152 * (k ? 2 * k : 8);
   L.sort_grid = 152 * (k ? k : 4);
+  L.tile_sort_sub = s->inst_capacity >= kWideTileSortMinCap ? 3 : 1;
+  L.tile_sort_grid = 152 * (k ? std::min(k, 3) : 3);
   const int64_t segs = (L.inst_cap + kCellSeg - 1) / kCellSeg;
   L.cell_grid = (int32_t)std::min<int64_t>(segs, 152 * (k ? 2 * k : 8));
   L.emit_grid = std::max(1, std::min(L.chunk_cap, 152 * (k ? 2 * k : 8)));

@@ -30,6 +30,11 @@ constexpr int kDepthSortItems = 4, kDepthSortItemsLarge = 8;
 constexpr int64_t kDepthSortLargeMin = int64_t(1) << 20;
 constexpr int kInstSortItems = 8;   // keys per thread per radix block of the instance (tile-id) sort
 constexpr int kInstSortTile = kSortThreads * kInstSortItems;
+// Instance capacity from which the instance sort takes three sub-tiles per
+// ticket (a third of the look-backs, fewer resident blocks); calls of few
+// Gaussians that span many tiles reach it, the others take the two-level
+// binning.
+constexpr int64_t kWideTileSortMinCap = int64_t(1) << 26;
 // Two-level binning (cells.cuh).
 constexpr int kCellChunk = 256;          // candidate (slot, cell) pairs per emission chunk, one per thread
 constexpr int kCellSeg = 256;            // sorted pairs per segment, one per thread
@@ -170,6 +175,8 @@ struct Layout {
   size_t pre_stage;
   int32_t pre_compact_grid;
   int32_t sort_grid;      // persistent radix-pass blocks (at most; one radix tile each at least)
+  int32_t tile_sort_sub;  // sub-tiles of kInstSortTile keys per ticket of the instance sort (1 or 3)
+  int32_t tile_sort_grid; // persistent instance-sort blocks with 3 sub-tiles per ticket
   bool cells;             // two-level binning (cells.cuh) instead of the instance sort
   int32_t total_cells, cell_passes;
   int32_t cell_grid;      // persistent count / write blocks

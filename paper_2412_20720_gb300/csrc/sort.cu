@@ -129,9 +129,12 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem, int src
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gmem), "r"(src_bytes) : "memory");
 }
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
-  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+// Waits until at most n (0..2) of this thread's copy groups are pending.
+__device__ __forceinline__ void cp_async_wait_pending(int n) {
+  if (n <= 0) asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  else if (n == 1) asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+  else asm volatile("cp.async.wait_group 2;\n" ::: "memory");
 }
 
 // Stable order of few keys by counting: key i goes to place #{j : key_j <
@@ -179,57 +182,65 @@ __device__ __forceinline__ void rank_sort(const uint32_t *__restrict__ keys, int
 }
 
 // Shared memory of one radix block: the ticket's keys and values (input,
-// then the block-local order), per-warp digit counts, the digits' block-local
-// and global starts.
-template <int kItems>
+// then the block-local order), per-warp digit counts (two sets, alternating
+// between sub-tiles), per-sub-tile digit starts and the digits' global
+// starts.
+template <int kItems, int kSub = 1>
 struct RadixSmem {
-  uint32_t keys[kSortThreads * kItems];
-  uint32_t vals[kSortThreads * kItems];
-  uint32_t wcount[kSortThreads / 32][kRadixBins];
-  uint32_t bstart[kRadixBins];  // first block-local position of each digit
-  uint32_t gstart[kRadixBins];  // global position of the ticket's first key of each digit
+  uint32_t keys[kSortThreads * kItems * kSub];
+  uint32_t vals[kSortThreads * kItems * kSub];
+  uint32_t wcount[kSub > 1 ? 2 : 1][kSortThreads / 32][kRadixBins];
+  uint32_t bstart[kSub][kRadixBins];  // first block-local position of each digit in sub-tile s
+  uint32_t sbase[kSub][kRadixBins];   // keys of each digit in the sub-tiles before s
+  uint32_t gstart[kRadixBins];        // global position of the ticket's first key of each digit
   uint32_t scan[12];
   uint32_t ticket;
   uint32_t scan_ranks[kSortThreads / 32][32];  // rank_sort: each warp's counts
 };
-template <int kItems>
+template <int kItems, int kSub = 1>
 constexpr size_t radix_smem_bytes() {
-  return sizeof(RadixSmem<kItems>);
+  return sizeof(RadixSmem<kItems, kSub>);
 }
 
 // One stable 8-bit LSD pass.  A block takes tickets in launch order; a
-// ticket is kSortThreads x kItems consecutive keys.  Each warp copies the
-// keys (and values) it ranks into shared memory with cp.async (16-byte
-// copies: keys_in and vals_in start on 16-byte boundaries, as the
-// workspace's arrays do).  Ranking is stable within a warp's segment
-// (item-major, lane-minor): the lanes holding the same digit are found by
-// nine ballots (eight digit bits and the padding bit), and the lowest of them
-// adds the group's size to the warp's count of that digit.  The ticket is
-// then placed in block-local digit order, a decoupled look-back gives its
-// global start of each digit, and the scatter writes each digit's run.  Small
-// sorts (the depth sort) take short tickets, so that more SMs share a pass.
+// ticket is kSub consecutive sub-tiles of kSortThreads x kItems keys.  Each
+// warp copies the keys (and values) it ranks into shared memory with
+// cp.async, one copy group per sub-tile, so later sub-tiles arrive while the
+// first is ranked (16-byte copies: keys_in and vals_in start on 16-byte
+// boundaries, as the workspace's arrays do).  Ranking is stable within a
+// warp's segment (item-major, lane-minor): the lanes holding the same digit
+// are found by nine ballots (eight digit bits and the padding bit), and the
+// lowest of them adds the group's size to the warp's count of that digit.
+// Each sub-tile is then placed in block-local digit order in its own part of
+// the buffer.  One decoupled look-back per ticket gives the ticket's global
+// start of each digit, and the scatter writes each sub-tile's digit runs.
+// Small sorts (the depth sort) take short sub-tiles, so that more SMs share a
+// pass; very large instance sorts take three sub-tiles per ticket, a third of
+// the look-backs per key (kWideTileSortMinCap).
 //
 // With `ranges` (the last pass of the tile or cell sort, keys = tile or cell
 // ids below total_tiles) the pass also records each id's [start, end) in the
-// sorted list.  A ticket's staged keys are ordered by the full key (the
+// sorted list.  A sub-tile's staged keys are ordered by the full key (the
 // pass input is ordered by the lower digits and the staging is stable), so
-// the equal keys of a ticket form one run; its first and last output
+// the equal keys of a sub-tile form one run; its first and last output
 // positions go to atomicMin on start and atomicMax on end, which the
 // emission initialised to (0xffffffff, 0).  An id with no key keeps
 // start > end, which every reader takes as empty.
-template <bool kValsAreIndex, int kItems>
+template <bool kValsAreIndex, int kItems, int kSub = 1>
 __global__ void __launch_bounds__(kSortThreads) radix_pass_kernel(
     const uint32_t *__restrict__ keys_in, const uint32_t *__restrict__ vals_in, uint32_t *__restrict__ keys_out,
     uint32_t *__restrict__ vals_out, const uint32_t *__restrict__ count_ptr, int64_t cap, int32_t shift,
     const uint32_t *__restrict__ hist, uint32_t *state, uint32_t *ticket, uint32_t *status, uint2 *ranges,
     int64_t total_tiles, int64_t small, uint32_t *__restrict__ small_out, int32_t range_shift) {
+  static_assert(kSub >= 1 && kSub <= 3, "copy groups are waited for by count (at most 2 pending)");
   static_assert(kItems % 4 == 0, "whole 16-byte copies per warp segment");
   grid_dependency_sync();
-  constexpr int kTileKeys = kSortThreads * kItems;
+  constexpr int kSubKeys = kSortThreads * kItems;
+  constexpr int kTileKeys = kSubKeys * kSub;
   constexpr int kWarps = kSortThreads / 32;
-  constexpr int kSegKeys = 32 * kItems;  // keys of one warp
+  constexpr int kSegKeys = 32 * kItems;  // keys of one warp in a sub-tile
   extern __shared__ __align__(16) unsigned char radix_smem[];
-  RadixSmem<kItems> &S = *reinterpret_cast<RadixSmem<kItems> *>(radix_smem);
+  RadixSmem<kItems, kSub> &S = *reinterpret_cast<RadixSmem<kItems, kSub> *>(radix_smem);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t lt_mask = (1u << lane) - 1u;
   const int64_t count = min64((int64_t)*count_ptr, cap);
@@ -237,7 +248,7 @@ __global__ void __launch_bounds__(kSortThreads) radix_pass_kernel(
     if (kValsAreIndex && small_out) rank_sort(keys_in, (int)count, small_out, S.scan_ranks);
     return;
   }
-  for (int i = threadIdx.x; i < (int)(sizeof S.wcount / sizeof(uint32_t)); i += kSortThreads) (&S.wcount[0][0])[i] = 0u;
+  for (int i = threadIdx.x; i < (int)(sizeof S.wcount / sizeof(uint32_t)); i += kSortThreads) (&S.wcount[0][0][0])[i] = 0u;
   uint32_t total;
   // Keys of the digits below each digit over the whole input: the same for
   // every ticket.
@@ -250,86 +261,100 @@ __global__ void __launch_bounds__(kSortThreads) radix_pass_kernel(
     const int64_t b = S.ticket;
     const int64_t tile0 = b * kTileKeys;
     if (tile0 >= count) return;
-    const int seg = warp * kSegKeys;
-    for (int c = lane; c < kSegKeys / 4; c += 32) {
-      const int64_t i0 = tile0 + seg + 4 * c;
-      if (i0 < count) {
-        const int bytes = (int)min64(16, (count - i0) * 4);
-        cp_async16(&S.keys[seg + 4 * c], keys_in + i0, bytes);
-        if (!kValsAreIndex) cp_async16(&S.vals[seg + 4 * c], vals_in + i0, bytes);
+#pragma unroll
+    for (int s = 0; s < kSub; ++s) {
+      const int seg = s * kSubKeys + warp * kSegKeys;
+      for (int c = lane; c < kSegKeys / 4; c += 32) {
+        const int64_t i0 = tile0 + seg + 4 * c;
+        if (i0 < count) {
+          const int bytes = (int)min64(16, (count - i0) * 4);
+          cp_async16(&S.keys[seg + 4 * c], keys_in + i0, bytes);
+          if (!kValsAreIndex) cp_async16(&S.vals[seg + 4 * c], vals_in + i0, bytes);
+        }
       }
+      cp_async_commit();
     }
-    cp_async_wait_all();
-    __syncwarp();  // the warp's copies are visible to all its lanes
     const int d = threadIdx.x;  // the digit this thread scans and looks back for
-    uint32_t key[kItems], val[kItems], rank[kItems];
-    int dig[kItems];
+    uint32_t tot = 0u;          // keys of digit d in the sub-tiles so far
 #pragma unroll
-    for (int k = 0; k < kItems; ++k) {
-      const int li = seg + k * 32 + lane;
-      if (tile0 + li < count) {
-        key[k] = S.keys[li];
-        val[k] = kValsAreIndex ? (uint32_t)(tile0 + li) : S.vals[li];
-        dig[k] = (key[k] >> shift) & (kRadixBins - 1);
-      } else {
-        key[k] = 0u;
-        val[k] = 0u;
-        dig[k] = kRadixBins;  // padding: ranked nowhere
+    for (int s = 0; s < kSub; ++s) {
+      uint32_t(&wc)[kWarps][kRadixBins] = S.wcount[kSub > 1 ? (s & 1) : 0];
+      cp_async_wait_pending(kSub - 1 - s);
+      __syncwarp();  // the warp's copies of sub-tile s are visible to all its lanes
+      const int seg = s * kSubKeys + warp * kSegKeys;
+      uint32_t key[kItems], val[kItems], rank[kItems];
+      int dig[kItems];
+#pragma unroll
+      for (int k = 0; k < kItems; ++k) {
+        const int li = seg + k * 32 + lane;
+        if (tile0 + li < count) {
+          key[k] = S.keys[li];
+          val[k] = kValsAreIndex ? (uint32_t)(tile0 + li) : S.vals[li];
+          dig[k] = (key[k] >> shift) & (kRadixBins - 1);
+        } else {
+          key[k] = 0u;
+          val[k] = 0u;
+          dig[k] = kRadixBins;  // padding: ranked nowhere
+        }
       }
-    }
 #pragma unroll
-    for (int k = 0; k < kItems; ++k) {
-      const int dk = dig[k];
-      uint32_t peers = 0xffffffffu;
+      for (int k = 0; k < kItems; ++k) {
+        const int dk = dig[k];
+        uint32_t peers = 0xffffffffu;
 #pragma unroll
-      for (int bit = 0; bit < 9; ++bit) {
-        const uint32_t set = (uint32_t)((dk >> bit) & 1);
-        peers &= ~(__ballot_sync(0xffffffffu, set) ^ (0u - set));
+        for (int bit = 0; bit < 9; ++bit) {
+          const uint32_t set = (uint32_t)((dk >> bit) & 1);
+          peers &= ~(__ballot_sync(0xffffffffu, set) ^ (0u - set));
+        }
+        const int leader = __ffs(peers) - 1;
+        uint32_t base = 0u;
+        if (lane == leader && dk < kRadixBins) base = atomicAdd(&wc[warp][dk], (uint32_t)__popc(peers));
+        base = __shfl_sync(0xffffffffu, base, leader);
+        __syncwarp();  // item k's counts land before item k + 1's
+        rank[k] = base + __popc(peers & lt_mask);
       }
-      const int leader = __ffs(peers) - 1;
-      uint32_t base = 0u;
-      if (lane == leader && dk < kRadixBins) base = atomicAdd(&S.wcount[warp][dk], (uint32_t)__popc(peers));
-      base = __shfl_sync(0xffffffffu, base, leader);
-      __syncwarp();  // item k's counts land before item k + 1's
-      rank[k] = base + __popc(peers & lt_mask);
-    }
-    __syncthreads();
-    // Per digit: exclusive prefix over warps; ticket count and start.
-    uint32_t cnt = 0u;
+      __syncthreads();
+      // Per digit: exclusive prefix over warps; sub-tile count and start.
+      uint32_t cnt = 0u;
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-      const uint32_t c = S.wcount[w][d];
-      S.wcount[w][d] = cnt;
-      cnt += c;
-    }
-    S.bstart[d] = block_exclusive_scan(cnt, S.scan, &total);
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < kItems; ++k) {
-      if (dig[k] < kRadixBins) {
-        const uint32_t pos = S.bstart[dig[k]] + S.wcount[warp][dig[k]] + rank[k];
-        S.keys[pos] = key[k];
-        S.vals[pos] = val[k];
+      for (int w = 0; w < kWarps; ++w) {
+        const uint32_t c = wc[w][d];
+        wc[w][d] = cnt;
+        cnt += c;
       }
+      S.sbase[s][d] = tot;
+      tot += cnt;
+      S.bstart[s][d] = block_exclusive_scan(cnt, S.scan, &total);
+      __syncthreads();
+#pragma unroll
+      for (int k = 0; k < kItems; ++k) {
+        if (dig[k] < kRadixBins) {
+          const uint32_t pos = s * kSubKeys + S.bstart[s][dig[k]] + wc[warp][dig[k]] + rank[k];
+          S.keys[pos] = key[k];
+          S.vals[pos] = val[k];
+        }
+      }
+      __syncwarp();
+      for (int i = lane; i < kRadixBins; i += 32) wc[warp][i] = 0u;  // the warp's row, for sub-tile s + 2
     }
-    __syncwarp();
-    for (int i = lane; i < kRadixBins; i += 32) S.wcount[warp][i] = 0u;  // the warp's row, for the next ticket
-    S.gstart[d] = gpre + radix_lookback(state, b, d, cnt, status);
+    S.gstart[d] = gpre + radix_lookback(state, b, d, tot, status);
     __syncthreads();
-    // Coalesced runs per digit.
+    // Coalesced runs per digit and sub-tile.
     const int32_t nvalid = (int32_t)min64(kTileKeys, count - tile0);
     for (int p = threadIdx.x; p < nvalid; p += kSortThreads) {
+      const int s = p / kSubKeys, q = p - s * kSubKeys;
       const uint32_t kk = S.keys[p];
       const int dd = (kk >> shift) & (kRadixBins - 1);
-      const uint32_t gpos = S.gstart[dd] + ((uint32_t)p - S.bstart[dd]);
+      const uint32_t gpos = S.gstart[dd] + S.sbase[s][dd] + ((uint32_t)q - S.bstart[s][dd]);
       if ((int64_t)gpos < count) {
         keys_out[gpos] = kk;
         vals_out[gpos] = S.vals[p];
         if (ranges) {
           if ((int64_t)kk < total_tiles) {
+            const int qend = min(kSubKeys, nvalid - s * kSubKeys);
             uint32_t *r = reinterpret_cast<uint32_t *>(&ranges[(int64_t)kk << range_shift]);
-            if (p == 0 || S.keys[p - 1] != kk) atomicMin(&r[0], gpos);
-            if (p == nvalid - 1 || S.keys[p + 1] != kk) atomicMax(&r[1], gpos + 1u);
+            if (q == 0 || S.keys[p - 1] != kk) atomicMin(&r[0], gpos);
+            if (q == qend - 1 || S.keys[p + 1] != kk) atomicMax(&r[1], gpos + 1u);
           } else {
             atomicOr(status, kStatusInternal);
           }
@@ -943,13 +968,22 @@ cudaError_t bin_sort_typed(const Layout &L, const fgs4d_view *views, int32_t nvi
   }
   // 3. Stable sort of the instances by global tile id (digit histograms
   // taken by the emission); the last pass also records the tile ranges.
-  const int pbt = std::min(L.tile_blocks, L.sort_grid);
-  constexpr size_t smem1 = radix_smem_bytes<kInstSortItems>();
+  // Very large instance lists take three sub-tiles per ticket (at most 3
+  // blocks of 74 KB per SM), the others one.
+  const bool wide = L.tile_sort_sub == 3;
+  const int tickets = (L.tile_blocks + L.tile_sort_sub - 1) / L.tile_sort_sub;
+  const int pbt = std::min(tickets, wide ? L.tile_sort_grid : L.sort_grid);
+  constexpr size_t smem1 = radix_smem_bytes<kInstSortItems>(), smem3 = radix_smem_bytes<kInstSortItems, 3>();
+  if (wide) {
+    e = allow_dynamic_smem(radix_pass_kernel<false, kInstSortItems, 3>, smem3);
+    if (e != cudaSuccess) return e;
+  }
   for (int p = 0; p < L.tile_passes; ++p) {
     const int in = p & 1, out = in ^ 1;
     const bool last = p == L.tile_passes - 1;
     uint32_t *state = tstate + (size_t)p * L.tile_blocks * kRadixBins;
-    e = launch_pdl_smem(radix_pass_kernel<false, kInstSortItems>, (unsigned)pbt, kSortThreads, smem1, st, (const uint32_t *)ik[in],
+    e = launch_pdl_smem(wide ? radix_pass_kernel<false, kInstSortItems, 3> : radix_pass_kernel<false, kInstSortItems>,
+                        (unsigned)pbt, kSortThreads, wide ? smem3 : smem1, st, (const uint32_t *)ik[in],
                         (const uint32_t *)iv[in], ik[out], iv[out], (const uint32_t *)(ctr + kCtrInstances),
                         (int64_t)L.inst_cap, (int32_t)(kRadixBits * p), (const uint32_t *)(hist_t + p * kRadixBins),
                         state, ctr + kCtrTicketTile + p, status, last ? ranges : (uint2 *)nullptr,
