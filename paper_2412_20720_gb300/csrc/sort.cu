@@ -18,6 +18,7 @@
 // their per-digit global offsets by decoupled look-back over the earlier
 // tickets (bounded waits), then scatter through shared memory.
 #include <algorithm>
+#include <type_traits>
 
 #include "fgs4d_internal.cuh"
 
@@ -615,15 +616,18 @@ __device__ __forceinline__ void load_emit_chunk(const EmitArgs &A, uint32_t c, u
   const uint32_t j0 = S.j0, ns = S.ns;
   if (ns <= (uint32_t)kEmitChunk)
     for (uint32_t k = threadIdx.x; k <= ns; k += kEmitBlock)
-      S.pref[k] = (int64_t)(j0 + k) <= nvis ? A.pair_prefix[j0 + k] : npairs;
+      S.pref[k] = k < ns ? A.pair_prefix[j0 + k] : 0xffffffffu;  // the last ends every walk
   if (ns <= (uint32_t)kEmitRecCache)
     for (uint32_t k = threadIdx.x; k < 3 * ns; k += kEmitBlock) S.rec[k] = A.emit_rec[3 * (size_t)j0 + k];
   __syncthreads();
 }
 
-// First pair of position k of the chunk (k <= ns).
+// First pair of position k of the chunk (k <= ns); kCached: the chunk's
+// positions fit the prefix cache (nearly all do; a test per look-up took 5 %
+// of the emission).
+template <bool kCached>
 __device__ __forceinline__ uint32_t chunk_pref(const EmitArgs &A, const EmitChunkSmem &S, int k) {
-  return S.ns <= (uint32_t)kEmitChunk ? S.pref[k] : A.pair_prefix[(size_t)S.j0 + k];
+  return kCached ? S.pref[k] : A.pair_prefix[(size_t)S.j0 + k];
 }
 
 // Walk over consecutive pairs of a chunk: the depth-sorted position the
@@ -655,16 +659,17 @@ __device__ __forceinline__ void walk_load(const EmitArgs &A, const EmitChunkSmem
 }
 
 // Positions the walk at pair f (one binary search over the chunk's prefix).
+template <bool kCached>
 __device__ __forceinline__ PairWalk walk_begin(const EmitArgs &A, const EmitChunkSmem &S, uint32_t f) {
   int lo = 0, hi = (int)S.ns - 1;
   while (lo < hi) {  // last position whose pair prefix is <= f
     const int mid = (lo + hi + 1) >> 1;
-    if (chunk_pref(A, S, mid) <= f) lo = mid;
+    if (chunk_pref<kCached>(A, S, mid) <= f) lo = mid;
     else hi = mid - 1;
   }
   PairWalk w;
   walk_load(A, S, lo, w);
-  const uint32_t local = f - chunk_pref(A, S, lo);
+  const uint32_t local = f - chunk_pref<kCached>(A, S, lo);
   const uint32_t wd = (uint32_t)max(w.x1 - w.x0, 1);
   const uint32_t qy = local / wd;
   w.tx = w.x0 + (int)(local - qy * wd);
@@ -673,14 +678,15 @@ __device__ __forceinline__ PairWalk walk_begin(const EmitArgs &A, const EmitChun
 }
 
 // Advances the walk to pair f, the pair after the current one.
+template <bool kCached>
 __device__ __forceinline__ void walk_next(const EmitArgs &A, const EmitChunkSmem &S, PairWalk &w, uint32_t f) {
   if (++w.tx >= w.x1) {
     w.tx = w.x0;
     ++w.ty;
   }
-  if (chunk_pref(A, S, w.lo + 1) <= f) {
-    int lo = min(w.lo + 1, (int)S.ns - 1);
-    while (lo + 1 < (int)S.ns && chunk_pref(A, S, lo + 1) <= f) ++lo;  // positions without pairs
+  if (chunk_pref<kCached>(A, S, w.lo + 1) <= f) {
+    int lo = kCached ? w.lo + 1 : min(w.lo + 1, (int)S.ns - 1);
+    while ((kCached || lo + 1 < (int)S.ns) && chunk_pref<kCached>(A, S, lo + 1) <= f) ++lo;  // positions without pairs
     walk_load(A, S, lo, w);
     w.tx = w.x0;
     w.ty = w.y0;
@@ -758,18 +764,23 @@ __global__ void __launch_bounds__(kEmitBlock) emit_kernel(EmitArgs A, RasterView
     const uint32_t fa = f0 + kPairsPerThread * threadIdx.x;
     uint32_t m = 0u;
     uint32_t kt[kPairsPerThread], ks[kPairsPerThread];
-    if (fa < f1) {
-      PairWalk w = walk_begin(A, S, fa);
+    auto decide = [&](auto cached_tag) {
+      constexpr bool kCached = decltype(cached_tag)::value;
+      PairWalk w = walk_begin<kCached>(A, S, fa);
 #pragma unroll
       for (int k = 0; k < kPairsPerThread; ++k) {
         if (k) {
           if (fa + k >= f1) break;
-          walk_next(A, S, w, fa + k);
+          walk_next<kCached>(A, S, w, fa + k);
         }
         m |= walk_keep<MAXV>(rv, w) ? (1u << k) : 0u;
         kt[k] = walk_tile<MAXV>(rv, w);
         ks[k] = w.slot;
       }
+    };
+    if (fa < f1) {
+      if (S.ns <= (uint32_t)kEmitChunk) decide(std::true_type());
+      else decide(std::false_type());
     }
     uint32_t total;
     const uint32_t local = block_exclusive_scan(__popc(m), s_scan, &total);
