@@ -5,8 +5,8 @@
 // colour of Eq. 6 (zero background).  The geometry is that of a pre-trained
 // 4DGS, so the backward pass returns dL/df and dL/dS(s) only.
 //
-// Both directions are contractions (for D <= 16 the forward stays scalar, see
-// render_features_scalar_kernel): the map is F[p][c] = sum_j w[p][j]
+// Both directions are contractions (short lists, and the map for D <= 16, take
+// scalar kernels: launch_feat_typed): the map is F[p][c] = sum_j w[p][j]
 // fhat[j][c], and the adjoint needs v[j][c] = sum_p w[p][j] dL/dF[p][c].  One
 // CTA per (view, tile), one pixel per thread; a warp computes the weights of
 // its 32 pixels for kChunk entries (pixel_alpha's skip/stop decisions, so the
@@ -27,9 +27,9 @@
 //
 // Measured at 300k Gaussians, one 1352x1014 view, before (multiply-adds with a
 // shuffle butterfly and D atomics per (warp, entry)) -> now, us: D = 32 forward
-// 900 -> 716, backward 1492 -> 860; D = 16 backward 933 -> 586; D = 8 663 -> 512.
-// Bound by issue (57 and 62 % of the slots at a quarter of the warps: the
-// accumulators or operands take 128 registers a thread).
+// 900 -> 726, backward 1490 -> 844; D = 16 backward 933 -> 572; D = 8 670 -> 457.
+// Bound by issue; at D = 32 a quarter of the warps are resident (operands or
+// accumulators take 128 registers a thread).
 #include <algorithm>
 
 #include "fgs4d_internal.cuh"
@@ -71,13 +71,22 @@ struct FeatArgs {
   float *g_gate;      // backward: [D] or null
 };
 
+// Pixels of a column per thread in the scalar kernels.  The adjoint reduces D
+// sums per (warp, entry): with D <= 16 it takes 4 at 16x16 (64 threads), half
+// the warps per tile and so half the reductions.
 constexpr int kScalarPPT = 2;
+template <int TILE, int D>
+__host__ __device__ constexpr int scalar_bwd_ppt() {
+  return (TILE == 16 && D <= 16) ? 4 : kScalarPPT;
+}
 
 // Stages entry `k` of the batch: geometry, opacity and normalised gated
-// feature (rows padded to D + 1 floats against bank conflicts).
-template <int D>
+// feature (rows padded to D + 1 floats against bank conflicts); for the
+// adjoint also the raw feature, its gated norm and the Gaussian.
+template <int D, bool kBwd>
 __device__ __forceinline__ void stage_feature(const FeatArgs &A, const float *s_gate, uint32_t idx, int k,
-                                              float4 *s_geom, float2 *s_ca, float *s_fhat) {
+                                              float4 *s_geom, float2 *s_ca, float *s_fhat, float *s_f, float *s_norm,
+                                              int32_t *s_gi) {
   const uint32_t s = A.inst_val[idx];
   float4 geom = make_float4(0.f, 0.f, 0.f, 0.f);
   float2 ca = make_float2(0.f, kLogAlphaNone);  // (b2, log2 a): every pixel skips the entry
@@ -112,6 +121,7 @@ __device__ __forceinline__ void stage_feature(const FeatArgs &A, const float *s_
   }
 #pragma unroll
   for (int c = 0; c < D; ++c) {
+    if (kBwd) s_f[k * (D + 1) + c] = g[c];
     g[c] *= s_gate[c];
     nn += g[c] * g[c];
   }
@@ -119,13 +129,17 @@ __device__ __forceinline__ void stage_feature(const FeatArgs &A, const float *s_
   const float inv = norm > 0.f ? 1.0f / norm : 0.f;
 #pragma unroll
   for (int c = 0; c < D; ++c) s_fhat[k * (D + 1) + c] = g[c] * inv;
+  if (kBwd) {
+    s_norm[k] = norm;
+    s_gi[k] = gi;
+  }
 }
 
 // Feature map with a multiply-add per component, pixel and entry, a thread on a
-// vertical pair of pixels.  For D <= 16 it beats the matrix form below, whose
-// weights cost a thread per pixel: 300k Gaussians at 1352x1014 (us, this /
-// matrix form) D = 8 331 / 409, D = 16 486 / 488, D = 32 900 / 717; a street
-// view of 14 entries a tile D = 16 44 / 63.
+// vertical pair of pixels: for D <= 16, where the matrix form's weights cost a
+// thread per pixel (300k Gaussians at 1352x1014, us, this / matrix form: D = 8
+// 331 / 409, D = 16 486 / 488; a street view of 14 entries a tile D = 16 44 /
+// 63), and for D = 32 on short lists (launch_feat_typed).
 template <int MAXV, int TILE, int D>
 __global__ void __launch_bounds__(TILE *TILE / kScalarPPT)
     render_features_scalar_kernel(FeatArgs A, RasterViews<MAXV> rv) {
@@ -160,7 +174,7 @@ __global__ void __launch_bounds__(TILE *TILE / kScalarPPT)
   for (uint32_t base = range.x; base < range.y; base += kBatch) {
     if (__syncthreads_count(live) == 0) break;
     if (base + threadIdx.x < range.y)
-      stage_feature<D>(A, s_gate, base + threadIdx.x, threadIdx.x, s_geom, s_ca, s_fhat);
+      stage_feature<D, false>(A, s_gate, base + threadIdx.x, threadIdx.x, s_geom, s_ca, s_fhat, nullptr, nullptr, nullptr);
     __syncthreads();
     const int nb = (int)min(range.y - base, (uint32_t)kBatch);
     for (int j = 0; j < nb && live; ++j) {
@@ -199,6 +213,124 @@ __global__ void __launch_bounds__(TILE *TILE / kScalarPPT)
 #pragma unroll
     for (int c = 0; c < D; ++c) out[c * HW + p] = F[k][c];
   }
+}
+
+// Sums D <= 32 per-lane values over the warp; on return a[0] of lane l holds
+// the total of value l (lanes >= D hold totals of zero padding).
+template <int D>
+__device__ __forceinline__ float warp_transpose_sum(float (&a)[32], int lane) {
+#pragma unroll
+  for (int half = 16; half >= 1; half >>= 1) {
+    const bool up = (lane & half) != 0;
+#pragma unroll
+    for (int i = 0; i < half; ++i) {
+      const float send = up ? a[i] : a[i + half];
+      const float keep = up ? a[i + half] : a[i];
+      a[i] = keep + __shfl_xor_sync(0xffffffffu, send, half);
+    }
+  }
+  return a[0];
+}
+
+// Adjoint with a multiply-add per component, pixel and entry and a butterfly
+// of D sums per (warp, entry): for short lists, where a matrix block's upstream
+// operands (split once per tile) and its barriers cost more than its products
+// save (launch_feat_typed).
+template <int MAXV, int TILE, int D>
+__global__ void __launch_bounds__(TILE *TILE / scalar_bwd_ppt<TILE, D>())
+    render_features_bwd_scalar_kernel(FeatArgs A, RasterViews<MAXV> rv) {
+  grid_dependency_sync();
+  constexpr int kPPT = scalar_bwd_ppt<TILE, D>();
+  constexpr int kBatch = TILE * TILE / kPPT;
+  __shared__ float4 s_geom[kBatch];
+  __shared__ float2 s_ca[kBatch];
+  __shared__ int32_t s_gi[kBatch];
+  __shared__ float s_fhat[kBatch * (D + 1)];
+  __shared__ float s_f[kBatch * (D + 1)];
+  __shared__ float s_norm[kBatch];
+  __shared__ float s_gate[D];
+  __shared__ float s_ggate[D];
+  const int32_t gt = blockIdx.x;
+  const RasterView &V = rv.v[find_view<MAXV>(rv, gt)];
+  const int32_t lt = gt - V.tile_base;
+  const int32_t tx = lt % V.gw, ty = lt / V.gw;
+  const int32_t px = tx * TILE + (threadIdx.x & (TILE - 1));
+  const int32_t py0 = ty * TILE + (threadIdx.x / TILE) * kPPT;
+  const uint2 range = tile_range(A.ranges, gt);
+  if (range.x == range.y) return;  // nothing to add
+  const float pxc = (float)px + 0.5f;
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x < D) {
+    s_gate[threadIdx.x] = A.gate ? A.gate[threadIdx.x] : 1.0f;
+    s_ggate[threadIdx.x] = 0.f;
+  }
+  const int64_t HW = (int64_t)V.width * V.height;
+  const float *dF = A.dL_dF + V.pix_base * D;
+  const float gyc = row_group_centre(py0);
+  float T[kPPT], off[kPPT], G[kPPT][D];
+  bool live = false;
+#pragma unroll
+  for (int k = 0; k < kPPT; ++k) {
+    const bool in = px < V.width && py0 + k < V.height;
+    T[k] = in ? 1.0f : -1.0f;
+    off[k] = in ? row_offset(py0 + k) : stopped_offset();
+    const int64_t p = (int64_t)(py0 + k) * V.width + px;
+#pragma unroll
+    for (int c = 0; c < D; ++c) G[k][c] = in ? dF[c * HW + p] : 0.f;
+    live = live || in;
+  }
+  for (uint32_t base = range.x; base < range.y; base += kBatch) {
+    if (__syncthreads_count(live) == 0) break;
+    if (base + threadIdx.x < range.y)
+      stage_feature<D, true>(A, s_gate, base + threadIdx.x, threadIdx.x, s_geom, s_ca, s_fhat, s_f, s_norm, s_gi);
+    __syncthreads();
+    const int nb = (int)min(range.y - base, (uint32_t)kBatch);
+    for (int j = 0; j < nb; ++j) {
+      if (!__any_sync(0xffffffffu, live)) break;  // the warp's pixels have all stopped
+      const float4 geom = s_geom[j];
+      const float2 ca = s_ca[j];
+      const ColumnTerms ct = column_terms(geom, pxc, ca.y);
+      const float w4 = group_w(ct, geom.y, ca.x, gyc);
+      const bool clamp = entry_clamps(ca.y);
+      float v[32];
+#pragma unroll
+      for (int c = 0; c < 32; ++c) v[c] = 0.f;
+      bool contrib = false;
+#pragma unroll
+      for (int k = 0; k < kPPT; ++k) {
+        const AlphaEval e = pixel_alpha(ct, w4, ca.x, off[k], clamp);
+        if (e.alpha >= kAlphaMin) {  // false for stopped pixels (row offset +inf)
+          const float w = __fmul_rn(e.alpha, T[k]);
+          const float Tn = __fsub_rn(T[k], w);
+          if (Tn < kTMin) {
+            T[k] = -T[k];
+            off[k] = stopped_offset();
+          } else {
+            contrib = true;
+#pragma unroll
+            for (int c = 0; c < D; ++c) v[c] = __fmaf_rn(G[k][c], w, v[c]);
+            T[k] = Tn;
+          }
+        }
+      }
+      live = false;
+#pragma unroll
+      for (int k = 0; k < kPPT; ++k) live = live || T[k] > 0.0f;
+      if (!__any_sync(0xffffffffu, contrib)) continue;
+      const int32_t gi = s_gi[j];
+      const float vc = warp_transpose_sum<D>(v, lane);  // lane c: component c of the warp's sum
+      const float fh = lane < D ? s_fhat[j * (D + 1) + lane] : 0.f;
+      const float dot = warp_sum(fh * vc);
+      const float norm = s_norm[j];
+      if (gi >= 0 && norm > 0.f && lane < D) {
+        const float dg = (vc - fh * dot) / norm;
+        atomicAdd(&A.g_feat[(int64_t)gi * D + lane], s_gate[lane] * dg);
+        if (A.g_gate) atomicAdd(&s_ggate[lane], s_f[j * (D + 1) + lane] * dg);
+      }
+    }
+  }
+  __syncthreads();
+  if (A.g_gate && threadIdx.x < D && s_ggate[threadIdx.x] != 0.f) atomicAdd(&A.g_gate[threadIdx.x], s_ggate[threadIdx.x]);
 }
 
 __device__ __forceinline__ float tf32_round(float x) {
@@ -391,12 +523,18 @@ __global__ void __launch_bounds__(feat_threads<TILE>()) render_features_kernel(F
     for (int j0 = 0; j0 < nb; j0 += kChunk) {
       if (!__any_sync(0xffffffffu, P.live())) break;
       bool some = false;
-#pragma unroll 4
-      for (int j = 0; j < kChunk; ++j) {
+      auto one = [&](int j) {
         const float x = P.weight(S.geom[j0 + j], S.ca[j0 + j]);
         if (any_bad && x > 0.f) poison |= S.bad[j0 + j];
         some = some || x > 0.f;
         w[j * kWFwd + lane] = x;
+      };
+      if (nb - j0 >= kChunk) {
+#pragma unroll 4
+        for (int j = 0; j < kChunk; ++j) one(j);
+      } else {  // the rest of the last chunk has no weights
+        for (int j = 0; j < nb - j0; ++j) one(j);
+        for (int j = nb - j0; j < kChunk; ++j) w[j * kWFwd + lane] = 0.f;
       }
       __syncwarp();
       if (__any_sync(0xffffffffu, some)) {
@@ -453,8 +591,15 @@ __global__ void __launch_bounds__(feat_threads<TILE>()) render_features_kernel(F
   }
 }
 
+// Resident blocks of 256 threads (or as many threads of 64) per SM: what the
+// operands and accumulators allow without spills (64, 80 and 128 registers).
+template <int TILE, int D>
+constexpr int bwd_min_blocks() {
+  return (D == 8 ? 4 : (D == 16 ? 3 : 2)) * (TILE == 16 ? 1 : 4);
+}
+
 template <int MAXV, int TILE, int D>
-__global__ void __launch_bounds__(feat_threads<TILE>()) render_features_bwd_kernel(FeatArgs A, RasterViews<MAXV> rv) {
+__global__ void __launch_bounds__(feat_threads<TILE>(), (bwd_min_blocks<TILE, D>())) render_features_bwd_kernel(FeatArgs A, RasterViews<MAXV> rv) {
   grid_dependency_sync();
   constexpr int NT = feat_threads<TILE>(), kWarps = NT / 32, kN = D / 8, kRow = D + 1;
   constexpr int kPart = feat_stride<D>();  // floats per entry row of a warp's sums
@@ -474,6 +619,7 @@ __global__ void __launch_bounds__(feat_threads<TILE>()) render_features_bwd_kern
   const int32_t px = tx0 + (threadIdx.x & (TILE - 1)), py = ty0 + threadIdx.x / TILE;
   const bool in = px < V.width && py < V.height;
   const uint2 range = tile_range(A.ranges, gt);
+  if (range.x == range.y) return;  // nothing to add
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lr = lane >> 2, lc = lane & 3;
   if (threadIdx.x < D) {
     s_gate[threadIdx.x] = A.gate ? A.gate[threadIdx.x] : 1.0f;
@@ -489,6 +635,15 @@ __global__ void __launch_bounds__(feat_threads<TILE>()) render_features_bwd_kern
   float up[D];  // all in flight before the first is used
 #pragma unroll
   for (int c = 0; c < D; ++c) up[c] = in ? dF[c * HW + pixel] : 0.f;
+  // The first batch is staged meanwhile.
+  auto stage = [&](uint32_t base, int nb) {
+    stage_features<NT, D>(A, s_gate, base, nb, S, [&](int k, int c, float f, float x) {
+      s_f[k * kRow + c] = f;
+      s_fhat[k * kRow + c] = x;
+    });
+  };
+  __syncthreads();  // s_gate
+  stage(range.x, (int)min(range.y - range.x, (uint32_t)kFeatBatch));
   bool bad = false;
 #pragma unroll
   for (int n = 0; n < kN; ++n) {
@@ -512,23 +667,30 @@ __global__ void __launch_bounds__(feat_threads<TILE>()) render_features_bwd_kern
   float ggate = 0.f;  // of component lane % D
   int buf = 0;
   for (uint32_t base = range.x; base < range.y; base += kFeatBatch) {
-    if (__syncthreads_count(P.live()) == 0) break;
     const int nb = (int)min(range.y - base, (uint32_t)kFeatBatch);
-    stage_features<NT, D>(A, s_gate, base, nb, S, [&](int k, int c, float f, float x) {
-      s_f[k * kRow + c] = f;
-      s_fhat[k * kRow + c] = x;
-    });
+    if (base != range.x) {
+      if (__syncthreads_count(P.live()) == 0) break;
+      stage(base, nb);
+    }
     __syncthreads();
     for (int j0 = 0; j0 < nb; j0 += kChunk, buf ^= 1) {
       float *w = s_buf[warp];
       bool some = false;
       if (__any_sync(0xffffffffu, P.live())) {
         uint32_t hit = 0u;
-#pragma unroll 4
-        for (int j = 0; j < kChunk; ++j) {
-          const float x = P.weight(S.geom[j0 + j], S.ca[j0 + j]);
-          if (x > 0.f) hit |= 1u << j;
-          w[j * kWBwd + lane] = x;
+        const int m = min(nb - j0, kChunk);  // the rest of the last chunk has no weights
+        for (int j4 = 0; j4 < kChunk; j4 += 4) {
+          if (j4 < m) {
+#pragma unroll
+            for (int j = j4; j < j4 + 4; ++j) {
+              const float x = P.weight(S.geom[j0 + j], S.ca[j0 + j]);
+              if (x > 0.f) hit |= 1u << j;
+              w[j * kWBwd + lane] = x;
+            }
+          } else {
+#pragma unroll
+            for (int j = j4; j < j4 + 4; ++j) w[j * kWBwd + lane] = 0.f;
+          }
         }
         if (bad_pixels) {
           const uint32_t e = __reduce_or_sync(0xffffffffu, bad ? hit : 0u);
@@ -605,15 +767,30 @@ __global__ void __launch_bounds__(feat_threads<TILE>()) render_features_bwd_kern
 
 template <int MAXV, int TILE, int D>
 cudaError_t launch_feat_tile(const FeatArgs &A, const RasterViews<MAXV> &rv, unsigned grid, bool backward,
-                             cudaStream_t st) {
+                             bool short_lists, cudaStream_t st) {
   constexpr unsigned NT = feat_threads<TILE>();
-  if (backward)
+  if (backward) {
+    if (short_lists)
+      return launch_pdl(render_features_bwd_scalar_kernel<MAXV, TILE, D>, grid,
+                        (unsigned)(TILE * TILE / scalar_bwd_ppt<TILE, D>()), st, A, rv);
     return launch_pdl(render_features_bwd_kernel<MAXV, TILE, D>, grid, NT, st, A, rv);
-  if constexpr (D <= 16)
-    return launch_pdl(render_features_scalar_kernel<MAXV, TILE, D>, grid, (unsigned)(TILE * TILE / kScalarPPT), st, A, rv);
-  else
-    return launch_pdl(render_features_kernel<MAXV, TILE, D>, grid, NT, st, A, rv);
+  }
+  if constexpr (D > 16) {
+    if (!short_lists) return launch_pdl(render_features_kernel<MAXV, TILE, D>, grid, NT, st, A, rv);
+  }
+  return launch_pdl(render_features_scalar_kernel<MAXV, TILE, D>, grid, (unsigned)(TILE * TILE / kScalarPPT), st, A, rv);
 }
+
+// Calls whose lists are surely short take the scalar kernels: the instance
+// capacity, an upper bound of the instances, is below this many a tile (twice
+// the lists' length or more, as capacities have headroom).  Scalar / matrix
+// (us) at 1352x1014, by instances a tile: adjoint D = 8 5.2 33 / 48, 10.6 50 /
+// 56, 15 64 / 66, 20.5 81 / 76, 308 670 / 457; D = 32 78 / 113, 115 / 126, 146 /
+// 142, 181 / 158, 1490 / 844; map D = 32 5.2 56 / 95, 10.6 74 / 105, 20.5 111 /
+// 132, 31 154 / 160, 41 197 / 187, 308 902 / 726.  With fewer tiles than some
+// 4000 one round of blocks holds most of a call and the longest list decides:
+// the adjoint of 1200 tiles with 10 entries a tile takes 25 / 19 at D = 8.
+constexpr int64_t kShortAdjointCap = 40, kShortAdjointMinTiles = 4096, kShortMapCap = 72;
 
 template <int MAXV, int D>
 cudaError_t launch_feat_typed(const Layout &L, const FeatArgs &A, const fgs4d_view *views, int32_t nviews,
@@ -622,8 +799,11 @@ cudaError_t launch_feat_typed(const Layout &L, const FeatArgs &A, const fgs4d_vi
   if (!make_raster_views<MAXV>(L, views, nviews, &rv)) return cudaErrorInvalidValue;
   if (L.total_tiles == 0) return cudaSuccess;
   const unsigned grid = (unsigned)L.total_tiles;
-  if (L.tile == 8) return launch_feat_tile<MAXV, 8, D>(A, rv, grid, backward, st);
-  return launch_feat_tile<MAXV, 16, D>(A, rv, grid, backward, st);
+  const bool short_lists =
+      backward ? L.total_tiles >= kShortAdjointMinTiles && L.inst_cap < kShortAdjointCap * L.total_tiles
+               : L.inst_cap < kShortMapCap * L.total_tiles;
+  if (L.tile == 8) return launch_feat_tile<MAXV, 8, D>(A, rv, grid, backward, short_lists, st);
+  return launch_feat_tile<MAXV, 16, D>(A, rv, grid, backward, short_lists, st);
 }
 
 template <int D>

@@ -72,3 +72,30 @@ def test_feature_backward_matches_oracle(D, tile):
     r.check()
     compare_group("dL/df", grad_f.cpu().numpy().astype(np.float64), gf, 1e-3, 1e-4)
     compare_group("dL/dgate", grad_g.cpu().numpy().astype(np.float64), gg, 1e-3, 1e-4)
+
+
+@pytest.mark.parametrize("D", [8, 16, 32])
+def test_short_list_kernels_match_the_matrix_kernels(D):
+    """The same calls by both routes (an instance capacity of fewer and of more
+    than 40 instances a tile, 4225 tiles).  Map: weights add up to at most 1,
+    so the split products stay within 2^-21 and up to 150 roundings of 2^-24;
+    gradients: 1e-4 of the largest, as atomics add in another order."""
+    import torch
+    params = to_device(sy.make_scene(3000, 21, (-1, -1, -1), (1, 1, 1), sh_degree=1, t_order=1).as_dict())
+    view = sy.tiny_view(1040, 1030)
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    feats, gate = torch.randn((3000, D), device="cuda", generator=gen), torch.rand((D,), device="cuda", generator=gen)
+    up = torch.randn(D * 1040 * 1030, device="cuda", generator=gen)
+    got = []
+    for cap in (39 * 4225, 1 << 21):
+        r = Renderer(3000, [view], RenderConfig(sh_degree=1, t_order=1, inst_capacity=cap))
+        out = r.forward_features(params, feats, gate)
+        assert r.check()[1] > 20_000
+        gf, gg = torch.zeros_like(feats), torch.zeros_like(gate)
+        r.backward_features(feats, gate, up, gf, gg)
+        got.append((out, gf, gg))
+    (ma, fa, ga), (mb, fb, gb) = got
+    assert float(ma.abs().max()) > 0.3
+    assert float((ma - mb).abs().max()) <= 2.0 ** -21 + 150 * 2.0 ** -24
+    assert float((fa - fb).abs().max()) <= 1e-4 * float(fa.abs().max())
+    assert float((ga - gb).abs().max()) <= 1e-4 * float(ga.abs().max())
