@@ -12,9 +12,11 @@
 // its 32 pixels for kChunk entries (pixel_alpha's skip/stop decisions, so the
 // weights equal those of the colour compositor bit for bit), passes them
 // through shared memory and multiplies on the tensor cores (mma.sync m16n8k8,
-// TF32 operands split in two: x = hi + lo with 11 bits each, hi hi + hi lo +
-// lo hi, so a product is within 2^-22; FP32 accumulators that start at zero
-// every chunk and are added up in FP32).  The warp-level instruction is taken
+// TF32 operands split in two: x = hi + lo with 11 bits each, lo hi + hi lo + hi
+// hi; with lo rounded to 2^-23 |x| and lo lo left out, up to 2^-22, a product
+// is within 2^-21; the accumulators start at zero every chunk, take a chunk's
+// small products before its large ones, as the matrix unit's sums lose bits at
+// the size they have reached, and are added up in FP32).  The warp-level instruction is taken
 // rather than tcgen05 because the weights come out of a per-pixel recurrence
 // 32 pixels at a time and the contraction is the small part: 48 products of
 // some 800 issued instructions per chunk of 16 entries and 32 pixels at D = 32.
@@ -539,14 +541,16 @@ __global__ void __launch_bounds__(feat_threads<TILE>()) render_features_kernel(F
       __syncwarp();
       if (__any_sync(0xffffffffu, some)) {
         float acc[2][kN][4] = {};
+        uint32_t ah[kChunk / 8][2][4];
+        // the small products of both K steps first
 #pragma unroll
         for (int ks = 0; ks < kChunk / 8; ++ks) {
-          uint32_t ah[2][4], al[2][4];
+          uint32_t al[2][4];
 #pragma unroll
           for (int m = 0; m < 2; ++m)
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-              tf32_split(w[(8 * ks + lc + (i >> 1) * 4) * kWFwd + 16 * m + lr + (i & 1) * 8], &ah[m][i], &al[m][i]);
+              tf32_split(w[(8 * ks + lc + (i >> 1) * 4) * kWFwd + 16 * m + lr + (i & 1) * 8], &ah[ks][m][i], &al[m][i]);
           const int r0 = (j0 + 8 * ks + lc) * kStride + lr, r1 = r0 + 4 * kStride;
 #pragma unroll
           for (int n = 0; n < kN; ++n) {
@@ -555,9 +559,18 @@ __global__ void __launch_bounds__(feat_threads<TILE>()) render_features_kernel(F
 #pragma unroll
             for (int m = 0; m < 2; ++m) {
               mma_tf32(acc[m][n], al[m], bh0, bh1);
-              mma_tf32(acc[m][n], ah[m], bl0, bl1);
-              mma_tf32(acc[m][n], ah[m], bh0, bh1);
+              mma_tf32(acc[m][n], ah[ks][m], bl0, bl1);
             }
+          }
+        }
+#pragma unroll
+        for (int ks = 0; ks < kChunk / 8; ++ks) {
+          const int r0 = (j0 + 8 * ks + lc) * kStride + lr, r1 = r0 + 4 * kStride;
+#pragma unroll
+          for (int n = 0; n < kN; ++n) {
+            const uint32_t bh0 = s_hi[r0 + 8 * n], bh1 = s_hi[r1 + 8 * n];
+#pragma unroll
+            for (int m = 0; m < 2; ++m) mma_tf32(acc[m][n], ah[ks][m], bh0, bh1);
           }
         }
 #pragma unroll
@@ -701,19 +714,23 @@ __global__ void __launch_bounds__(feat_threads<TILE>(), (bwd_min_blocks<TILE, D>
       __syncwarp();
       if (some) {
         float acc[kN][4] = {};
+        uint32_t ah[4][4];
 #pragma unroll
         for (int ks = 0; ks < 4; ++ks) {
-          uint32_t ah[4], al[4];
+          uint32_t al[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i)
-            tf32_split(w[(lr + (i & 1) * 8) * kWBwd + 8 * ks + lc + (i >> 1) * 4], &ah[i], &al[i]);
+            tf32_split(w[(lr + (i & 1) * 8) * kWBwd + 8 * ks + lc + (i >> 1) * 4], &ah[ks][i], &al[i]);
 #pragma unroll
           for (int n = 0; n < kN; ++n) {
             mma_tf32(acc[n], al, Gh[ks][n][0], Gh[ks][n][1]);
-            mma_tf32(acc[n], ah, Gl[ks][n][0], Gl[ks][n][1]);
-            mma_tf32(acc[n], ah, Gh[ks][n][0], Gh[ks][n][1]);
+            mma_tf32(acc[n], ah[ks], Gl[ks][n][0], Gl[ks][n][1]);
           }
         }
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+          for (int n = 0; n < kN; ++n) mma_tf32(acc[n], ah[ks], Gh[ks][n][0], Gh[ks][n][1]);
         __syncwarp();  // the weights have been read
 #pragma unroll
         for (int n = 0; n < kN; ++n)

@@ -99,3 +99,44 @@ def test_short_list_kernels_match_the_matrix_kernels(D):
     assert float((ma - mb).abs().max()) <= 2.0 ** -21 + 150 * 2.0 ** -24
     assert float((fa - fb).abs().max()) <= 1e-4 * float(fa.abs().max())
     assert float((ga - gb).abs().max()) <= 1e-4 * float(ga.abs().max())
+
+
+def _eleven_bits(x):
+    """x rounded to 11 significant bits."""
+    m, e = np.frexp(x)
+    return np.ldexp(np.round(m * 2048) / 2048, e)
+
+
+def test_split_products_keep_their_bits():
+    """The matrix kernels' sums against FP64 sums of the same weights, which
+    one-hot features give exactly.  A product is within 2^-21 of itself and the
+    accumulation within some roundings of 2^-24, so 2^-19 of the sum of the
+    magnitudes bounds the error; operands of 11 bits miss it."""
+    import torch
+    n, W, H, tol = 32, 48, 40, 2.0 ** -19
+    params = to_device(sy.make_scene(n, 4, (-0.7, -0.7, -0.7), (0.7, 0.7, 0.7), sh_degree=1, t_order=1).as_dict())
+    params["opacity_logit"] += 1.5
+    r = Renderer(n, [sy.tiny_view(W, H)], RenderConfig(sh_degree=1, t_order=1, inst_capacity=1 << 16))
+    rng = np.random.default_rng(6)
+    w = r.forward_features(params, torch.eye(n, device="cuda")).view(n, -1).cpu().numpy().astype(np.float64)
+    assert (w.max(1) > 0.05).sum() >= 8
+    for D in (32, 16, 8):
+        f = rng.standard_normal((n, D)).astype(np.float32)
+        g = rng.standard_normal((D, H * W)).astype(np.float32)
+        norm = np.sqrt((f.astype(np.float64) ** 2).sum(1, keepdims=True))
+        fhat = f / norm
+        feats = torch.from_numpy(f).cuda()
+        out = r.forward_features(params, feats).view(D, -1).cpu().numpy()
+        want, size = fhat.T @ w, np.abs(fhat).T @ w
+        assert np.all(np.abs(out - want) <= tol * size)
+        if D == 32:
+            assert np.any(np.abs(fhat.T @ _eleven_bits(w) - want) > 4 * tol * size)
+        gf = torch.zeros_like(feats)
+        r.backward_features(feats, None, torch.from_numpy(g.reshape(-1)).cuda(), gf)
+        jac = lambda v: (v - fhat * (fhat * v).sum(1, keepdims=True)) / norm
+        want, mag = jac(w @ g.T.astype(np.float64)), w @ np.abs(g.T)
+        size = (mag + np.abs(fhat) * (np.abs(fhat) * mag).sum(1, keepdims=True)) / norm
+        assert np.all(np.abs(gf.cpu().numpy() - want) <= tol * size)
+        assert np.any(np.abs(jac(_eleven_bits(w) @ g.T) - want) > 4 * tol * size)
+        assert np.any(np.abs(jac(w @ _eleven_bits(g).T) - want) > 4 * tol * size)
+    r.check()
