@@ -84,6 +84,7 @@ enum Counter : int {
   kCtrNeedVisible = 3,
   kCtrNeedInstances = 4,
   kCtrTicketPre = 5,
+  kCtrBlockFirst = 6,  // block_first_mark() of the preprocess call whose block_first the workspace holds
   // bytes [0, 32) are reset by preprocess only; the rest by bin_sort as well
   kCtrTicketEmit = 8,
   kCtrTicketChunk = 9,
@@ -185,6 +186,13 @@ struct Layout {
   int32_t depth_passes, tile_passes;
   int32_t tile_bits;
 };
+
+// Names the block_first array that a preprocess call with this layout writes.
+// The adjoint takes groups of logical blocks only where it finds the mark:
+// records that the caller filled in come without the array.
+inline uint32_t block_first_mark(const Layout &L) {
+  return 0x80000000u | ((uint32_t)(L.block_first / 256) ^ ((uint32_t)L.pre_blocks << 7) ^ ((uint32_t)L.nviews << 21));
+}
 
 // Host: computes the layout; returns FGS4D_OK or an error code.
 int compute_layout(const fgs4d_settings *s, int64_t n, const fgs4d_view *views, int32_t nviews, Layout *out);

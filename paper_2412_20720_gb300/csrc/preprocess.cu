@@ -44,6 +44,7 @@ struct PreArgs {
   int4 *rec_meta;
   uint32_t *depth_key;
   uint32_t *block_first;  // first slot of each logical block
+  uint32_t block_first_mark;
   // Staged form: per logical block its visible count and kPreBlock places for
   // its records.
   uint32_t *stage_count;
@@ -67,6 +68,7 @@ struct BwdArgs {
   int32_t blocks_per_view;
   bool grouped;  // blocks take groups of logical blocks, views fastest
   const uint32_t *block_first;
+  uint32_t block_first_mark;
   const float4 *slot_grad;
   float4 *g_mean, *g_log_scale, *g_q_l, *g_q_r;
   float *g_logit, *g_sh;
@@ -347,11 +349,13 @@ __device__ __forceinline__ bool forward_chain(int32_t i, const float4 *__restric
   return true;
 }
 
-// Sets the visible total (clamped to the capacity) and its overflow flag.
+// Sets the visible total (clamped to the capacity), its overflow flag and the
+// mark of the block_first array.
 __device__ __forceinline__ void set_visible_total(const PreArgs &A, uint64_t all) {
   A.counters[kCtrNeedVisible] = (uint32_t)umin64(all, 0xffffffffull);
   A.counters[kCtrVisible] = (uint32_t)umin64(all, (uint64_t)A.vis_cap);
   if (all > (uint64_t)A.vis_cap) atomicOr(&A.counters[kCtrStatus], kStatusVisOverflow);
+  A.counters[kCtrBlockFirst] = A.block_first_mark;
 }
 
 // kStaged: every logical block leaves its records, compacted, at its own
@@ -796,9 +800,13 @@ template <int L, int MAXV>
 __global__ void __launch_bounds__(128, 4) preprocess_bwd_kernel(BwdArgs A, PreViews<MAXV> views) {
   grid_dependency_sync();
   const int64_t nvis = min64((int64_t)A.counters[kCtrVisible], A.vis_cap);
-  if (MAXV == 1 || !A.grouped) {
-    const int64_t slot = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (slot < nvis) slot_adjoint<L, MAXV>(A, views, slot);
+  if (MAXV == 1 || !A.grouped || A.counters[kCtrBlockFirst] != A.block_first_mark) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    int64_t slot = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    do {
+      if (slot < nvis) slot_adjoint<L, MAXV>(A, views, slot);
+      slot += stride;
+    } while (MAXV > 1 && A.grouped && slot < nvis);  // (a grid sized for the groups)
     return;
   }
   // Block (group of kBwdGroup logical blocks, view), views fastest: the slots
@@ -876,6 +884,7 @@ cudaError_t launch_pre_typed(const PreLaunch &p, const fgs4d_view *views, int32_
   A.rec_meta = reinterpret_cast<int4 *>(p.ws + Lo.rec_meta);
   A.depth_key = reinterpret_cast<uint32_t *>(p.ws + Lo.depth_key);
   A.block_first = reinterpret_cast<uint32_t *>(p.ws + Lo.block_first);
+  A.block_first_mark = block_first_mark(Lo);
   if (Lo.pre_blocks == 0) return cudaSuccess;
   if (!Lo.pre_staged)
     return launch_pdl(preprocess_kernel<L, MAXV, false>, (unsigned)Lo.pre_grid, kPreBlock, p.stream, A, pv);
@@ -931,6 +940,7 @@ cudaError_t launch_bwd_typed(const PreLaunch &p, const fgs4d_view *views, int32_
   A.densify_stats = reinterpret_cast<float4 *>(gr->densify_stats);
   A.blocks_per_view = Lo.pre_blocks_per_view;
   A.block_first = reinterpret_cast<const uint32_t *>(p.ws + Lo.block_first);
+  A.block_first_mark = block_first_mark(Lo);
   // Several views whose SH rows and gradients do not fit L2 together (129 MB)
   // take the grouped order; otherwise slots in their own order fill the blocks.
   A.grouped = MAXV > 1 && p.g->n * A.k3 * (int64_t)(2 * sizeof(float)) > kBwdGroupedMinBytes;

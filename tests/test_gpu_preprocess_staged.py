@@ -54,3 +54,37 @@ def test_a_second_preprocess_keeps_the_lists(n, nviews, inst_cap):
     got = torch.empty_like(want)
     fgs4d.render_fwd(n, r.views, r.nviews, r.settings, ws, r.ws_bytes, got.data_ptr(), None, r.stream())
     assert not torch.equal(first, want) and torch.equal(got, want)
+
+
+def test_adjoint_of_records_the_caller_filled():
+    """Records copied into a workspace that no preprocess ran on give the
+    gradients of the workspace they came from (several views, SH rows that
+    make the adjoint take groups of Gaussians)."""
+    import torch
+    n, nviews = 90_001, 3
+    params = to_device(sy.make_scene(n, 7, (-2, -2, -2), (2, 2, 2), sh_degree=3, t_order=2).as_dict())
+    views = [sy.tiny_view(400, 300, t=0.2 + 0.3 * k) for k in range(nviews)]
+    cfg = RenderConfig(sh_degree=3, t_order=2, inst_capacity=1 << 22)
+    a, b = Renderer(n, views, cfg), Renderer(n, views, cfg)
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    d = torch.randn(3 * a.total_pixels, device="cuda", generator=gen)
+    a.forward(params)
+    v, L = a.check()[0], a.layout
+    b.ws.fill_(0x7f)
+    b.ws[L.counters:L.counters + 256] = 0
+    b.workspace_view(L.counters, torch.int32, 1).fill_(v)
+    for off, words in ((L.rec_geom, 4), (L.rec_color, 4), (L.rec_blue, 1), (L.rec_tau, 1), (L.rec_meta, 4), (L.depth_key, 1)):
+        b.workspace_view(off, torch.int32, words * v).copy_(a.workspace_view(off, torch.int32, words * v))
+    ws = b.ws.data_ptr()
+    img = torch.empty(3 * b.total_pixels, device="cuda")
+    fgs4d.bin_sort(n, b.views, b.nviews, b.settings, ws, b.ws_bytes, b.stream())
+    fgs4d.render_fwd(n, b.views, b.nviews, b.settings, ws, b.ws_bytes, img.data_ptr(), None, b.stream())
+    got = []
+    for r in (a, b):
+        grads = {k: torch.zeros_like(x) for k, x in params.items()}
+        r.backward(params, d, grads)
+        r.check()
+        got.append(grads)
+    for k, want in got[0].items():  # atomics add in another order from run to run
+        assert float(want.abs().max()) > 0
+        assert float((got[1][k] - want).abs().max()) <= 1e-4 * float(want.abs().max()), k
