@@ -791,9 +791,14 @@ __device__ __forceinline__ void slot_adjoint(const BwdArgs &A, const PreViews<MA
            (gqr[3] - s * dr) * ir);
 }
 
-// 1M Gaussians, 8 views (1.15 GB): 790 -> 642 us; 60k, 2 views (39 MB, few
-// blocks) 20.0 -> 24.9, left as it was.
-constexpr int64_t kBwdGroupedMinBytes = int64_t(96) << 20;
+// Groups are taken from three views on, when the SH rows and their gradients
+// exceed L2 and the slots (the visible capacity) touch many more bytes than
+// that.  Slots in their own order / groups (us), degree 3: 1M Gaussians, 8
+// views, 2.6 GB touched 578 / 408; 300k, 4 views, 402 MB 115 / 103; 200k, 4
+// views, 268 MB 103 / 113; 100k, 8 views, 271 MB 80 / 104; 1M, 2 views, 656 MB
+// 95 / 101; 1M, 6 views of which 2 % are visible, 154 MB 21 / 37 (a group of
+// 1024 Gaussians leaves most of its block idle).
+constexpr int64_t kBwdGroupedMinBytes = int64_t(96) << 20, kBwdGroupedMinTouched = int64_t(400) << 20;
 constexpr int kBwdGroup = 4;  // logical blocks whose slots one block takes (about 290 of 1024 at 28 % visible)
 
 template <int L, int MAXV>
@@ -941,9 +946,10 @@ cudaError_t launch_bwd_typed(const PreLaunch &p, const fgs4d_view *views, int32_
   A.blocks_per_view = Lo.pre_blocks_per_view;
   A.block_first = reinterpret_cast<const uint32_t *>(p.ws + Lo.block_first);
   A.block_first_mark = block_first_mark(Lo);
-  // Several views whose SH rows and gradients do not fit L2 together (129 MB)
-  // take the grouped order; otherwise slots in their own order fill the blocks.
-  A.grouped = MAXV > 1 && p.g->n * A.k3 * (int64_t)(2 * sizeof(float)) > kBwdGroupedMinBytes;
+  // Views side by side, or slots in their own order (kBwdGroupedMinTouched).
+  const int64_t row_bytes = A.k3 * (int64_t)(2 * sizeof(float));
+  A.grouped = MAXV > 1 && nviews >= 3 && p.g->n * row_bytes > kBwdGroupedMinBytes &&
+              Lo.vis_cap * row_bytes > kBwdGroupedMinTouched;
   const int64_t blocks = A.grouped ? (int64_t)((Lo.pre_blocks_per_view + kBwdGroup - 1) / kBwdGroup) * nviews
                                    : (Lo.vis_cap + 127) / 128;
   if (blocks == 0) return cudaSuccess;

@@ -61,9 +61,9 @@ def test_adjoint_of_records_the_caller_filled():
     gradients of the workspace they came from (several views, SH rows that
     make the adjoint take groups of Gaussians)."""
     import torch
-    n, nviews = 90_001, 3
+    n, nviews = 100_003, 4  # 115 MB of SH rows and gradients, 461 MB by slots
     params = to_device(sy.make_scene(n, 7, (-2, -2, -2), (2, 2, 2), sh_degree=3, t_order=2).as_dict())
-    views = [sy.tiny_view(400, 300, t=0.2 + 0.3 * k) for k in range(nviews)]
+    views = [sy.tiny_view(400, 300, t=0.2 + 0.2 * k) for k in range(nviews)]
     cfg = RenderConfig(sh_degree=3, t_order=2, inst_capacity=1 << 22)
     a, b = Renderer(n, views, cfg), Renderer(n, views, cfg)
     gen = torch.Generator(device="cuda").manual_seed(1)
