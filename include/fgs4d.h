@@ -201,8 +201,11 @@ int fgs4d_preprocess(const fgs4d_gaussians *gaussians, const fgs4d_view *views, 
  * slot emits one instance per tile of its rect whose pixel-centre box meets
  * the slot's 1/255 ellipse (tiles it misses would skip the slot at every
  * pixel, so the image is that of the full rect membership); instances are
- * ordered by (global tile, FP32 depth, slot) with a hand-written radix sort,
- * and each tile's [start, end) range is computed.  Reads only what fgs4d_preprocess
+ * ordered by (global tile, FP32 depth, slot), and each tile's [start, end)
+ * range is computed.  Calls of many slots (the visible capacity decides) bin in
+ * two levels, the others by radix sort; list, ranges and counts are the same,
+ * and the former takes some 13 more bytes of workspace per instance of
+ * capacity.  Reads only what fgs4d_preprocess
  * (or a caller filling rec_meta, depth_key and counters[0]) wrote.
  * Device-detected: instance capacity. */
 int fgs4d_bin_sort(int64_t n, const fgs4d_view *views, int32_t nviews, const fgs4d_settings *settings,
@@ -216,9 +219,9 @@ int fgs4d_preprocess_kernels(int64_t n, const fgs4d_view *views, int32_t nviews,
                              int32_t *count_out);
 
 /* Diagnostic: *count_out = the number of kernels fgs4d_bin_sort launches for
- * these arguments (the count depends on the tile grid's size, which sets the
- * number of tile-sort passes).  Launches nothing; has no counterpart in the
- * paper. */
+ * these arguments (the count depends on the tile grids' sizes, which set the
+ * number of sort passes, and on the visible capacity, which selects the
+ * binning).  Launches nothing; has no counterpart in the paper. */
 int fgs4d_bin_sort_kernels(int64_t n, const fgs4d_view *views, int32_t nviews, const fgs4d_settings *settings,
                            int32_t *count_out);
 
@@ -479,7 +482,10 @@ int fgs4d_sort_depth_static_status(void *stream);
 /* Synchronises `stream`, then reads the workspace status word.  Returns
  * FGS4D_OK, or the first recorded device condition (FGS4D_ERR_CAPACITY,
  * FGS4D_ERR_TIMEOUT, FGS4D_ERR_INTERNAL).  counts_out (optional, 4 entries):
- * visible pairs, instances, visible pairs needed, instances needed. */
+ * visible pairs, instances, visible pairs needed, instances needed (exact, or,
+ * when the call has more candidate pairs than 8 x inst_capacity, the tiles of
+ * the slots' rects, which bound it; enough for a call with the same settings
+ * and a larger inst_capacity). */
 int fgs4d_get_status(const void *workspace, size_t workspace_bytes, void *stream, int64_t *counts_out);
 
 /* Static description of a status code. */

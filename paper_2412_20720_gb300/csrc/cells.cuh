@@ -23,7 +23,7 @@
 constexpr int kCellShift = 3;
 constexpr int kCellEdge = 1 << kCellShift;
 constexpr int kCellTiles = kCellEdge * kCellEdge;  // bits of a mask
-static_assert(kCellTiles == 64, "one 64-bit mask per pair, one 8-bit row of tiles per warp");
+static_assert(kCellTiles == 64, "one 64-bit mask per pair");
 
 struct CellArgs {
   EmitArgs e;

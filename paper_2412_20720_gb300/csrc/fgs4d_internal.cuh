@@ -38,7 +38,7 @@ constexpr int64_t kWideTileSortMinCap = int64_t(1) << 26;
 // Two-level binning (cells.cuh).
 constexpr int kCellChunk = 256;          // candidate (slot, cell) pairs per emission chunk, one per thread
 constexpr int kCellSeg = 256;            // sorted pairs per segment, one per thread
-constexpr int kCellBlock = kCellSeg;     // threads of the count and write kernels: one warp per row of a cell's tiles
+constexpr int kCellBlock = kCellSeg;     // threads of the count and write kernels: one pair each
 constexpr int kCellPrefixThreads = 512;
 // A cell's range has a 128-byte line of its own: the cell sort's blocks update
 // the ranges by atomics, and eight or sixteen cells a line cost 75 or 105 us a
@@ -268,43 +268,13 @@ __device__ __forceinline__ void st_relaxed(uint64_t *p, uint64_t v) {
 }
 
 // Decoupled look-back over uint64 block states (flag in bits 62-63: 1 =
-// aggregate only, 2 = inclusive prefix).  Called by one thread of logical
-// block `bid` with the block's aggregate; returns the exclusive prefix.
-// Predecessors hold smaller tickets, so they are resident or finished and the
-// wait ends; the poll count is still bounded.
-__device__ __forceinline__ uint64_t lookback_u64(uint64_t *state, int32_t bid, uint64_t agg, uint32_t *status) {
-  constexpr uint64_t kAgg = 1ull << 62, kInc = 2ull << 62, kMask = (1ull << 62) - 1;
-  if (bid == 0) {
-    st_relaxed(&state[0], kInc | agg);
-    return 0;
-  }
-  st_relaxed(&state[bid], kAgg | agg);
-  uint64_t prefix = 0;
-  int32_t j = bid - 1;
-  uint32_t polls = 0;
-  while (j >= 0) {
-    const uint64_t s = ld_relaxed(&state[j]);
-    const uint64_t f = s & ~kMask;
-    if (f == 0) {
-      if (++polls > kSpinLimit) {
-        atomicOr(status, kStatusTimeout);
-        break;
-      }
-      __nanosleep(32);
-      continue;
-    }
-    prefix += s & kMask;
-    if (f == kInc) break;
-    --j;
-  }
-  st_relaxed(&state[bid], kInc | (prefix + agg));
-  return prefix;
-}
-
-// The same look-back run by a whole warp, reading 32 predecessor states per
-// step: lane i looks at block (window - i).  The walk stops at the nearest
-// inclusive prefix; a lane that is not ready yet makes the warp poll again
-// (bounded).  Every lane returns the exclusive prefix; lane 0 publishes.
+// aggregate only, 2 = inclusive prefix), called by a warp of logical block
+// `bid` with the block's aggregate.  A step reads 32 predecessor states: lane
+// i looks at block (window - i).  The walk stops at the nearest inclusive
+// prefix; a lane that is not ready yet makes the warp poll again (predecessors
+// hold smaller tickets, so they are resident or finished and the wait ends;
+// the poll count is still bounded).  Every lane returns the exclusive prefix;
+// lane 0 publishes.
 __device__ __forceinline__ uint64_t lookback_u64_warp(uint64_t *state, int32_t bid, uint64_t agg,
                                                       uint32_t *status) {
   constexpr uint64_t kAgg = 1ull << 62, kInc = 2ull << 62, kMask = (1ull << 62) - 1;

@@ -361,9 +361,9 @@ constexpr int kRedEntries = 3;  // entries per reduction: 3 x 9 or 10 sums, one 
 constexpr int kRedStride = 36;  // floats per row: 16-byte rows whose float4 reads by 8 lanes hit 32 banks
 
 // Resident blocks asked of the compiler for strips on 16x16 tiles: 4 pixels,
-// 16 blocks of 64 threads (64 registers, no spills; 12 at 80 with the
-// auxiliary channels); 8 pixels, 18 of 32 threads (95 registers and 21 blocks
-// instead of 117 and 17).
+// 16 blocks of 64 threads (64 registers, 4 to 8 bytes spilled outside the
+// pixel loop; 12 at 80 with the auxiliary channels); 8 pixels, 18 of 32 threads
+// (96 registers, 4 to 12 bytes spilled, instead of 117 and 17 blocks).
 template <int TILE, int PPT, bool kAux>
 constexpr int bwd_min_blocks() {
   if (TILE != 16) return 1;
@@ -379,9 +379,9 @@ constexpr int bwd_min_blocks() {
 // kRedEntries entries are rows, and each lane then adds up one row (8 float4
 // loads) and adds it with one atomic -- about 25 warp instructions an entry
 // where the transposed shuffle butterfly and its operands took about 70.
-// 4 views of 1352x1014, 349k visible, 6.3M instances: 1.85 -> 1.11 G warp
-// instructions, 1.755 -> 1.399 ms (8 rows a thread; 1.525 with 4); it now issues
-// in 67 % of the slots with 28 % of the warps resident.
+// 4 views of 1352x1014, 349k visible, 6.3M instances: 1.755 -> 1.343 ms (8 rows
+// a thread).  Ordinary batches take a copy of the pixel loop that tests neither
+// the clamp nor the range of the products (1.403 -> 1.343 ms).
 //
 // kAux: the loss also has gradients dL/dD, dL/dO with respect to the depth
 // and opacity channels (zero background, x_i = z_i resp. 1 in the colour

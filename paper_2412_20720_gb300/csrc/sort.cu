@@ -80,17 +80,14 @@ __device__ __forceinline__ uint32_t radix_lookback(uint32_t *state, int64_t b, i
 
 // Digit histograms of keys [0, count) for `passes` 8-bit digits starting at
 // bit 0, grid-stride over radix tiles (kSortThreads x kItems keys); also
-// clears each tile's look-back rows and the tile ranges.
+// clears each tile's look-back rows.  Up to `small` keys nothing is done.
 template <int kItems>
 __global__ void __launch_bounds__(kSortThreads) radix_hist_kernel(const uint32_t *__restrict__ keys,
                                                                   const uint32_t *__restrict__ count_ptr, int64_t cap,
                                                                   int32_t passes, uint32_t *hist, uint32_t *state,
-                                                                  int32_t state_blocks, uint2 *ranges,
-                                                                  int64_t nranges, int64_t small) {
+                                                                  int32_t state_blocks, int64_t small) {
   grid_dependency_sync();
   __shared__ uint32_t s_hist[kMaxPasses][kRadixBins];
-  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < nranges; r += (int64_t)gridDim.x * blockDim.x)
-    ranges[r] = make_uint2(0u, 0u);
   const int64_t count = min64((int64_t)*count_ptr, cap);
   constexpr int kTileKeys = kSortThreads * kItems;
   if ((int64_t)blockIdx.x * kTileKeys >= count || count <= small) return;
@@ -905,7 +902,7 @@ cudaError_t depth_sort(const Layout &L, unsigned char *ws, uint32_t *sorted, cud
   constexpr size_t smem = radix_smem_bytes<kItems>();
   cudaError_t e = launch_pdl(radix_hist_kernel<kItems>, (unsigned)pb, kSortThreads, st, dkey,
                              (const uint32_t *)(ctr + kCtrVisible), (int64_t)L.vis_cap, (int32_t)L.depth_passes, hist,
-                             dstate, (int32_t)L.depth_blocks, (uint2 *)nullptr, (int64_t)0, kRankSortMax);
+                             dstate, (int32_t)L.depth_blocks, kRankSortMax);
   if (e != cudaSuccess) return e;
   for (int p = 0; p < L.depth_passes; ++p) {
     const int out = p & 1, in = out ^ 1;
@@ -1134,7 +1131,7 @@ extern "C" int fgs4d_sort_depth_static(const uint32_t *depth_keys, int64_t n, ui
   static_sort_init_kernel<<<1, 256, 0, st>>>(s, (uint32_t)n);
   radix_hist_kernel<kSortItems><<<blocks, kSortThreads, 0, st>>>(depth_keys, &s->ctl[0], FGS4D_STATIC_SORT_MAX,
                                                           kMaxPasses, &s->hist[0][0], &s->state[0][0][0],
-                                                          kStaticSortBlocks, nullptr, 0, -1);
+                                                          kStaticSortBlocks, -1);
   // The passes stage keys with 16-byte copies: keys that do not start on a
   // 16-byte boundary are first copied into the buffer pass 0 does not write.
   const uint32_t *keys0 = depth_keys;
