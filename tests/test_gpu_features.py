@@ -74,21 +74,21 @@ def test_feature_backward_matches_oracle(D, tile):
     compare_group("dL/dgate", grad_g.cpu().numpy().astype(np.float64), gg, 1e-3, 1e-4)
 
 
-@pytest.mark.parametrize("D", [8, 16, 32])
-def test_short_list_kernels_match_the_matrix_kernels(D):
+@pytest.mark.parametrize("D,tile", [(8, 16), (16, 16), (32, 16), (16, 8), (32, 8)])
+def test_short_list_kernels_match_the_matrix_kernels(D, tile):
     """The same calls by both routes (an instance capacity of fewer and of more
     than 40 instances a tile, 4225 tiles).  Map: weights add up to at most 1,
     so the split products stay within 2^-21 and up to 150 roundings of 2^-24;
     gradients: 1e-4 of the largest, as atomics add in another order."""
     import torch
     params = to_device(sy.make_scene(3000, 21, (-1, -1, -1), (1, 1, 1), sh_degree=1, t_order=1).as_dict())
-    view = sy.tiny_view(1040, 1030)
+    W, H = 65 * tile, 65 * tile - 9
     gen = torch.Generator(device="cuda").manual_seed(5)
     feats, gate = torch.randn((3000, D), device="cuda", generator=gen), torch.rand((D,), device="cuda", generator=gen)
-    up = torch.randn(D * 1040 * 1030, device="cuda", generator=gen)
+    up = torch.randn(D * W * H, device="cuda", generator=gen)
     got = []
     for cap in (39 * 4225, 1 << 21):
-        r = Renderer(3000, [view], RenderConfig(sh_degree=1, t_order=1, inst_capacity=cap))
+        r = Renderer(3000, [sy.tiny_view(W, H)], RenderConfig(sh_degree=1, t_order=1, inst_capacity=cap, tile=tile))
         out = r.forward_features(params, feats, gate)
         assert r.check()[1] > 20_000
         gf, gg = torch.zeros_like(feats), torch.zeros_like(gate)
