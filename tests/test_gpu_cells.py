@@ -200,3 +200,23 @@ def test_pairs_beyond_the_capacity_whose_masks_are_empty(stage_blocks):
     assert code == fgs4d.OK and got == want
     for x, y in zip(_lists(a, want, ntiles), _lists(b, got, ntiles)):
         np.testing.assert_array_equal(x, y)
+
+
+def test_lists_do_not_depend_on_the_capacities():
+    """The same list at both sides of every line that the capacities draw: the
+    binning's route, four slots a thread in the pair scan (2^19), eight keys a
+    thread in the depth sort (2^20), three sub-tiles a ticket in the instance
+    sort (2^26)."""
+    n, W, H = 30_000, 640, 480
+    rng = np.random.default_rng(12)
+    rec = _synthetic_records(rng, n, W, H, 20)
+    _stretched(rec, rng, 2.0, 60.0)
+    views, ntiles, want = [sy.tiny_view(W, H)], 40 * 30, None
+    for vis_cap, inst_cap in ((n, 1 << 22), (n, 1 << 26), (65_535, 1 << 26), (65_536, 1 << 22), ((1 << 19) - 1, 1 << 22),
+                              (1 << 19, 1 << 22), ((1 << 20) - 1, 1 << 22), (1 << 20, 1 << 22)):
+        r, (code, counts) = _run(rec, views, 16, inst_cap, vis_cap=vis_cap)
+        assert code == fgs4d.OK and counts[1] > 10 * n
+        got = [np.array(counts)] + list(_lists(r, counts, ntiles))
+        want = want or got
+        for x, y in zip(want, got):
+            np.testing.assert_array_equal(x, y)
