@@ -58,20 +58,24 @@ struct RenderBwdArgs {
 };
 
 // Pixels per thread of the compositor kernels (the autotuned block shape):
-// 16x16 tiles take 2, 4 or 8, 8x8 tiles 1 or 2.  Defaults for 16x16 tiles by
-// the tile count: 4; with few tiles, whose lists too few warps would walk, 2;
-// with many the adjoint of the image, whose per-entry work (moments and
-// reduction rows) is shared by a strip, 8.  Measured forward / adjoint (us)
+// 16x16 tiles take 2, 4 or 8, 8x8 tiles 1 or 2.  Defaults for 16x16 tiles: 4;
+// with few tiles, whose lists too few warps would walk, 2; with many tiles the
+// adjoint of the image, whose per-entry work (moments and reduction rows) is
+// shared by a strip, 8 -- unless the instance capacity says that the lists are
+// short, where a block's set-up counts.  Measured forward / adjoint (us)
 // with 2, 4 and 8 rows a thread: 48 tiles 12.0 / 26.7, 18.5 / 39.2, 35.0 /
 // 63.5; 690 tiles 26.8 / 63.7, 38.9 / 84.0, 70.6 / 123; 1200 tiles 32.3 / 76.4,
 // 33.1 / 74.6, 59.1 / 107; 3978 tiles 54.5 / 155, 56.7 / 139, 77.5 / 146; 5440
-// tiles 190 / 581, 186 / 454, 267 / 442.
-constexpr int64_t kFewTiles = 1024, kManyTiles = 5000;
+// tiles of 308 entries 190 / 561, 186 / 438, 267 / 411.  Adjoint with 4 and 8
+// rows at 21,760 tiles and more, by entries a tile: 1.7 110 / 121, 2.7 151 /
+// 162, 9.8 111 / 114, 19 178 / 174, 39 321 / 303, 77 605 / 552 (capacities are
+// some twice that).
+constexpr int64_t kFewTiles = 1024, kManyTiles = 5000, kLongListCap = 32;
 inline int render_ppt(const fgs4d_settings *s, const Layout &L, bool adjoint) {
   if (s->tile == 8) return s->pixels_per_thread == 1 ? 1 : 2;
   if (s->pixels_per_thread) return s->pixels_per_thread;
   if (L.total_tiles < kFewTiles) return 2;
-  return adjoint && L.total_tiles >= kManyTiles ? 8 : 4;
+  return adjoint && L.total_tiles >= kManyTiles && L.inst_cap >= kLongListCap * L.total_tiles ? 8 : 4;
 }
 
 
@@ -430,6 +434,7 @@ __global__ void __launch_bounds__(TILE *TILE / kPPT, (bwd_min_blocks<TILE, kPPT,
   const int32_t px = tx * TILE + (threadIdx.x & (TILE - 1));
   const int32_t py0 = ty * TILE + (threadIdx.x / TILE) * kPPT;
   const uint2 range = tile_range(A.ranges, gt);
+  if (range.x == range.y) return;  // nothing was composited: no gradient, and its planes need no reading
   const float pxc = (float)px + 0.5f;
   const int64_t HW = (int64_t)V.width * V.height;
   constexpr int kGroups = (kPPT + 3) / 4;  // row groups of the strip (see group_w)
