@@ -71,7 +71,7 @@ ISSUE_PER_SM_CLK = 4
 # views 0-2).  Valid only for the compositor sources it was taken from
 # (sha256 prefix of csrc/render.cu + csrc/fgs4d_internal.cuh) and block
 # shape; any other build reports null.
-NCU_RENDER_FWD = {"render_cu_sha256": "592025e0ed3e05ba", "shape": "16/4/128", "dram_bytes": 5.02e6, "warp_insts": 101.02e6,
+NCU_RENDER_FWD = {"render_cu_sha256": "1c1abb1d36f6ba92", "shape": "16/4/128", "dram_bytes": 5.02e6, "warp_insts": 101.02e6,
                   "views": [0, 1, 2], "capture": "ncu --metrics (bytes, instructions) --clock-control none --nvtx --nvtx-include timed/ "
                                                  "-k regex:render_fwd_kernel -c 3 on python bench.py --steps 1 "
                                                  "--warmup 3 --shape 16/4/128 (no other legs)"}
