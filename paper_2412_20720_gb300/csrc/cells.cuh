@@ -119,7 +119,8 @@ __device__ __forceinline__ uint64_t cell_mask(float u, float v, float a1, float 
   while (maybe) {
     const int bit = __ffsll((long long)maybe) - 1;
     maybe &= maybe - 1ull;
-    const int tx = (tx0 & ~(kCellEdge - 1)) + (bit & (kCellEdge - 1)), ty = (ty0 & ~(kCellEdge - 1)) + (bit >> kCellShift);
+    const int tx = (tx0 & ~(kCellEdge - 1)) + (bit & (kCellEdge - 1));
+    const int ty = (ty0 & ~(kCellEdge - 1)) + (bit >> kCellShift);
     if (tile_meets(u, v, a1, b1, b2, kx, ky, tau, V, tx, ty)) sure |= 1ull << bit;
   }
   return sure;

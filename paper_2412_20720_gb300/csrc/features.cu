@@ -176,7 +176,8 @@ __global__ void __launch_bounds__(TILE *TILE / kScalarPPT)
   for (uint32_t base = range.x; base < range.y; base += kBatch) {
     if (__syncthreads_count(live) == 0) break;
     if (base + threadIdx.x < range.y)
-      stage_feature<D, false>(A, s_gate, base + threadIdx.x, threadIdx.x, s_geom, s_ca, s_fhat, nullptr, nullptr, nullptr);
+      stage_feature<D, false>(A, s_gate, base + threadIdx.x, threadIdx.x, s_geom, s_ca, s_fhat, nullptr, nullptr,
+                              nullptr);
     __syncthreads();
     const int nb = (int)min(range.y - base, (uint32_t)kBatch);
     for (int j = 0; j < nb && live; ++j) {
@@ -612,7 +613,8 @@ constexpr int bwd_min_blocks() {
 }
 
 template <int MAXV, int TILE, int D>
-__global__ void __launch_bounds__(feat_threads<TILE>(), (bwd_min_blocks<TILE, D>())) render_features_bwd_kernel(FeatArgs A, RasterViews<MAXV> rv) {
+__global__ void __launch_bounds__(feat_threads<TILE>(), (bwd_min_blocks<TILE, D>()))
+    render_features_bwd_kernel(FeatArgs A, RasterViews<MAXV> rv) {
   grid_dependency_sync();
   constexpr int NT = feat_threads<TILE>(), kWarps = NT / 32, kN = D / 8, kRow = D + 1;
   constexpr int kPart = feat_stride<D>();  // floats per entry row of a warp's sums
