@@ -29,7 +29,7 @@
 //
 // Measured at 300k Gaussians, one 1352x1014 view, before (multiply-adds with a
 // shuffle butterfly and D atomics per (warp, entry)) -> now, us: D = 32 forward
-// 900 -> 726, backward 1490 -> 844; D = 16 backward 933 -> 572; D = 8 670 -> 457.
+// 900 -> 726, backward 1490 -> 851; D = 16 backward 933 -> 574; D = 8 670 -> 465.
 // Bound by issue; at D = 32 a quarter of the warps are resident (operands or
 // accumulators take 128 registers a thread).
 #include <algorithm>
@@ -804,8 +804,8 @@ cudaError_t launch_feat_tile(const FeatArgs &A, const RasterViews<MAXV> &rv, uns
 // capacity, an upper bound of the instances, is below this many a tile (twice
 // the lists' length or more, as capacities have headroom).  Scalar / matrix
 // (us) at 1352x1014, by instances a tile: adjoint D = 8 5.2 33 / 48, 10.6 50 /
-// 56, 15 64 / 66, 20.5 81 / 76, 308 670 / 457; D = 32 78 / 113, 115 / 126, 146 /
-// 142, 181 / 158, 1490 / 844; map D = 32 5.2 56 / 95, 10.6 74 / 105, 20.5 111 /
+// 56, 15 64 / 66, 20.5 81 / 76, 308 670 / 465; D = 32 78 / 113, 115 / 126, 146 /
+// 142, 181 / 158, 1490 / 851; map D = 32 5.2 56 / 95, 10.6 74 / 105, 20.5 111 /
 // 132, 31 154 / 160, 41 197 / 187, 308 902 / 726.  With fewer tiles than some
 // 4000 one round of blocks holds most of a call and the longest list decides:
 // the adjoint of 1200 tiles with 10 entries a tile takes 25 / 19 at D = 8.
